@@ -239,6 +239,10 @@ int launch_variant(const uint8_t *msgs, uint64_t stride, uint64_t len, uint32_t 
 
 int launch_uniform(const uint8_t *msgs, uint64_t stride, uint64_t len, int variant, uint32_t out_len,
                    uint8_t *digests, uint64_t n, cudaStream_t stream, const DeviceInfo &dev) {
+    int rc = KB_OK;
+    if (tuning_get(KB_TUNE_REPRESENTATION) == KB_REP_PLAIN &&
+        launch_uniform_small(msgs, stride, len, variant, out_len, digests, n, stream, dev, &rc))
+        return rc;
     switch (variant) {
         case 0: return launch_variant<0>(msgs, stride, len, out_len, digests, n, stream, dev);
         case 1: return launch_variant<1>(msgs, stride, len, out_len, digests, n, stream, dev);

@@ -1,0 +1,71 @@
+"""Batches too small to fill the GPU with a thread per message: the forms with thirty and with two threads a
+message, at the edges of their size ranges, of the rate and of the alignment, against hashlib."""
+import hashlib
+
+import numpy as np
+import pytest
+
+from paper_1902_05320_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+HASHES = (hashlib.sha3_224, hashlib.sha3_256, hashlib.sha3_384, hashlib.sha3_512, hashlib.shake_128,
+          hashlib.shake_256)
+RATES = (144, 136, 104, 72, 168, 136)
+
+
+def want(variant, data, out_len):
+    h = HASHES[variant](data)
+    return h.digest(out_len) if variant >= 4 else h.digest()
+
+
+def run_uniform(cuda_lib, data, shift, stride, length, variant, out_len, n):
+    """Digests of n messages whose first byte sits `shift` bytes into an allocation, with guard bytes around the
+    output (one byte in, so no store is aligned by luck when shift is odd)."""
+    import torch
+
+    raw = torch.zeros(shift + data.size + 16, dtype=torch.uint8, device="cuda")
+    raw[shift:shift + data.size] = torch.from_numpy(data).cuda()
+    out = torch.full((n * out_len + 32,), 0xEE, dtype=torch.uint8, device="cuda")
+    o = 16 + (shift & 1)
+    cuda_lib.keccak_batch_uniform(raw.data_ptr() + shift, stride, length, variant, out_len, out.data_ptr() + o, n)
+    got = out.cpu().numpy()
+    assert (got[:o] == 0xEE).all() and (got[o + n * out_len:] == 0xEE).all(), "bytes outside the output were written"
+    return got[o:o + n * out_len].reshape(n, out_len)
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3, 4, 7])
+@pytest.mark.parametrize("variant", range(6))
+@pytest.mark.parametrize("per_sm", [0, 13])  # thirty threads a message; two threads
+def test_lengths_and_alignments(cuda_lib, variant, shift, per_sm):
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = max(3, per_sm * sms)
+    rate = RATES[variant]
+    rng = np.random.default_rng(1000 * variant + shift)
+    for length in (0, 1, 6, 7, 8, rate - 1, rate, rate + 1, 2 * rate - 8, 2 * rate, 3 * rate - 1, 3 * rate, 4 * rate + 5):
+        for out_len in ((W.DIGEST_BYTES[variant],) if variant < 4 else (1, 33, rate, rate + 1, 2 * rate + 3)):
+            if variant >= 4 and length not in (0, rate, 3 * rate) and out_len != 33:
+                continue
+            stride = length + (shift % 3)
+            data = rng.integers(0, 256, size=max(1, n * stride), dtype=np.uint8)
+            got = run_uniform(cuda_lib, data, shift, stride, length, variant, out_len, n)
+            blob = data.tobytes()
+            for i in sorted({0, 1, 2, 31, 32, n // 2, n - 2, n - 1} & set(range(n))):
+                assert got[i].tobytes() == want(variant, blob[i * stride:i * stride + length], out_len), (length, out_len, i)
+
+
+@pytest.mark.parametrize("blocks", [1, 3])
+@pytest.mark.parametrize("edge", [8, 12, 64])  # the lines between the forms, in messages per SM
+def test_batch_sizes_around_the_lines(cuda_lib, edge, blocks):
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    length = 136 * blocks - 9
+    for n in (edge * sms - 1, edge * sms, edge * sms + 1):
+        data = np.random.default_rng(n).integers(0, 256, size=n * length, dtype=np.uint8)
+        got = run_uniform(cuda_lib, data, 0, length, length, 1, 32, n)
+        blob = data.tobytes()
+        for i in range(n):
+            assert got[i].tobytes() == hashlib.sha3_256(blob[i * length:(i + 1) * length]).digest(), (n, i)
