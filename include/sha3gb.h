@@ -477,9 +477,9 @@ void keccak_release(void);
 /*   KB_TUNE_RAGGED_SCHEDULE: how keccak_batch orders its work --
  *     KB_SCHEDULE_QUEUE (default: messages sorted into cost buckets, longest
  *     first, consumed by one persistent launch, one thread per message),
- *     KB_SCHEDULE_LANE_PARALLEL (the same order, one warp per message: the 25
- *     state lanes on 25 threads; about 2x lower latency per message at about
- *     4x the instructions, for few long messages), KB_SCHEDULE_PER_VARIANT (a
+ *     KB_SCHEDULE_LANE_PARALLEL (the same order, one warp per message: the
+ *     state on 30 threads; about 3x lower latency per message at about 6x the
+ *     issue time, for few long messages), KB_SCHEDULE_PER_VARIANT (a
  *     control: one launch per variant over that variant's messages, rate fixed
  *     at compile time, not ordered by length) or KB_SCHEDULE_INPUT_ORDER (one
  *     thread per message in input order, the plain one-launch control).
@@ -538,7 +538,7 @@ void keccak_release(void);
  *     2 and 3); with another budget the kernel loads directly.
  *   KB_TUNE_QUEUE_WARP_MESSAGES: threads per message -- -1 (default: tuned,
  *     else 0) or K >= 0: the K costliest messages of a batch run one warp each
- *     (the lane-parallel sponge) in a kernel started first on a side stream,
+ *     (the cooperative sponge) in a kernel started first on a side stream,
  *     concurrently with the queue kernel, which takes the rest one thread
  *     each. */
 #define KB_TUNE_QUEUE_STAGING 8

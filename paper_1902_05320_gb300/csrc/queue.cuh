@@ -38,8 +38,8 @@
 #include <cstdint>
 
 #include "../../include/sha3gb.h"
+#include "coop_sponge.cuh"
 #include "keccak_core.cuh"
-#include "lane_parallel.cuh"
 #include "runtime.cuh"
 #include "scan.cuh"
 #include "sponge.cuh"

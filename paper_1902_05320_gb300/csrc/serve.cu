@@ -35,8 +35,8 @@
 #include <vector>
 
 #include "arena_heap.h"
+#include "coop_sponge.cuh"
 #include "keccak_core.cuh"
-#include "lane_parallel.cuh"
 #include "runtime.cuh"
 #include "sponge.cuh"
 
@@ -120,14 +120,22 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     }
 }
 
-// Long requests: one warp per request (lane-parallel sponge).
-__global__ void __launch_bounds__(kThreads)
-    k_serve_hash_lanes(const ReqDesc *__restrict__ d, uint32_t m, const uint8_t *__restrict__ arena,
-                       CompletionRing *ring) {
-    const uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) / 32;
-    if (r >= m) return;
-    const ReqDesc q = d[r];
-    lane_sponge<true>(arena + q.arena_off, q.len, int(q.variant), reinterpret_cast<uint8_t *>(q.out), q.out_len);
+// Long requests: one warp per request (coop_sponge.cuh), one warp per block.  A
+// long request's latency is its chain of permutations: 1.55 us each here, 2.36
+// with a lane of the state per thread, the form before.  The launch asks for
+// kLongSmem bytes of shared memory that it does not use, so that an SM holds at
+// most nine of these warps: batches start while others' blocks occupy most SMs,
+// and without a limit the scheduler put up to 32 long chains on the few SMs with
+// room, where they share the path to shared memory (2000 requests of up to 1 MiB
+// at once: 26 to 51 ms from run to run without the limit, 25 to 27 with it, 40 to
+// 43 before; blocks of four warps, three of them idle, to the same end: 31).
+constexpr size_t kLongSmem = 24 * 1024;
+__global__ void __launch_bounds__(32)
+    k_serve_hash_lanes(const ReqDesc *__restrict__ d, const uint8_t *__restrict__ arena, CompletionRing *ring) {
+    __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
+    const Coop c(mem);
+    const ReqDesc q = d[blockIdx.x];
+    coop_sponge(c, arena + q.arena_off, q.len, int(q.variant), reinterpret_cast<uint8_t *>(q.out), q.out_len);
     __syncwarp();
     if (ring && (threadIdx.x & 31) == 0) {
         __threadfence_system();
@@ -360,8 +368,7 @@ struct Server {
             const uint64_t gblocks = std::min<uint64_t>(chunks, uint64_t(sm_count) * 16);
             k_gather<<<unsigned(gblocks), kGatherThreads, 0, s.stream>>>(s.d_desc, m, chunks, arena);
             if (lanes_kernel)
-                k_serve_hash_lanes<<<(m * 32 + kThreads - 1) / kThreads, kThreads, 0, s.stream>>>(
-                    s.d_desc, m, arena, ring_mode ? ring : nullptr);
+                k_serve_hash_lanes<<<m, 32, kLongSmem, s.stream>>>(s.d_desc, arena, ring_mode ? ring : nullptr);
             else
                 k_serve_hash<<<(m + kThreads - 1) / kThreads, kThreads, 0, s.stream>>>(s.d_desc, m, arena,
                                                                                        ring_mode ? ring : nullptr);

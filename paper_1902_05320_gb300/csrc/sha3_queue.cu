@@ -18,7 +18,7 @@
 //     memory during the permutation (with the runtime-rate or the
 //     rate-specialised absorb);
 //   * threads per message: 1 for every message, or a hybrid in which the K
-//     costliest messages run one warp each (the lane-parallel sponge) in a
+//     costliest messages run one warp each (the cooperative sponge) in a
 //     kernel launched first on a side stream, concurrently with the queue.
 #include <cuda_runtime.h>
 
@@ -43,14 +43,17 @@ static_assert(kb::QueueConfig().stage == (kb::kStageRegs | kb::kLooped), "defaul
 
 namespace kb {
 
-// One warp per message (lane-parallel sponge) over entries [0, limit) of the
-// order, taken one at a time from *head.
-__global__ void __launch_bounds__(kThreads)
+// One warp per message (the cooperative sponge of coop_sponge.cuh) over entries
+// [0, limit) of the order, taken one at a time from *head; one warp per block, so
+// that the warps spread over the SMs.
+__global__ void __launch_bounds__(32)
     k_sha3_lanes(const uint8_t *__restrict__ msgs, const uint64_t *__restrict__ offsets,
                  const uint64_t *__restrict__ lens, const uint8_t *__restrict__ variants,
                  const uint32_t *__restrict__ out_lens, const uint64_t *__restrict__ out_off,
                  const uint32_t *__restrict__ order, uint8_t *__restrict__ digests, uint64_t limit,
                  unsigned long long *head, unsigned int *status) {
+    __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
+    const Coop c(mem);
     const int lane = threadIdx.x & 31;
     for (;;) {
         unsigned long long idx = 0;
@@ -64,9 +67,7 @@ __global__ void __launch_bounds__(kThreads)
             if (lane == 0) atomicOr(status, v > 5 ? KB_DEV_BAD_VARIANT : KB_DEV_BAD_OUTLEN);
             continue;
         }
-        const uint8_t *p = msgs + offsets[i];
-        if ((reinterpret_cast<uintptr_t>(p) & 7) == 0) lane_sponge<true>(p, lens[i], v, digests + out_off[i], dlen);
-        else lane_sponge<false>(p, lens[i], v, digests + out_off[i], dlen);
+        coop_sponge(c, msgs + offsets[i], lens[i], v, digests + out_off[i], dlen);
     }
 }
 
@@ -156,13 +157,14 @@ int resident_blocks(const void *fn, int device) {
 // Blocks of the hashing launch for n messages.
 uint64_t queue_grid(const QueueConfig &cfg, uint64_t n, int device, int sm_count) {
     const void *fn = cfg.per_variant ? reinterpret_cast<const void *>(&k_sha3_variant<1>)
-                     : cfg.lanes     ? reinterpret_cast<const void *>(&k_sha3_lanes)
                                      : queue_kernel(cfg.minb, cfg.stage);
     uint64_t per_sm = uint64_t(resident_blocks(fn, device));
-    if (!cfg.per_variant && !cfg.lanes && cfg.blocks_per_sm > 0) per_sm = std::min<uint64_t>(per_sm, cfg.blocks_per_sm);
+    if (!cfg.per_variant && cfg.blocks_per_sm > 0) per_sm = std::min<uint64_t>(per_sm, cfg.blocks_per_sm);
     const uint64_t full = per_sm * uint64_t(sm_count > 0 ? sm_count : 1);
-    const uint64_t threads_per_item = cfg.lanes ? 32 : 1;
-    const uint64_t need = (n * threads_per_item + kThreads - 1) / kThreads;
+    // One warp per message: a block each, kCoopPerSm per SM (beyond it the warps
+    // of an SM only share its shared-memory path; entries are longest first).
+    if (cfg.lanes) return std::max<uint64_t>(1, std::min(n, kCoopPerSm * uint64_t(sm_count > 0 ? sm_count : 1)));
+    const uint64_t need = (n + kThreads - 1) / kThreads;
     return std::max<uint64_t>(1, std::min(need, full));
 }
 
@@ -211,9 +213,8 @@ int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *le
         if (cudaEventRecord(aux->fork, stream) != cudaSuccess || cudaStreamWaitEvent(aux->side, aux->fork, 0) != cudaSuccess)
             return KB_ERR_CUDA;
         const uint64_t warps = std::min<uint64_t>(k, uint64_t(4) * uint64_t(sm_count > 0 ? sm_count : 1));
-        k_sha3_lanes<<<unsigned((warps + 3) / 4), kThreads, 0, aux->side>>>(msgs, offsets, lens, variants, out_lens,
-                                                                          bf.out_off, bf.order, digests, k,
-                                                                          &bf.ctl->lane_head, status);
+        k_sha3_lanes<<<unsigned(warps), 32, 0, aux->side>>>(msgs, offsets, lens, variants, out_lens, bf.out_off,
+                                                             bf.order, digests, k, &bf.ctl->lane_head, status);
         if (cudaEventRecord(aux->join, aux->side) != cudaSuccess) return KB_ERR_CUDA;
     }
     if (k < n || cfg.lanes) {
@@ -225,7 +226,7 @@ int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *le
             uint64_t limit = n;
             void *args[] = {&msgs, &offsets, &lens, &variants, &out_lens, const_cast<uint64_t **>(&bf.out_off),
                             const_cast<uint32_t **>(&bf.order), &digests, &limit, &head, &status};
-            e = cudaLaunchKernel(fn, dim3(unsigned(grid)), dim3(kThreads), args, 0, stream);
+            e = cudaLaunchKernel(fn, dim3(unsigned(grid)), dim3(32), args, 0, stream);
         } else {
             Control *ctl = bf.ctl;
             void *args[] = {&msgs, &offsets, &lens, &variants, &out_lens, const_cast<uint64_t **>(&bf.out_off),
