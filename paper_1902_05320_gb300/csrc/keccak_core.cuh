@@ -151,6 +151,62 @@ __device__ __forceinline__ void rotl64(uint32_t lo, uint32_t hi, uint32_t &nl, u
     }
 }
 
+// ---- the same rotations beside the ALU pipe ------------------------------------
+//
+// (hi << N) | (lo >> (32 - N)), 0 < N < 12, without an ALU-pipe instruction.
+// The ALU pipe (LOP3, SHF: 16 lanes per sub-partition per clock) bounds every
+// sponge kernel here, while the multiply pipe beside it idles.  A left shift is
+// a multiply by 2^N; a right shift is read off a dot product of 16-bit halves:
+// dp2a multiplies the top half of lo by 2^N, and a second dp2a adds the top half
+// of that product, which is lo >> (32 - N), to hi << N (the bits are disjoint,
+// so the sum is the OR).  dp2a's weights are bytes, so from N = 8 on the product
+// is a separate multiply; N = 8 itself is one dp4a that adds the top byte.
+// Probed on GB300 (cycles a warp and sub-partition): LOP3, SHF, mad.lo, dp2a and
+// dp4a take 2 each, mad.lo and dp2a beside LOP3 take no ALU time, mul.hi and
+// mul.wide take 2 of the ALU's as well as 4 of their own (so they gain nothing).
+template <int N>
+__device__ __forceinline__ uint32_t shl_pair_mul(uint32_t lo, uint32_t hi) {
+    static_assert(N >= 1 && N <= 11, "one of the offsets that pay");
+    uint32_t c, d;
+    asm("mad.lo.u32 %0, %1, %2, 0;" : "=r"(c) : "r"(hi), "n"(1u << N));
+    if constexpr (N == 8) {
+        asm("dp4a.u32.u32 %0, %1, 0x01000000, %2;" : "=r"(d) : "r"(lo), "r"(c));
+        return d;
+    } else {
+        uint32_t t;
+        if constexpr (N < 8) {
+            asm("dp2a.lo.u32.u32 %0, %1, %2, 0;" : "=r"(t) : "r"(lo), "n"(256u << N));
+        } else {
+            uint32_t top;
+            asm("dp2a.lo.u32.u32 %0, %1, 0x0100, 0;" : "=r"(top) : "r"(lo));
+            asm("mad.lo.u32 %0, %1, %2, 0;" : "=r"(t) : "r"(top), "n"(1u << N));
+        }
+        asm("dp2a.lo.u32.u32 %0, %1, 0x0100, %2;" : "=r"(d) : "r"(t), "r"(c));
+        return d;
+    }
+}
+
+// The rounds' 64-bit rotation: by multiplies for offsets of 1..11 modulo 32
+// (theta's 1 and rho's 1, 2, 3, 6, 8, 10, 36, 39, 41 and 43), by funnel shifts
+// otherwise.  A round then has 149 ALU instructions and 96 multiplies instead
+// of 180 and none: 361 -> 328 cycles a warp and sub-partition in the looped
+// permutation.  It does not reach the ALU's 298: the register file's read
+// ports bind next (a multiply with two register operands beside three-operand
+// LOP3s costs 0.45 cycles).  So the line lies at 11: offsets of 9..11 cost
+// five register reads a word and still pay (335 -> 328), 12 and 13 lose
+// (336), all up to 15 more (339); bit reversals on the otherwise idle XU pipe
+// for the offsets near 32 lose as well (330 -> 334..347).
+template <int N>
+__device__ __forceinline__ void rotl64_round(uint32_t lo, uint32_t hi, uint32_t &nl, uint32_t &nh) {
+    constexpr int M = N & 31;
+    if constexpr (M >= 1 && M <= 11) {
+        nl = N < 32 ? shl_pair_mul<M>(hi, lo) : shl_pair_mul<M>(lo, hi);
+        nh = N < 32 ? shl_pair_mul<M>(lo, hi) : shl_pair_mul<M>(hi, lo);
+    } else {
+        rotl64<N>(lo, hi, nl, nh);
+    }
+}
+
 // theta's column terms for the source lane of (X, Y), then rho; pi is the
 // choice of source: Eq. 6, A'[x,y] = A[(x+3y) mod 5, x].
 template <int X, int Y>
@@ -163,7 +219,7 @@ __device__ __forceinline__ void plain_theta_rho_pi(const uint32_t (&L)[25], cons
     // Eq. 4 with D[x] = C[x-1] ^ rot(C[x+1], 1) (Eq. 3).
     const uint32_t tl = xor3(L[SRC], CL[(SX + 4) % 5], RL[(SX + 1) % 5]);
     const uint32_t th = xor3(H[SRC], CH[(SX + 4) % 5], RH[(SX + 1) % 5]);
-    rotl64<rho_offset(SRC)>(tl, th, bl, bh);
+    rotl64_round<rho_offset(SRC)>(tl, th, bl, bh);
 }
 
 template <int Y>
@@ -193,7 +249,7 @@ __device__ __forceinline__ void plain_round_body(uint32_t (&L)[25], uint32_t (&H
         CH[x] = xor3(xor3(H[x], H[x + 5], H[x + 10]), H[x + 15], H[x + 20]);
     }
 #pragma unroll
-    for (int x = 0; x < 5; ++x) rotl64<1>(CL[x], CH[x], RL[x], RH[x]);
+    for (int x = 0; x < 5; ++x) rotl64_round<1>(CL[x], CH[x], RL[x], RH[x]);
     plain_row<0>(L, H, CL, CH, RL, RH, NL, NH);
     plain_row<1>(L, H, CL, CH, RL, RH, NL, NH);
     plain_row<2>(L, H, CL, CH, RL, RH, NL, NH);
@@ -206,7 +262,7 @@ __device__ __forceinline__ void plain_round_rt(uint32_t (&L)[25], uint32_t (&H)[
     uint32_t NL[25], NH[25];
     plain_round_body(L, H, NL, NH);
     NL[0] ^= c_rc.w[2 * ir];  // Eq. 9
-    NH[0] ^= c_rc.w[2 * ir + 1];
+    NH[0] += c_rc.w[2 * ir + 1];  // bit 31 alone or nothing, so the sum is the XOR (off the ALU pipe)
 #pragma unroll
     for (int i = 0; i < 25; ++i) {
         L[i] = NL[i];
@@ -221,7 +277,7 @@ __device__ __forceinline__ void plain_round_ct(uint32_t (&L)[25], uint32_t (&H)[
     uint32_t NL[25], NH[25];
     plain_round_body(L, H, NL, NH);
     if constexpr (uint32_t(RC) != 0) NL[0] ^= uint32_t(RC);
-    if constexpr (uint32_t(RC >> 32) != 0) NH[0] ^= uint32_t(RC >> 32);
+    if constexpr (uint32_t(RC >> 32) != 0) NH[0] += uint32_t(RC >> 32);  // bit 31 alone
 #pragma unroll
     for (int i = 0; i < 25; ++i) {
         L[i] = NL[i];
@@ -235,20 +291,25 @@ __device__ __forceinline__ void plain_rounds_ct(uint32_t (&L)[25], uint32_t (&H)
     (plain_round_ct<FIRST + K>(L, H), ...);
 }
 
-// Keccak-f[1600] = Keccak-p[1600, 24] (Eq. 10, i_r = 0..23).  PEEL0 runs
-// round 0 with an immediate constant so that known-zero input lanes fold.
-template <bool PEEL0>
+// Keccak-f[1600] = Keccak-p[1600, 24] (Eq. 10, i_r = 0..23): the rounds before
+// TAIL in a loop of four, the others unrolled.  PEEL0 runs round 0 with an
+// immediate constant so that known-zero input lanes fold.  A round is about 4 KB
+// of code: an unrolled tail pays where the last round folds (a digest of a few
+// lanes) or where nothing else competes for the instruction cache (raw states,
+// 897 -> 885 us on 2^22), and costs where blocks are absorbed in between (15
+// blocks of SHA3-512 on 2^18 messages 821 -> 827 us, a 4 GiB tree 6.62 -> 6.66 ms).
+template <bool PEEL0, int TAIL>
 __device__ __forceinline__ void keccak_f1600_plain(uint32_t (&L)[25], uint32_t (&H)[25]) {
     constexpr int kLoopUnroll = 4;
     constexpr int kFirst = PEEL0 ? 1 : 0;
-    constexpr int kTail = PEEL0 ? 21 : 20;  // rounds [kTail, 24) unrolled
+    static_assert((TAIL - kFirst) % kLoopUnroll == 0 && TAIL <= 24, "whole passes of the loop");
     if constexpr (PEEL0) plain_round_ct<0>(L, H);
 #pragma unroll 1
-    for (int r = kFirst; r < kTail; r += kLoopUnroll) {
+    for (int r = kFirst; r < TAIL; r += kLoopUnroll) {
 #pragma unroll
         for (int j = 0; j < kLoopUnroll; ++j) plain_round_rt(L, H, r + j);
     }
-    plain_rounds_ct<kTail>(L, H, std::make_integer_sequence<int, 24 - kTail>{});
+    plain_rounds_ct<TAIL>(L, H, std::make_integer_sequence<int, 24 - TAIL>{});
 }
 
 // ---- representations ------------------------------------------------------------
@@ -273,7 +334,7 @@ struct PlainRep {
     __host__ __device__ static constexpr uint32_t word_b(uint64_t v) { return uint32_t(v >> 32); }
     template <bool PEEL0>
     __device__ __forceinline__ static void permute(uint32_t (&A)[25], uint32_t (&B)[25]) {
-        keccak_f1600_plain<PEEL0>(A, B);
+        keccak_f1600_plain<PEEL0, PEEL0 ? 21 : 24>(A, B);
     }
 };
 

@@ -177,7 +177,7 @@ __device__ __forceinline__ void p1600_round(uint32_t (&L)[25], uint32_t (&H)[25]
 // renames the state between rounds instead of copying it.
 __device__ __forceinline__ void p1600_rounds(uint32_t (&L)[25], uint32_t (&H)[25], int first_ir, int nr) {
     if (first_ir == 0 && nr == 24) {
-        keccak_f1600_plain<false>(L, H);
+        keccak_f1600_plain<false, 20>(L, H);
         return;
     }
     int ir = ((first_ir % 255) + 255) % 255, r = 0;  // rc has period 255 (Algorithm 5)

@@ -24,11 +24,18 @@
 namespace kb {
 namespace {
 
+// Blocks per SM the one-block kernels are compiled for.  With rotations on the
+// multiply pipe more warps are wanted to keep both pipes fed: 2^24 64-byte
+// messages take 3.31 ms at a budget of 4 (5 blocks fit), 3.29 at 5, 3.24 at 6.
+// The multi-block kernels stay at kMinBlocks (2^18 messages of 1023 bytes
+// 820 us at 4; 837 at 5 and 851 at 6, which spill).
+constexpr int kOneBlockMinBlocks = 6;
+
 // LEN >= 0: compile-time message length; -1: runtime; -2: runtime, below the
 // rate, with at most one block of output.  A8: base and stride are multiples
 // of 8 (16 when LEN == 64).
 template <int V, int LEN, bool A8, class Rep>
-__global__ void __launch_bounds__(kThreads, kMinBlocks)
+__global__ void __launch_bounds__(kThreads, LEN == -1 ? kMinBlocks : kOneBlockMinBlocks)
     k_sha3_uniform(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len_rt,
                    uint8_t *__restrict__ out, uint32_t out_len, uint64_t n) {
     using P = Variant<V>;
@@ -93,7 +100,7 @@ constexpr uint32_t kTileBytes = kThreads * 64;  // 8 KiB
 constexpr uint64_t kWaitNs = 1000000000ull;     // 1 s
 
 template <int V, class Rep>
-__global__ void __launch_bounds__(kThreads, kMinBlocks)
+__global__ void __launch_bounds__(kThreads, kOneBlockMinBlocks)
     k_sha3_uniform64_tma(const uint8_t *__restrict__ msgs, uint8_t *__restrict__ out, uint32_t out_len, uint64_t n,
                          unsigned int *status) {
     using P = Variant<V>;

@@ -130,21 +130,12 @@ __device__ __forceinline__ void absorb_staged_last(uint32_t (&A)[25], uint32_t (
     }
 }
 
-// Keccak-f[1600] with all 24 rounds in a loop of four (constants from the
-// __constant__ table): half the code of the form with an unrolled tail,
-// for kernels whose instruction footprint matters more than the immediates.
-__device__ __forceinline__ void keccak_f1600_looped(uint32_t (&L)[25], uint32_t (&H)[25]) {
-#pragma unroll 1
-    for (int r = 0; r < 24; r += 4) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) plain_round_rt(L, H, r + j);
-    }
-}
-
+// LOOPED: all 24 rounds in the loop of four, half the code of the form with an
+// unrolled tail, for kernels whose instruction footprint matters more than the
+// immediates.
 template <bool LOOPED>
 __device__ __forceinline__ void permute_plain(uint32_t (&A)[25], uint32_t (&B)[25]) {
-    if constexpr (LOOPED) keccak_f1600_looped(A, B);
-    else keccak_f1600_plain<false>(A, B);
+    keccak_f1600_plain<false, LOOPED ? 24 : 20>(A, B);
 }
 
 // One whole sponge of a message of len bytes at p with variant `variant`
