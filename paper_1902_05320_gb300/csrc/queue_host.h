@@ -55,6 +55,15 @@ int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *le
                 const uint32_t *out_lens, uint8_t *digests, uint64_t n, uint8_t *scratch, const QueueConfig &cfg,
                 uint64_t grid, int sm_count, unsigned int *status, cudaStream_t stream, const AuxStream *aux);
 
+// Whether a batch of n messages takes the single launch of one warp per message:
+// few enough messages, and no knob that asks for the queue.
+bool ragged_small(uint64_t n, int sm_count);
+
+// Enqueues that launch: no scratch, no allocation, no synchronisation.
+int ragged_small_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens, const uint8_t *variants,
+                       const uint32_t *out_lens, uint8_t *digests, uint64_t n, unsigned int *status,
+                       cudaStream_t stream);
+
 // keccak_batch's queue path: configuration from knobs, tuned entries and the
 // cache file; graph capture and replay.
 int launch_ragged_queue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens, const uint8_t *variants,

@@ -71,6 +71,35 @@ __global__ void __launch_bounds__(32)
     }
 }
 
+// A batch of at most kCoopPerSm messages per SM in one launch: block i is the warp
+// of message i, and sums the output sizes before it for its digest's place, so
+// there is no work order, no scratch and no launch but this one.  The queue's five
+// launches (a memset and four kernels, one of them a single block) took 72 us for
+// 200 messages of up to 600 bytes, of which the hashing's chain of nine
+// permutations is 14 on this form.
+__global__ void __launch_bounds__(32)
+    k_sha3_ragged_coop(const uint8_t *__restrict__ msgs, const uint64_t *__restrict__ offsets,
+                       const uint64_t *__restrict__ lens, const uint8_t *__restrict__ variants,
+                       const uint32_t *__restrict__ out_lens, uint8_t *__restrict__ digests, unsigned int *status) {
+    __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
+    const uint32_t i = blockIdx.x, lane = threadIdx.x;
+    const int v = variants[i];
+    const uint32_t dlen = out_lens[i];
+    const uint8_t *p = msgs + offsets[i];
+    const uint64_t len = lens[i];
+    uint64_t before = 0;
+#pragma unroll 8
+    for (uint32_t j = lane; j < i; j += 32) before += out_lens[j];
+    const Coop c(mem);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    if (v > 5 || (v < 4 && dlen != uint32_t(variant_digest(v)))) {
+        if (lane == 0) atomicOr(status, v > 5 ? KB_DEV_BAD_VARIANT : KB_DEV_BAD_OUTLEN);
+        return;
+    }
+    coop_sponge(c, p, len, v, digests + before, dlen);
+}
+
 namespace {
 
 // Per-variant control schedule: one launch per variant, each over the
@@ -236,6 +265,20 @@ int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *le
         if (e != cudaSuccess) return KB_ERR_CUDA;
     }
     if (k && cudaStreamWaitEvent(stream, aux->join, 0) != cudaSuccess) return KB_ERR_CUDA;
+    return cuda_status(cudaGetLastError());
+}
+
+bool ragged_small(uint64_t n, int sm_count) {
+    return n <= kCoopPerSm * uint64_t(sm_count > 0 ? sm_count : 1) &&
+           tuning_get(KB_TUNE_RAGGED_SCHEDULE) == KB_SCHEDULE_QUEUE && tuning_get(KB_TUNE_QUEUE_MIN_BLOCKS) == 0 &&
+           tuning_get(KB_TUNE_QUEUE_BLOCKS_PER_SM) == 0 && tuning_get(KB_TUNE_QUEUE_STAGING) == 0 &&
+           tuning_get(KB_TUNE_QUEUE_WARP_MESSAGES) < 0;
+}
+
+int ragged_small_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens, const uint8_t *variants,
+                       const uint32_t *out_lens, uint8_t *digests, uint64_t n, unsigned int *status,
+                       cudaStream_t stream) {
+    k_sha3_ragged_coop<<<unsigned(n), 32, 0, stream>>>(msgs, offsets, lens, variants, out_lens, digests, status);
     return cuda_status(cudaGetLastError());
 }
 
@@ -552,6 +595,8 @@ int launch_ragged_queue(const uint8_t *msgs, const uint64_t *offsets, const uint
         cudaStreamIsCapturing(stream, &cap0) == cudaSuccess && cap0 == cudaStreamCaptureStatusNone &&
         !have_tuned(n, dev))
         return autotune_ragged_queue(msgs, offsets, lens, variants, out_lens, digests, n, stream, dev, nullptr);
+    if (ragged_small(n, dev.sm_count))
+        return ragged_small_issue(msgs, offsets, lens, variants, out_lens, digests, n, dev.d_status, stream);
     const size_t bytes = queue_scratch_bytes(n);
     uint8_t *scratch = static_cast<uint8_t *>(stream_scratch(stream, bytes, &err));
     if (!scratch) return err;

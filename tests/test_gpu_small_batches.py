@@ -69,3 +69,53 @@ def test_batch_sizes_around_the_lines(cuda_lib, edge, blocks):
         blob = data.tobytes()
         for i in range(n):
             assert got[i].tobytes() == hashlib.sha3_256(blob[i * length:(i + 1) * length]).digest(), (n, i)
+
+
+def run_ragged(cuda_lib, b, noalloc=False):
+    """(output bytes with 0xEE where nothing was written, device status) of a RaggedBatch."""
+    import torch
+
+    view = {8: np.int64, 4: np.int32, 1: np.uint8}
+    args = [torch.from_numpy(np.ascontiguousarray(a).view(view[a.itemsize])).cuda()
+            for a in (b.msgs, b.offsets, b.lens, b.variants, b.out_lens)]
+    out = torch.full((b.total_out() + 16,), 0xEE, dtype=torch.uint8, device="cuda")
+    cuda_lib.keccak_last_error()
+    (cuda_lib.keccak_batch_noalloc if noalloc else cuda_lib.keccak_batch)(*args, out, b.n)
+    err = cuda_lib.keccak_last_error()
+    got = out.cpu().numpy()
+    assert (got[b.total_out():] == 0xEE).all()
+    return got[:b.total_out()], err
+
+
+def want_ragged(b):
+    blob = b.msgs.tobytes()
+    return b"".join(want(int(v), blob[int(o):int(o) + int(n)], int(d))
+                    for o, n, v, d in zip(b.offsets, b.lens, b.variants, b.out_lens))
+
+
+@pytest.mark.parametrize("noalloc", [False, True])
+@pytest.mark.parametrize("per_sm,more", [(0, 1), (0, 2), (0, 33), (12, 0), (12, 1), (40, 0)])
+def test_ragged_sizes_around_the_line(cuda_lib, per_sm, more, noalloc):
+    import torch
+
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + more
+    b = W.ragged_batch(n, seed=n, max_len=1500, shake_out=(0, 400), gap=3)
+    got, err = run_ragged(cuda_lib, b, noalloc)
+    assert err == 0 and got.tobytes() == want_ragged(b)
+
+
+def test_ragged_small_skips_bad_descriptors(cuda_lib):
+    b = W.ragged_batch(300, seed=5, max_len=900, gap=2)
+    bad = [3, 299] + [int(i) for i in np.flatnonzero(b.variants < 4)[5:8]]
+    b.variants[bad[:2]] = 9
+    b.out_lens[bad[2:]] += 1
+    got, err = run_ragged(cuda_lib, b)
+    assert err == cuda_lib.KB_DEV_BAD_VARIANT | cuda_lib.KB_DEV_BAD_OUTLEN
+    blob, ends = b.msgs.tobytes(), np.cumsum(b.out_lens.astype(np.int64))
+    for i in range(b.n):
+        part = got[int(ends[i]) - int(b.out_lens[i]):int(ends[i])]
+        if i in bad:
+            assert (part == 0xEE).all(), i
+        else:
+            o, k = int(b.offsets[i]), int(b.lens[i])
+            assert part.tobytes() == want(int(b.variants[i]), blob[o:o + k], int(b.out_lens[i])), i
