@@ -83,6 +83,9 @@ __global__ void __launch_bounds__(32)
                        const uint32_t *__restrict__ out_lens, uint8_t *__restrict__ digests, unsigned int *status) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     const uint32_t i = blockIdx.x, lane = threadIdx.x;
+    launch_next();
+    const Coop c(mem);
+    launch_wait();
     const int v = variants[i];
     const uint32_t dlen = out_lens[i];
     const uint8_t *p = msgs + offsets[i];
@@ -90,7 +93,6 @@ __global__ void __launch_bounds__(32)
     uint64_t before = 0;
 #pragma unroll 8
     for (uint32_t j = lane; j < i; j += 32) before += out_lens[j];
-    const Coop c(mem);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
     if (v > 5 || (v < 4 && dlen != uint32_t(variant_digest(v)))) {
@@ -278,8 +280,8 @@ bool ragged_small(uint64_t n, int sm_count) {
 int ragged_small_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens, const uint8_t *variants,
                        const uint32_t *out_lens, uint8_t *digests, uint64_t n, unsigned int *status,
                        cudaStream_t stream) {
-    k_sha3_ragged_coop<<<unsigned(n), 32, 0, stream>>>(msgs, offsets, lens, variants, out_lens, digests, status);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_overlapped(k_sha3_ragged_coop, unsigned(n), 32, 0, stream, msgs, offsets, lens, variants,
+                                         out_lens, digests, status));
 }
 
 uint64_t queue_grid_for(const QueueConfig &cfg, uint64_t n, int device, int sm_count) {

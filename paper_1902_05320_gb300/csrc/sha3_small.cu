@@ -18,8 +18,10 @@ __global__ void __launch_bounds__(32)
     k_sha3_uniform_coop(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len, int variant,
                         uint8_t *__restrict__ out, uint32_t out_len) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
+    launch_next();
     const Coop c(mem);
     const uint64_t m = blockIdx.x;
+    launch_wait();
     coop_sponge(c, msgs + m * stride, len, variant, out + m * out_len, out_len);
 }
 
@@ -27,7 +29,9 @@ template <int V>
 __global__ void __launch_bounds__(kThreads)
     k_sha3_uniform_pair(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len, uint8_t *__restrict__ out,
                         uint32_t out_len, uint64_t n) {
+    launch_next();
     const uint64_t m = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 1;
+    launch_wait();
     pair_sponge<Variant<V>::rate, Variant<V>::domain>(m < n, msgs + m * stride, len, out + m * out_len, out_len);
 }
 
@@ -35,9 +39,8 @@ template <int V>
 int launch_pair(const uint8_t *msgs, uint64_t stride, uint64_t len, uint32_t out_len, uint8_t *digests, uint64_t n,
                 cudaStream_t stream) {
     const uint64_t per_block = kThreads / 2;
-    k_sha3_uniform_pair<V><<<unsigned((n + per_block - 1) / per_block), kThreads, 0, stream>>>(msgs, stride, len,
-                                                                                                digests, out_len, n);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_overlapped(k_sha3_uniform_pair<V>, unsigned((n + per_block - 1) / per_block), kThreads, 0,
+                                         stream, msgs, stride, len, digests, out_len, n));
 }
 
 }  // namespace
@@ -50,8 +53,8 @@ bool launch_uniform_small(const uint8_t *msgs, uint64_t stride, uint64_t len, in
     const uint32_t rate = uint32_t(variant_rate(variant));
     const bool one = len < rate && out_len <= rate;
     if (n <= (one ? kCoopOnePerSm : kCoopPerSm) * sms) {
-        k_sha3_uniform_coop<<<unsigned(n), 32, 0, stream>>>(msgs, stride, len, variant, digests, out_len);
-        *rc = cuda_status(cudaGetLastError());
+        *rc = cuda_status(launch_overlapped(k_sha3_uniform_coop, unsigned(n), 32, 0, stream, msgs, stride, len, variant,
+                                            digests, out_len));
         return true;
     }
     if (one || n > kPairPerSm * sms) return false;

@@ -39,6 +39,8 @@ __global__ void __launch_bounds__(kThreads, LEN == -1 ? kMinBlocks : kOneBlockMi
     k_sha3_uniform(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len_rt,
                    uint8_t *__restrict__ out, uint32_t out_len, uint64_t n) {
     using P = Variant<V>;
+    launch_next();
+    launch_wait();
     const uint64_t len = LEN >= 0 ? uint64_t(LEN) : len_rt;
     const uint32_t dlen = P::digest ? uint32_t(P::digest) : out_len;
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
@@ -119,12 +121,14 @@ __global__ void __launch_bounds__(kThreads, kOneBlockMinBlocks)
         bulk_copy_g2s(buf[b], msgs + first * 64, bytes, &bar[b]);
         ++uses[b];
     };
+    launch_next();
     if (threadIdx.x == 0) {
         mbar_init(&bar[0], 1);
         mbar_init(&bar[1], 1);
         fence_barrier_init();
     }
     __syncthreads();
+    launch_wait();
     if (threadIdx.x == 0) {
         if (blockIdx.x < ntiles) issue(blockIdx.x, 0);
         if (blockIdx.x + stride < ntiles) issue(blockIdx.x + stride, 1);
@@ -190,9 +194,8 @@ int launch_one(const uint8_t *msgs, uint64_t stride, uint64_t len, uint32_t out_
     const uint64_t need = (n + kThreads - 1) / kThreads;
     const uint64_t grid = len < uint64_t(Variant<V>::rate) ? persistent_grid(fn, kThreads, 0, n, dev)
                                                            : std::min<uint64_t>(need, uint64_t(INT32_MAX));
-    k_sha3_uniform<V, LEN, A8, Rep><<<unsigned(grid), kThreads, 0, stream>>>(msgs, stride, len, digests,
-                                                                              out_len, n);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_overlapped(k_sha3_uniform<V, LEN, A8, Rep>, unsigned(grid), kThreads, 0, stream, msgs,
+                                         stride, len, digests, out_len, n));
 }
 
 template <int V>
@@ -200,9 +203,8 @@ int launch_tma(const uint8_t *msgs, uint32_t out_len, uint8_t *digests, uint64_t
                const DeviceInfo &dev) {
     const void *fn = reinterpret_cast<const void *>(&k_sha3_uniform64_tma<V, PlainRep>);
     const uint64_t grid = persistent_grid(fn, kThreads, 0, n, dev);
-    k_sha3_uniform64_tma<V, PlainRep><<<unsigned(grid), kThreads, 0, stream>>>(msgs, digests, out_len, n,
-                                                                                 dev.d_status);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_overlapped(k_sha3_uniform64_tma<V, PlainRep>, unsigned(grid), kThreads, 0, stream, msgs,
+                                         digests, out_len, n, dev.d_status));
 }
 
 // True when p is device memory of this device (not host-mapped, not a peer's).

@@ -119,3 +119,31 @@ def test_ragged_small_skips_bad_descriptors(cuda_lib):
         else:
             o, k = int(b.offsets[i]), int(b.lens[i])
             assert part.tobytes() == want(int(b.variants[i]), blob[o:o + k], int(b.out_lens[i])), i
+
+
+@pytest.mark.parametrize("n,pad", [(3, 0), (3, 200), (2500, 200), (5000, 0), (20000, 0), (20000, 32)])
+def test_chained_calls_see_each_other(cuda_lib, n, pad):
+    """Launches overlap the set-up of the next one with the end of the last: each call here reads what the call
+    before it wrote and overwrites what the one before that read, with a torch copy in between now and then."""
+    import torch
+
+    length = 32 + pad
+    rng = np.random.default_rng(n + pad)
+    start = rng.integers(0, 256, size=(n, length), dtype=np.uint8)
+    a, b = torch.from_numpy(start).cuda(), torch.from_numpy(start).cuda()
+    d, d2 = (torch.empty((n, 32), dtype=torch.uint8, device="cuda") for _ in range(2))
+    ref = [start[i].tobytes() for i in range(min(n, 64))]
+    for step in range(24):
+        # The first 32 bytes of every message become its digest.
+        cuda_lib.keccak_batch_uniform(a, length, length, 1, 32, d, n)
+        if step % 3 == 0:
+            b[:, :32].copy_(d)
+        else:
+            cuda_lib.keccak_batch_uniform(d, 32, 32, 1, 32, d2, n)
+            b[:, :32].copy_(d2)
+        a, b = b, a
+        b.copy_(a)
+        ref = [(hashlib.sha3_256(m).digest() if step % 3 == 0 else
+                hashlib.sha3_256(hashlib.sha3_256(m).digest()).digest()) + m[32:] for m in ref]
+    got = a.cpu().numpy()
+    assert [got[i].tobytes() for i in range(len(ref))] == ref
