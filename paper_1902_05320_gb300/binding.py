@@ -125,11 +125,28 @@ def _ptr(x) -> int | None:
     raise TypeError(f"cannot take the address of {type(x).__name__}")
 
 
+_current_stream = None
+
+
+def _bind_current_stream():
+    """Torch's current stream as a plain handle.  torch.cuda.current_stream() builds a Stream object, 2.9 us of the
+    7.4 us a small call took; the handle alone is read in 0.3 us where torch offers it."""
+    global _current_stream
+    import torch
+
+    torch.cuda.current_stream()  # initialises CUDA, or raises as it did
+    raw, device = (getattr(torch._C, name, None) for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+    if raw is None or device is None:
+        _current_stream = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
+    else:
+        _current_stream = lambda: raw(device())  # noqa: E731
+
+
 def _stream(stream) -> int | None:
     if stream is None:
-        import torch
-
-        return torch.cuda.current_stream().cuda_stream
+        if _current_stream is None:
+            _bind_current_stream()
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
