@@ -145,7 +145,8 @@ int keccak_batch_autotune(const uint8_t *msgs, const uint64_t *offsets, const ui
  *                  (below)
  *   warp_messages  threads per message: the warp_messages costliest messages
  *                  run one warp (32 threads) each, the rest one thread each;
- *                  0 = one thread for every message
+ *                  0 = as many as the plan of each batch finds worth it (none
+ *                  where the KB_TUNE_QUEUE_WARP_MESSAGES knob is 0)
  *   ms             keccak_batch_autotune_ex: time of the chosen configuration
  *                  on the tuned batch; 0 elsewhere
  */
@@ -537,10 +538,12 @@ void keccak_release(void);
  *     The looped forms exist for register budgets 2..4 (KB_QUEUE_STAGING_REGS:
  *     2 and 3); with another budget the kernel loads directly.
  *   KB_TUNE_QUEUE_WARP_MESSAGES: threads per message -- -1 (default: tuned,
- *     else 0) or K >= 0: the K costliest messages of a batch run one warp each
- *     (the cooperative sponge) in a kernel started first on a side stream,
- *     concurrently with the queue kernel, which takes the rest one thread
- *     each. */
+ *     else chosen on the device from the batch's costs) or K >= 0: the K
+ *     costliest messages of a batch run one warp each (the cooperative sponge)
+ *     in a kernel beside the queue kernel, which takes the rest one thread
+ *     each.
+ *   A batch of at most 20 messages per SM, with none of the queue's knobs set,
+ *   takes neither: one launch, one warp per message, in input order. */
 #define KB_TUNE_QUEUE_STAGING 8
 #define KB_QUEUE_STAGING_DIRECT 1
 #define KB_QUEUE_STAGING_DIRECT_LOOPED 2

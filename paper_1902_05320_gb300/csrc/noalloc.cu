@@ -9,10 +9,10 @@
 // synchronise the whole device and stall unrelated work), or code that must
 // know its memory footprint before it runs.  This entry point runs the same
 // cost-bucketed queue (its prep, plan, scatter and hashing kernels, in the
-// built-in configuration, one thread per message, launched directly without
-// a graph) with the scratch in a fixed, file-scope device array instead:
-// every GPU that loads the library holds that array until the process exits,
-// and no call here allocates or frees device memory.
+// built-in configuration, launched directly without a graph) with the
+// scratch in a fixed, file-scope device array instead: every GPU that loads
+// the library holds that array until the process exits, and no call here
+// allocates or frees device memory.
 //
 // The array is shared by every call: each call overwrites it, so calls whose
 // work overlaps on the GPU (different streams, or different host threads)
@@ -128,9 +128,7 @@ extern "C" int keccak_batch_noalloc(const uint8_t *msgs, const uint64_t *offsets
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     unsigned int *status = reinterpret_cast<unsigned int *>(s.scratch);
     uint8_t *queue_scratch = s.scratch + kStatusBytes;
-    // Built-in configuration, one thread per message (no side stream needed).
-    QueueConfig cfg;
-    cfg.warp_messages = 0;
+    const QueueConfig cfg;  // the built-in configuration
     // The status word must start at zero; the control block is cleared by
     // queue_issue itself.
     if (cudaMemsetAsync(status, 0, sizeof(unsigned int), st) != cudaSuccess) return KB_ERR_CUDA;
@@ -138,5 +136,5 @@ extern "C" int keccak_batch_noalloc(const uint8_t *msgs, const uint64_t *offsets
         return ragged_small_issue(msgs, offsets, lens, variant, out_lens, digests, n, status, st);
     const uint64_t grid = queue_grid_for(cfg, n, s.device, s.sms);
     return queue_issue(msgs, offsets, lens, variant, out_lens, digests, n, queue_scratch, cfg, grid, s.sms, status,
-                       st, nullptr);
+                       st);
 }

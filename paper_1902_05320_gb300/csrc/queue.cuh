@@ -19,9 +19,10 @@
 //      queue has two ends: on every SM sub-partition the warp in the lowest
 //      hardware slot takes groups from the costly end (the longest chains
 //      start first), the others from the cheap end.
-//   Optionally k_sha3_lanes runs the first K entries of the order (the K
-//   costliest messages) one warp per message, concurrently with the queue
-//   kernel, which then covers the entries from K on.
+//   k_sha3_lanes runs the first K entries of the order (the K costliest
+//   messages; K from k_plan, or given) one warp per message, concurrently with
+//   the queue kernel, which covers the entries from K on: it is launched first and
+//   lets the queue kernel start as soon as its own blocks have.
 //
 // Why two ends.  Measured on GB300: when two warps of one sub-partition both
 // have ALU work ready, the one in the lower hardware warp slot (%warpid)
@@ -87,6 +88,8 @@ __device__ __forceinline__ uint32_t bucket_key(uint64_t len, int v, uint32_t dle
     else return cost_bucket(message_cost(len, v, dlen)) * kRateClasses + (v > 5 ? 0u : rate_class(v));
 }
 
+constexpr uint32_t kSlotWords = 48;  // SMs told apart: 192 (beyond, they share bytes, which affects speed only)
+
 struct Control {
     uint32_t count[kBuckets];        // messages per bucket
     uint32_t cursor[kBuckets];       // next free slot of each bucket in the order
@@ -94,6 +97,7 @@ struct Control {
     unsigned long long lane_head;    // hybrid: next of the first K entries (one warp each)
     unsigned long long ends;         // queue: groups taken from the back (high 32 bits) and front (low)
     unsigned long long queue_start;  // queue: first entry of the order it covers (K)
+    uint32_t slots[kSlotWords];      // queue: a byte per SM, a bit per group of four hardware warp slots in use
 };
 
 template <bool BY_VARIANT>
@@ -101,8 +105,10 @@ __global__ void __launch_bounds__(kScanThreads)
     k_prep(const uint64_t *__restrict__ lens, const uint8_t *__restrict__ variants,
            const uint32_t *__restrict__ out_lens, uint64_t n, uint64_t *__restrict__ tile_sums, Control *ctl) {
     __shared__ uint32_t hist[kBuckets];
+    launch_next();
     for (int b = threadIdx.x; b < kBuckets; b += blockDim.x) hist[b] = 0;
     __syncthreads();
+    launch_wait();
     const uint64_t base = uint64_t(blockIdx.x) * kScanTile + uint64_t(threadIdx.x) * kScanItems;
     uint64_t s = 0;
 #pragma unroll
@@ -122,10 +128,42 @@ __global__ void __launch_bounds__(kScanThreads)
         if (hist[b]) atomicAdd(&ctl->count[b], hist[b]);
 }
 
-// One block: exclusive scan of the tile sums, bucket starts in descending
-// order (bucket kBuckets-1 first), and the queue kernel's first entry.
+// Permutations of a message of bucket b (the middle of the bucket's range).
+__device__ __forceinline__ uint64_t bucket_cost(int b) {
+    const int cb = b / kRateClasses;
+    if (cb < 64) return uint64_t(cb);
+    const int e = 6 + (cb - 64) / kBucketsPerOctave, m = (cb - 64) % kBucketsPerOctave;
+    return (uint64_t(2 * (kBucketsPerOctave + m) + 1) << e) / (2 * kBucketsPerOctave);
+}
+
+// How the batch is split between one warp per message (the costliest) and one
+// thread per message (the rest), in picoseconds of a GB300: a permutation takes
+// kThreadChain in a thread of the queue kernel and kWarpChain in a warp of its
+// own; with the GPU full the queue kernel needs kThreadWork for each (4.65 G/s), and
+// the kLanesPerSm warps per SM beside it kWarpWork.  kWarpWork is fitted (alone they
+// reach 670 M/s, 1500 ps): the two kernels share the issue slots.  Batches of
+// lengths log-uniform to 64 KiB, us before, at 2200 and at 3000: 2,000 messages
+// 4123, 1706, 1727; 20,000 4120, 2335, 2386; 100,000 4127, 2813, 2904; 200,000
+// 4201, 3659, 3522; 300,000 4215, 4145, 4196.  A larger kThreadChain (6000000,
+// 7500000) gains a tenth at 20,000 and loses a tenth to a quarter at 300,000.
+constexpr uint64_t kThreadChain = 4800000, kWarpChain = 1700000, kThreadWork = 215, kWarpWork = 3000;
+constexpr uint64_t kAutoSplit = ~uint64_t(0);
+
+// One block: exclusive scan of the tile sums, bucket starts in descending order
+// (bucket kBuckets-1 first), and the queue kernel's first entry: `split`, or for
+// kAutoSplit the number of messages that are better off with a warp each.  With W
+// permutations in all, w(b) of them in buckets above b and c(b) the cost of bucket
+// b, the batch lasts about max(c(b) kThreadChain, W kThreadWork, w(b) kWarpWork,
+// c_max kWarpChain) when the buckets above b go to warps; the first term falls
+// with b, the third rises, so the split is the first b where the first is no
+// longer the largest.  (A batch big enough to fill the GPU for its longest chain's
+// time splits off nothing.)
 static __global__ void __launch_bounds__(kScanThreads)
-    k_plan(uint64_t *tile_sums, uint64_t ntiles, Control *ctl, uint64_t queue_start) {
+    k_plan(uint64_t *tile_sums, uint64_t ntiles, Control *ctl, uint64_t split) {
+    constexpr int kPer = (kBuckets + kScanThreads - 1) / kScanThreads;  // buckets per thread
+    __shared__ unsigned long long first_cut, cost_max;
+    launch_next();
+    launch_wait();
     uint64_t carry = 0;
     for (uint64_t start = 0; start < ntiles; start += kScanThreads) {
         const uint64_t i = start + threadIdx.x;
@@ -135,17 +173,51 @@ static __global__ void __launch_bounds__(kScanThreads)
         if (i < ntiles) tile_sums[i] = carry + excl;
         carry += total;
     }
-    carry = 0;
-    for (int start = 0; start < kBuckets; start += kScanThreads) {
-        const int t = start + int(threadIdx.x);
-        const int b = kBuckets - 1 - t;
-        const uint64_t v = t < kBuckets ? ctl->count[b] : 0;
-        uint64_t excl;
-        const uint64_t total = block_exclusive_scan(v, excl);
-        if (t < kBuckets) ctl->cursor[b] = uint32_t(carry + excl);
-        carry += total;
+    if (threadIdx.x == 0) {
+        first_cut = ~0ull;
+        cost_max = 0;
     }
-    if (threadIdx.x == 0) ctl->queue_start = queue_start;
+    uint32_t count[kPer];
+    uint64_t messages = 0, work = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+        count[j] = b >= 0 ? ctl->count[b] : 0u;
+        messages += count[j];
+        if (b >= 0) work += count[j] * bucket_cost(b);
+    }
+    uint64_t m0, w0;
+    block_exclusive_scan(messages, m0);
+    const uint64_t all = block_exclusive_scan(work, w0);
+    if (split == kAutoSplit) {
+#pragma unroll
+        for (int j = kPer - 1; j >= 0; --j) {
+            const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+            if (b >= 0 && count[j]) atomicMax(&cost_max, (unsigned long long)bucket_cost(b));
+        }
+        __syncthreads();
+        uint64_t m = m0, w = w0;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+            if (b < 0) break;
+            const uint64_t chain = bucket_cost(b) * kThreadChain;
+            if (count[j] && (chain <= all * kThreadWork || chain <= w * kWarpWork || chain <= cost_max * kWarpChain))
+                atomicMin(&first_cut, (unsigned long long)m);
+            m += count[j];
+            w += count[j] * bucket_cost(b);
+        }
+        __syncthreads();
+    }
+    uint64_t m = m0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+        if (b >= 0) ctl->cursor[b] = uint32_t(m);
+        m += count[j];
+    }
+    // No bucket met the condition: every message gets a warp.
+    if (threadIdx.x == 0) ctl->queue_start = split == kAutoSplit ? first_cut : split;
 }
 
 template <bool BY_VARIANT>
@@ -155,8 +227,10 @@ __global__ void __launch_bounds__(kScanThreads)
               uint64_t *__restrict__ out_off, uint32_t *__restrict__ order, Control *ctl) {
     __shared__ uint32_t hist[kBuckets];
     __shared__ uint32_t start[kBuckets];
+    launch_next();
     for (int b = threadIdx.x; b < kBuckets; b += blockDim.x) hist[b] = 0;
     __syncthreads();
+    launch_wait();
     const uint64_t base = uint64_t(blockIdx.x) * kScanTile + uint64_t(threadIdx.x) * kScanItems;
     uint32_t d[kScanItems], key[kScanItems], rank[kScanItems];
     uint64_t s = 0;
@@ -207,9 +281,24 @@ __global__ void __launch_bounds__(kThreads, MINB)
     const int lane = threadIdx.x & 31;
     const uint64_t start = ctl->queue_start;
     const unsigned long long ngroups = n > start ? (n - start + 31) / 32 : 0;
-    unsigned slot;
-    asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
-    const bool front = slot < 4;  // the lowest hardware slot of each sub-partition
+    // Whether this warp is in the lowest hardware slot of its sub-partition that a
+    // warp of this kernel holds: warps of k_sha3_lanes may sit below.
+    bool front;
+    {
+        unsigned slot, sm;
+        asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
+        asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+        sm %= 4 * kSlotWords;
+        const uint32_t bit = 1u << (slot < 28 ? slot / 4 : 7u);
+        uint32_t *word = &ctl->slots[sm / 4];
+        uint32_t held = 0;
+        if (lane == 0) {
+            atomicOr(word, bit << (8 * (sm & 3)));
+            __nanosleep(400);  // the SM's other blocks start within this time, if they start now
+            held = atomicOr(word, 0u) >> (8 * (sm & 3));
+        }
+        front = (__shfl_sync(0xffffffffu, held, 0) & 0xffu & (bit - 1)) == 0;
+    }
     for (;;) {
         // One atomic on both ends: group g is taken at most once, from the
         // front (g = f) or the back (g = ngroups - 1 - b), and the two ends
@@ -242,6 +331,7 @@ __global__ void __launch_bounds__(kThreads, MINB)
             }
         }
     }
+    launch_wait();  // for k_sha3_lanes, beside which this kernel runs
 }
 
 // Device scratch of one call for n messages (the layout queue_issue carves):

@@ -18,22 +18,26 @@ struct QueueConfig {
     int minb = 2;               // register budget: blocks of 128 threads per SM compiled for
     int blocks_per_sm = 0;      // blocks per SM of the launch (0: as many as fit)
     int stage = 2 | 4;          // how message blocks are read: registers, looped permutation (kStageRegs | kLooped)
-    int64_t warp_messages = 0;  // the K costliest messages run one warp each (0: one thread for every message)
+    int64_t warp_messages = 0;  // the K costliest messages run one warp each, unless auto_split
+    bool auto_split = true;     // K from the batch's costs (k_plan)
     bool lanes = false;         // control: every message one warp
     bool per_variant = false;   // control: one launch per variant, unsorted
     float ms = 0;               // the autotuner's time for this configuration
 };
 
-// The hybrid splits the autotuner tries on its best one-thread-per-message
-// configuration: one warp each for the 32 or the 608 (4 per SM on 152 SMs)
-// costliest messages.
+// The fixed splits the autotuner tries on its best configuration beside the plan's
+// own: one warp each for the 32 or the 608 (4 per SM on 152 SMs) costliest messages.
 constexpr int64_t kHybridChoices[] = {32, 608};
 
-// Side stream and fork/join events of the hybrid schedule for one stream.
-struct AuxStream {
-    cudaStream_t side = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
-};
+// Warps per SM of the kernel that gives the costliest messages a warp each.  On
+// 100,000 messages to 64 KiB: 3.5 ms at 4, 3.2 to 3.4 at 6, 2.8 at 8, 2.9 at 12.
+constexpr uint64_t kLanesPerSm = 8;
+
+// Messages per SM up to which a ragged batch takes the single launch of one warp
+// per message, in input order.  Equal long messages bound it: 1.4 ns a permutation
+// with every SM busy, against 4.6 us for any number up to 128 per SM in threads,
+// cross at 21.
+constexpr uint64_t kRaggedCoopPerSm = 20;
 
 // Device scratch of one call for n messages: the queue's control block, the
 // digest offsets (8 B per message), the scan's tile sums and the work order
@@ -50,10 +54,10 @@ uint64_t queue_grid_for(const QueueConfig &cfg, uint64_t n, int device, int sm_c
 // Enqueues the whole pipeline on `stream` using `scratch`
 // (queue_scratch_bytes(n) bytes, 256-byte aligned): no allocation, no
 // synchronisation.  status is the device status word per-message errors go
-// to; aux is required when cfg.warp_messages > 0.
+// to.
 int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens, const uint8_t *variants,
                 const uint32_t *out_lens, uint8_t *digests, uint64_t n, uint8_t *scratch, const QueueConfig &cfg,
-                uint64_t grid, int sm_count, unsigned int *status, cudaStream_t stream, const AuxStream *aux);
+                uint64_t grid, int sm_count, unsigned int *status, cudaStream_t stream);
 
 // Whether a batch of n messages takes the single launch of one warp per message:
 // few enough messages, and no knob that asks for the queue.

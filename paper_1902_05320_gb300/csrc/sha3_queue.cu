@@ -3,9 +3,9 @@
 // autotuner, plus the direct-load instances of the queue kernel and the two
 // control schedules.
 //
-// The five operations of a call (a memset and four kernels; six and a fork
-// onto a side stream when the costliest messages run one warp each) are
-// captured once per call signature into a CUDA graph and replayed afterwards.
+// The six operations of a call (a memset and five kernels, the last two side by
+// side) are captured once per call signature into a CUDA graph and replayed
+// afterwards.
 // A control schedule groups the messages by variant instead and hashes each
 // variant with its own launch (the plain per-variant form the queue is
 // measured against).
@@ -17,9 +17,9 @@
 //   * staging: direct loads, or each thread's next block copied into shared
 //     memory during the permutation (with the runtime-rate or the
 //     rate-specialised absorb);
-//   * threads per message: 1 for every message, or a hybrid in which the K
-//     costliest messages run one warp each (the cooperative sponge) in a
-//     kernel launched first on a side stream, concurrently with the queue.
+//   * threads per message: the K costliest messages run one warp each (the
+//     cooperative sponge) in a kernel beside the queue's, K chosen by the plan for
+//     each batch unless a knob or a tuned entry fixes it.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -43,16 +43,20 @@ static_assert(kb::QueueConfig().stage == (kb::kStageRegs | kb::kLooped), "defaul
 
 namespace kb {
 
-// One warp per message (the cooperative sponge of coop_sponge.cuh) over entries
-// [0, limit) of the order, taken one at a time from *head; one warp per block, so
-// that the warps spread over the SMs.
+// One warp per message (the cooperative sponge of coop_sponge.cuh), over all n
+// entries of the order or over those before the queue kernel's first, taken one at
+// a time; one warp per block, so that the warps spread over the SMs.
 __global__ void __launch_bounds__(32)
     k_sha3_lanes(const uint8_t *__restrict__ msgs, const uint64_t *__restrict__ offsets,
                  const uint64_t *__restrict__ lens, const uint8_t *__restrict__ variants,
                  const uint32_t *__restrict__ out_lens, const uint64_t *__restrict__ out_off,
-                 const uint32_t *__restrict__ order, uint8_t *__restrict__ digests, uint64_t limit,
-                 unsigned long long *head, unsigned int *status) {
+                 const uint32_t *__restrict__ order, uint8_t *__restrict__ digests, uint64_t n, bool all, Control *ctl,
+                 unsigned int *status) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
+    const uint64_t limit = all || ctl->queue_start > n ? n : ctl->queue_start;
+    unsigned long long *head = all ? &ctl->head : &ctl->lane_head;
+    if (limit == 0) return;
+    launch_next();  // the queue kernel needs nothing of this one
     const Coop c(mem);
     const int lane = threadIdx.x & 31;
     for (;;) {
@@ -71,7 +75,7 @@ __global__ void __launch_bounds__(32)
     }
 }
 
-// A batch of at most kCoopPerSm messages per SM in one launch: block i is the warp
+// A batch of at most kRaggedCoopPerSm messages per SM in one launch: block i is the warp
 // of message i, and sums the output sizes before it for its digest's place, so
 // there is no work order, no scratch and no launch but this one.  The queue's five
 // launches (a memset and four kernels, one of them a single block) took 72 us for
@@ -209,11 +213,10 @@ bool queue_config_valid(const QueueConfig &cfg) {
 }
 
 // Enqueues the whole ragged pipeline on `stream` (capturable: no allocation,
-// no synchronisation, no occupancy queries once the grid is known).  A
-// hybrid configuration forks onto aux->side and joins back.
+// no synchronisation, no occupancy queries once the grid is known).
 int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens, const uint8_t *variants,
                 const uint32_t *out_lens, uint8_t *digests, uint64_t n, uint8_t *scratch, const QueueConfig &cfg,
-                uint64_t grid, int sm_count, unsigned int *status, cudaStream_t stream, const AuxStream *aux) {
+                uint64_t grid, int sm_count, unsigned int *status, cudaStream_t stream) {
     const uint64_t ntiles = digest_offsets_tiles(n);
     const Buffers bf = carve(scratch, n, ntiles);
     if (cudaMemsetAsync(bf.ctl, 0, sizeof(Control), stream) != cudaSuccess) return KB_ERR_CUDA;
@@ -232,46 +235,48 @@ int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *le
         k_flag_invalid_variants<<<1, 1, 0, stream>>>(bf.ctl, status);
         return cuda_status(cudaGetLastError());
     }
-    // The warp-per-message share: the K costliest messages (entries [0, K) of
-    // the order); the queue kernel starts after them.
-    const uint64_t k = cfg.lanes ? 0 : std::min<uint64_t>(uint64_t(cfg.warp_messages), n);
-    if (k && !aux) return KB_ERR_INVALID;
+    // The warp-per-message share: the costliest messages (the order's first
+    // entries), as many as k_plan finds or a fixed number.
+    const uint64_t fixed = std::min<uint64_t>(uint64_t(cfg.warp_messages), n);
+    const uint64_t split = cfg.lanes ? 0 : cfg.auto_split ? kAutoSplit : fixed;
     k_prep<false><<<unsigned(ntiles), kScanThreads, 0, stream>>>(lens, variants, out_lens, n, bf.tile_sums, bf.ctl);
-    k_plan<<<1, kScanThreads, 0, stream>>>(bf.tile_sums, ntiles, bf.ctl, k);
-    k_scatter<false><<<unsigned(ntiles), kScanThreads, 0, stream>>>(lens, variants, out_lens, n, bf.tile_sums,
-                                                                    bf.out_off, bf.order, bf.ctl);
-    if (k) {
-        if (cudaEventRecord(aux->fork, stream) != cudaSuccess || cudaStreamWaitEvent(aux->side, aux->fork, 0) != cudaSuccess)
-            return KB_ERR_CUDA;
-        const uint64_t warps = std::min<uint64_t>(k, uint64_t(4) * uint64_t(sm_count > 0 ? sm_count : 1));
-        k_sha3_lanes<<<unsigned(warps), 32, 0, aux->side>>>(msgs, offsets, lens, variants, out_lens, bf.out_off,
-                                                             bf.order, digests, k, &bf.ctl->lane_head, status);
-        if (cudaEventRecord(aux->join, aux->side) != cudaSuccess) return KB_ERR_CUDA;
+    if (launch_overlapped(k_plan, 1, kScanThreads, 0, stream, bf.tile_sums, ntiles, bf.ctl, split) != cudaSuccess ||
+        launch_overlapped(k_scatter<false>, unsigned(ntiles), kScanThreads, 0, stream, lens, variants, out_lens, n,
+                          bf.tile_sums, bf.out_off, bf.order, bf.ctl) != cudaSuccess)
+        return KB_ERR_CUDA;
+    if (cfg.lanes) {
+        k_sha3_lanes<<<unsigned(grid), 32, 0, stream>>>(msgs, offsets, lens, variants, out_lens, bf.out_off, bf.order,
+                                                       digests, n, true, bf.ctl, status);
+        return cuda_status(cudaGetLastError());
     }
-    if (k < n || cfg.lanes) {
-        unsigned long long *head = &bf.ctl->head;
-        const void *fn = cfg.lanes ? reinterpret_cast<const void *>(&k_sha3_lanes) : queue_kernel(cfg.minb, cfg.stage);
-        if (!fn) return KB_ERR_INVALID;
-        cudaError_t e;
-        if (cfg.lanes) {
-            uint64_t limit = n;
-            void *args[] = {&msgs, &offsets, &lens, &variants, &out_lens, const_cast<uint64_t **>(&bf.out_off),
-                            const_cast<uint32_t **>(&bf.order), &digests, &limit, &head, &status};
-            e = cudaLaunchKernel(fn, dim3(unsigned(grid)), dim3(32), args, 0, stream);
-        } else {
-            Control *ctl = bf.ctl;
-            void *args[] = {&msgs, &offsets, &lens, &variants, &out_lens, const_cast<uint64_t **>(&bf.out_off),
-                            const_cast<uint32_t **>(&bf.order), &digests, &n, &ctl, &status};
-            e = cudaLaunchKernel(fn, dim3(unsigned(grid)), dim3(kThreads), args, 0, stream);
-        }
-        if (e != cudaSuccess) return KB_ERR_CUDA;
+    if (split != 0) {
+        const uint64_t most = kLanesPerSm * uint64_t(sm_count > 0 ? sm_count : 1);
+        k_sha3_lanes<<<unsigned(std::min(cfg.auto_split ? n : fixed, most)), 32, 0, stream>>>(
+            msgs, offsets, lens, variants, out_lens, bf.out_off, bf.order, digests, n, false, bf.ctl, status);
+        if (cudaGetLastError() != cudaSuccess) return KB_ERR_CUDA;
     }
-    if (k && cudaStreamWaitEvent(stream, aux->join, 0) != cudaSuccess) return KB_ERR_CUDA;
-    return cuda_status(cudaGetLastError());
+    if (!cfg.auto_split && fixed == n) return KB_OK;  // every message has a warp
+    const void *fn = queue_kernel(cfg.minb, cfg.stage);
+    if (!fn) return KB_ERR_INVALID;
+    Control *ctl = bf.ctl;
+    void *args[] = {&msgs, &offsets, &lens, &variants, &out_lens, const_cast<uint64_t **>(&bf.out_off),
+                    const_cast<uint32_t **>(&bf.order), &digests, &n, &ctl, &status};
+    // Beside k_sha3_lanes: both need k_scatter alone, which had ended before the
+    // first block of k_sha3_lanes started.
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(unsigned(grid));
+    lc.blockDim = dim3(kThreads);
+    lc.stream = stream;
+    lc.attrs = &attr;
+    lc.numAttrs = split != 0 ? 1 : 0;
+    return cuda_status(cudaLaunchKernelExC(&lc, fn, args));
 }
 
 bool ragged_small(uint64_t n, int sm_count) {
-    return n <= kCoopPerSm * uint64_t(sm_count > 0 ? sm_count : 1) &&
+    return n <= kRaggedCoopPerSm * uint64_t(sm_count > 0 ? sm_count : 1) &&
            tuning_get(KB_TUNE_RAGGED_SCHEDULE) == KB_SCHEDULE_QUEUE && tuning_get(KB_TUNE_QUEUE_MIN_BLOCKS) == 0 &&
            tuning_get(KB_TUNE_QUEUE_BLOCKS_PER_SM) == 0 && tuning_get(KB_TUNE_QUEUE_STAGING) == 0 &&
            tuning_get(KB_TUNE_QUEUE_WARP_MESSAGES) < 0;
@@ -290,48 +295,6 @@ uint64_t queue_grid_for(const QueueConfig &cfg, uint64_t n, int device, int sm_c
 
 namespace {
 
-// ---- side streams of the hybrid schedule, one per (device, stream) -----------
-
-std::mutex g_aux_mu;
-std::map<std::pair<int, cudaStream_t>, AuxStream> g_aux;
-
-// The side stream of `stream`, created on first use (outside any capture).
-const AuxStream *aux_for(int device, cudaStream_t stream, int *err) {
-    std::lock_guard<std::mutex> lk(g_aux_mu);
-    const auto key = std::make_pair(device, stream);
-    auto it = g_aux.find(key);
-    if (it != g_aux.end()) return &it->second;
-    AuxStream a;
-    int lo = 0, hi = 0;
-    cudaDeviceGetStreamPriorityRange(&lo, &hi);
-    if (cudaStreamCreateWithPriority(&a.side, cudaStreamNonBlocking, hi) != cudaSuccess ||
-        cudaEventCreateWithFlags(&a.fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&a.join, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        if (a.side) cudaStreamDestroy(a.side);
-        if (a.fork) cudaEventDestroy(a.fork);
-        if (a.join) cudaEventDestroy(a.join);
-        *err = KB_ERR_CUDA;
-        return nullptr;
-    }
-    return &g_aux.emplace(key, a).first->second;
-}
-
-void drop_aux(int device) {
-    std::lock_guard<std::mutex> lk(g_aux_mu);
-    for (auto it = g_aux.begin(); it != g_aux.end();) {
-        if (device < 0 || it->first.first == device) {
-            cudaStreamSynchronize(it->second.side);
-            cudaStreamDestroy(it->second.side);
-            cudaEventDestroy(it->second.fork);
-            cudaEventDestroy(it->second.join);
-            it = g_aux.erase(it);
-        } else {
-            ++it;
-        }
-    }
-}
-
 // ---- graph cache --------------------------------------------------------------
 
 struct GraphKey {
@@ -339,7 +302,7 @@ struct GraphKey {
     uint64_t n;
     cudaStream_t stream;
     int minb, blocks_per_sm, stage, schedule, device;
-    int64_t warp_messages;
+    int64_t warp_messages;  // -1: the plan's split
     bool operator==(const GraphKey &o) const {
         return std::memcmp(ptrs, o.ptrs, sizeof ptrs) == 0 && n == o.n && stream == o.stream && minb == o.minb &&
                blocks_per_sm == o.blocks_per_sm && stage == o.stage && schedule == o.schedule &&
@@ -468,6 +431,7 @@ QueueConfig config_of(const CacheLine &c) {
     cfg.blocks_per_sm = c.bps;
     cfg.stage = stage_of(c.staging);
     cfg.warp_messages = c.warp_messages;
+    cfg.auto_split = c.warp_messages == 0;
     return cfg;
 }
 
@@ -567,7 +531,10 @@ void apply_knobs(QueueConfig &cfg) {
     if (regs > 0) cfg.minb = int(regs);
     if (bps > 0) cfg.blocks_per_sm = int(bps);
     if (staging > 0) cfg.stage = stage_of(int(staging));
-    if (warp >= 0) cfg.warp_messages = warp;
+    if (warp >= 0) {
+        cfg.warp_messages = warp;
+        cfg.auto_split = false;
+    }
     // A register budget the chosen staging is not compiled for falls back to
     // direct loads.
     if (!queue_kernel(cfg.minb, cfg.stage)) cfg.stage = kStageDirect;
@@ -577,11 +544,8 @@ void apply_knobs(QueueConfig &cfg) {
 }
 
 void release_queue_graphs(int device) {
-    {
-        std::lock_guard<std::mutex> lk(g_graph_mu);
-        drop_graphs_locked(device);
-    }
-    drop_aux(device);
+    std::lock_guard<std::mutex> lk(g_graph_mu);
+    drop_graphs_locked(device);
 }
 
 int launch_ragged_queue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens, const uint8_t *variants,
@@ -604,14 +568,9 @@ int launch_ragged_queue(const uint8_t *msgs, const uint64_t *offsets, const uint
     if (!scratch) return err;
     const QueueConfig cfg = choose_config(n, dev);
     const uint64_t grid = queue_grid(cfg, n, dev.device, dev.sm_count);
-    const AuxStream *aux = nullptr;
-    if (!cfg.lanes && !cfg.per_variant && cfg.warp_messages > 0) {
-        aux = aux_for(dev.device, stream, &err);
-        if (!aux) return err;
-    }
     auto run = [&] {
         return queue_issue(msgs, offsets, lens, variants, out_lens, digests, n, scratch, cfg, grid, dev.sm_count,
-                           dev.d_status, stream, aux);
+                           dev.d_status, stream);
     };
 
     // Graph replay needs a capturable stream that is not already capturing.
@@ -622,7 +581,8 @@ int launch_ragged_queue(const uint8_t *msgs, const uint64_t *offsets, const uint
 
     GraphKey key{{msgs, offsets, lens, variants, out_lens, digests, scratch},
                  n, stream, cfg.minb, cfg.blocks_per_sm, cfg.stage,
-                 cfg.per_variant ? 2 : cfg.lanes ? 1 : 0, dev.device, cfg.warp_messages};
+                 cfg.per_variant ? 2 : cfg.lanes ? 1 : 0, dev.device,
+                 cfg.auto_split ? -1 : cfg.warp_messages};
     {
         std::lock_guard<std::mutex> lk(g_graph_mu);
         for (auto it = g_graphs.begin(); it != g_graphs.end(); ++it) {
@@ -711,8 +671,6 @@ int autotune_ragged_queue(const uint8_t *msgs, const uint64_t *offsets, const ui
     int err = KB_OK;
     uint8_t *scratch = static_cast<uint8_t *>(stream_scratch(stream, queue_scratch_bytes(n), &err));
     if (!scratch) return err;
-    const AuxStream *aux = aux_for(dev.device, stream, &err);
-    if (!aux) return err;
     const Buffers bf = carve(scratch, n, digest_offsets_tiles(n));
     cudaEvent_t a = nullptr, b = nullptr;
     uint8_t *ref = nullptr;
@@ -732,7 +690,7 @@ int autotune_ragged_queue(const uint8_t *msgs, const uint64_t *offsets, const ui
         const uint64_t grid = queue_grid(cfg, n, dev.device, dev.sm_count);
         auto go = [&] {
             return queue_issue(msgs, offsets, lens, variants, out_lens, digests, n, scratch, cfg, grid, dev.sm_count,
-                               dev.d_status, stream, aux);
+                               dev.d_status, stream);
         };
         rc = go();
         if (rc == KB_OK) rc = cuda_status(cudaEventRecord(a, stream));
@@ -791,6 +749,7 @@ int autotune_ragged_queue(const uint8_t *msgs, const uint64_t *offsets, const ui
         if (rc != KB_OK || uint64_t(k) >= n) break;
         QueueConfig cfg = base;
         cfg.warp_messages = k;
+        cfg.auto_split = false;
         trial(cfg);
     }
     if (a) cudaEventDestroy(a);
@@ -808,7 +767,7 @@ int autotune_ragged_queue(const uint8_t *msgs, const uint64_t *offsets, const ui
     }
     // Leave the caller's digests from the chosen configuration.
     rc = queue_issue(msgs, offsets, lens, variants, out_lens, digests, n, scratch, best,
-                     queue_grid(best, n, dev.device, dev.sm_count), dev.sm_count, dev.d_status, stream, aux);
+                     queue_grid(best, n, dev.device, dev.sm_count), dev.sm_count, dev.d_status, stream);
     if (chosen) {
         *chosen = best;
         chosen->ms = best_t;

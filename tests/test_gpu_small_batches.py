@@ -94,7 +94,7 @@ def want_ragged(b):
 
 
 @pytest.mark.parametrize("noalloc", [False, True])
-@pytest.mark.parametrize("per_sm,more", [(0, 1), (0, 2), (0, 33), (12, 0), (12, 1), (40, 0)])
+@pytest.mark.parametrize("per_sm,more", [(0, 1), (0, 2), (0, 33), (20, 0), (20, 1), (40, 0)])
 def test_ragged_sizes_around_the_line(cuda_lib, per_sm, more, noalloc):
     import torch
 
@@ -147,3 +147,16 @@ def test_chained_calls_see_each_other(cuda_lib, n, pad):
                 hashlib.sha3_256(hashlib.sha3_256(m).digest()).digest()) + m[32:] for m in ref]
     got = a.cpu().numpy()
     assert [got[i].tobytes() for i in range(len(ref))] == ref
+
+
+@pytest.mark.parametrize("n,long_len,long_every", [(4000, 60000, 3), (9000, 60000, 40), (9000, 0, 1), (30000, 30000, 1000)])
+def test_ragged_split_between_warps_and_threads(cuda_lib, n, long_len, long_every):
+    """Batches whose plan gives a warp each to many, to a few or to all of the messages, beside the queue."""
+    rng = np.random.default_rng(n + long_every)
+    lens = rng.integers(0, 700, size=n)
+    if long_len:
+        lens[::long_every] = rng.integers(long_len // 2, long_len, size=lens[::long_every].size)
+    b = W.ragged_batch(n, seed=n + 1, lens=lens, shake_out=(0, 200), gap=3)
+    for noalloc in (False, True):
+        got, err = run_ragged(cuda_lib, b, noalloc)
+        assert err == 0 and got.tobytes() == want_ragged(b)
