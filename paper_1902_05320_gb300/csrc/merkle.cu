@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <climits>
 
+#include "coop_sponge.cuh"
 #include "keccak_core.cuh"
 #include "runtime.cuh"
 #include "sponge.cuh"
@@ -92,6 +93,8 @@ __device__ __forceinline__ void leaf_state_a8(const uint8_t *p, uint64_t leaf_by
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_merkle_leaves_a8(const uint8_t *__restrict__ buf, uint64_t n_leaves, uint64_t leaf_bytes,
                        uint8_t *__restrict__ out) {
+    launch_next();
+    launch_wait();
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n_leaves; i += step) {
         uint32_t A[25], B[25];
@@ -100,10 +103,72 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     }
 }
 
-// Any alignment / leaf size: byte-exact reads through ld_word_any.
+// Leaves at any alignment and of any size.  XORs block b of the padded message
+// 0x00 || leaf (leaf at p, nfull full blocks, rem bytes in the last) into the state.
+// The block's bytes are leaf bytes from 136 b - 1 on: lanes 1..16 are funnel shifts
+// of the aligned 32-bit words that hold them, lane 0 alone, which takes the prefix
+// in block 0, is read byte-exactly.  (Every lane byte-exactly, as before, was 45
+// instructions a lane: 2^18 leaves of 1001 bytes 670 us a tree.)
+__device__ __forceinline__ void absorb_leaf_block_any(uint32_t (&A)[25], uint32_t (&B)[25], const uint8_t *p,
+                                                      uint64_t b, uint64_t nfull, uint32_t rem) {
+    const bool full = b < nfull;
+    const uint32_t valid = full ? uint32_t(kRate) : rem;  // message bytes in this block, the prefix among them
+    uint32_t lo = 0, hi = 0;
+    const uint32_t first = valid < 8 ? valid : 8u;  // of them in lane 0
+    if (b == 0) {
+        if (first > 1) ld_word_any(p, first - 1, lo, hi);
+        hi = __funnelshift_l(lo, hi, 8);
+        lo = lo << 8;  // prefix byte 0x00
+    } else if (first) {
+        ld_word_any(p + (b * kRate - 1), first, lo, hi);
+    }
+    if (rem < 8 && !full) {
+        if (rem < 4) lo ^= uint32_t(kDomain) << (8 * rem);
+        else hi ^= uint32_t(kDomain) << (8 * (rem - 4));
+    }
+    PlainRep::xor_word(A[0], B[0], lo, hi);
+    // Lanes 1..16, leaf bytes from 136 b + 7 on.
+    const uint8_t *q = p + b * kRate + 7;
+    const uintptr_t start = reinterpret_cast<uintptr_t>(q);
+    const uint32_t *a = reinterpret_cast<const uint32_t *>(start & ~uintptr_t(3));
+    const uint32_t sh = uint32_t(start & 3) * 8;
+    if (full) {
+        uint32_t prev = __ldg(a);
+#pragma unroll
+        for (int k = 1; k < kRate / 8; ++k) {
+            const uint32_t w1 = __ldg(a + 2 * k - 1);
+            const uint32_t w2 = (k + 1 < kRate / 8 || sh != 0) ? __ldg(a + 2 * k) : 0u;
+            PlainRep::xor_word(A[k], B[k], __funnelshift_r(prev, w1, sh), __funnelshift_r(w1, w2, sh));
+            prev = w2;
+        }
+    } else {
+        // Aligned words 0 .. nw-1 hold the bytes; those past the message are masked.
+        const uint32_t left = rem > 8 ? rem - 8 : 0u;
+        const uint32_t nw = left ? uint32_t(((start + left - 1) >> 2) - (start >> 2)) + 1 : 0u;
+        int rb = int(8 * rem) - 64;  // message bits still to come, from lane k on
+        uint32_t prev = nw ? __ldg(a) : 0u;
+#pragma unroll
+        for (int k = 1; k < kRate / 8; ++k) {
+            const uint32_t w1 = uint32_t(2 * k - 1) < nw ? __ldg(a + 2 * k - 1) : 0u;
+            const uint32_t w2 = uint32_t(2 * k) < nw ? __ldg(a + 2 * k) : 0u;
+            uint32_t vl = __funnelshift_r(prev, w1, sh), vh = __funnelshift_r(w1, w2, sh);
+            prev = w2;
+            vl &= __funnelshift_lc(0xFFFFFFFFu, 0u, uint32_t(max(rb, 0)));
+            vh &= __funnelshift_lc(0xFFFFFFFFu, 0u, uint32_t(max(rb - 32, 0)));
+            if (uint32_t(rb) < 32u) vl ^= uint32_t(kDomain) << rb;
+            else if (uint32_t(rb - 32) < 32u) vh ^= uint32_t(kDomain) << (rb - 32);
+            if (k == kRate / 8 - 1) vh ^= 0x80000000u;
+            rb -= 64;
+            PlainRep::xor_word(A[k], B[k], vl, vh);
+        }
+    }
+}
+
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_merkle_leaves_any(const uint8_t *__restrict__ buf, uint64_t n_leaves, uint64_t leaf_bytes,
                         uint8_t *__restrict__ out) {
+    launch_next();
+    launch_wait();
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
     const uint64_t vlen = leaf_bytes + 1;
     const uint64_t nfull = vlen / kRate;
@@ -114,33 +179,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
 #pragma unroll
         for (int k = 0; k < 25; ++k) A[k] = B[k] = 0;
         for (uint64_t b = 0; b <= nfull; ++b) {
-            const uint32_t valid = b < nfull ? uint32_t(kRate) : rem;  // virtual bytes in this block
-#pragma unroll
-            for (int k = 0; k < kRate / 8; ++k) {
-                // Virtual bytes [v0, v0 + 8) are leaf bytes [v0 - 1, v0 + 7).
-                const uint64_t v0 = b * kRate + 8 * k;
-                uint32_t lo = 0, hi = 0;
-                const uint32_t inblk = 8 * k;
-                if (inblk < valid) {
-                    const uint32_t nv = valid - inblk < 8 ? valid - inblk : 8;  // virtual bytes present
-                    if (v0 == 0) {
-                        if (nv > 1) ld_word_any(p, nv - 1, lo, hi);
-                        hi = __funnelshift_l(lo, hi, 8);
-                        lo = (lo << 8) | 0x00u;
-                    } else {
-                        ld_word_any(p + (v0 - 1), nv, lo, hi);
-                    }
-                }
-                if (b == nfull) {
-                    if (uint32_t(k) == rem / 8) {
-                        const uint32_t sh = (rem % 8) * 8;
-                        if (sh < 32) lo ^= uint32_t(kDomain) << sh;
-                        else hi ^= uint32_t(kDomain) << (sh - 32);
-                    }
-                    if (k == kRate / 8 - 1) hi ^= 0x80000000u;
-                }
-                PlainRep::xor_word(A[k], B[k], lo, hi);
-            }
+            absorb_leaf_block_any(A, B, p, b, nfull, rem);
             PlainRep::permute<false>(A, B);
         }
         squeeze<kRate, PlainRep>(A, B, out + 32 * i, 32);
@@ -185,6 +224,8 @@ __device__ __forceinline__ void merkle_parent(const uint8_t *in, uint64_t count,
 // One level, one thread per parent.
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_merkle_level(const uint8_t *in, uint64_t count, uint8_t *out) {
+    launch_next();
+    launch_wait();
     const uint64_t parents = count / 2 + (count & 1);
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t j = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < parents; j += step)
@@ -192,38 +233,6 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
 }
 
 // ---- many small trees, one thread per tree ----------------------------------
-
-// XORs block b of the padded message 0x00 || leaf (leaf_bytes bytes at p, any
-// alignment; nfull full blocks, rem bytes in the last) into the state,
-// reading the leaf byte-exactly.
-__device__ __forceinline__ void absorb_leaf_block_any(uint32_t (&A)[25], uint32_t (&B)[25], const uint8_t *p,
-                                                      uint64_t b, uint64_t nfull, uint32_t rem) {
-    const uint32_t valid = b < nfull ? uint32_t(kRate) : rem;
-#pragma unroll
-    for (int k = 0; k < kRate / 8; ++k) {
-        const uint64_t v0 = b * kRate + 8 * k;  // virtual bytes [v0, v0+8) = leaf bytes [v0-1, v0+7)
-        uint32_t lo = 0, hi = 0;
-        if (uint32_t(8 * k) < valid) {
-            const uint32_t nv = valid - 8 * k < 8 ? valid - 8 * k : 8;
-            if (v0 == 0) {
-                if (nv > 1) ld_word_any(p, nv - 1, lo, hi);
-                hi = __funnelshift_l(lo, hi, 8);
-                lo = lo << 8;  // prefix byte 0x00
-            } else {
-                ld_word_any(p + (v0 - 1), nv, lo, hi);
-            }
-        }
-        if (b == nfull) {
-            if (uint32_t(k) == rem / 8) {
-                const uint32_t sh = (rem % 8) * 8;
-                if (sh < 32) lo ^= uint32_t(kDomain) << sh;
-                else hi ^= uint32_t(kDomain) << (sh - 32);
-            }
-            if (k == kRate / 8 - 1) hi ^= 0x80000000u;
-        }
-        PlainRep::xor_word(A[k], B[k], lo, hi);
-    }
-}
 
 // The state holding the padded block of 0x01 || left || right (digests as
 // eight little-endian 32-bit words each), ready to permute.
@@ -244,84 +253,90 @@ __device__ __forceinline__ void load_node_block(uint32_t (&A)[25], uint32_t (&B)
     B[kRate / 8 - 1] ^= 0x80000000u;
 }
 
-// Digest (eight little-endian 32-bit words) of SHA3-256(0x01 || l || r).
-__device__ __forceinline__ void node_digest(const uint32_t (&l)[8], const uint32_t (&r)[8], uint32_t (&d)[8]) {
-    uint32_t A[25], B[25];
-    load_node_block(A, B, l, r);
-    PlainRep::permute<true>(A, B);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        d[2 * k] = A[k];
-        d[2 * k + 1] = B[k];
-    }
+// Few leaves: one warp each (coop_sponge.cuh), which takes a third of the time of a
+// thread for a leaf's chain of permutations.
+__global__ void __launch_bounds__(32)
+    k_merkle_leaves_coop(const uint8_t *__restrict__ buf, uint64_t leaf_bytes, uint8_t *__restrict__ out) {
+    __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
+    const Coop c(mem);
+    const uint64_t i = blockIdx.x;
+    launch_wait();
+    coop_sponge<0, true>(c, buf + i * leaf_bytes, leaf_bytes, 1, out + 32 * i, 32);
 }
 
-// Levels where a permutation's latency, not the ALU pipe's throughput, sets
-// the time (at most kClimbParents parents: under one warp per SM
-// sub-partition), up to kClimbLevels + 1 of them in one launch.  Warp w takes
-// parents [32w, 32w + 32) of the first level, one thread each; at climb step
-// l, lane i (a multiple of 2^l) combines its node with that of lane
-// i + 2^(l-1), fetched by a shuffle, into node (32w + i) / 2^l of the next
-// level, or carries it up unchanged when it is that level's odd last node.
-// The warps' ranges nest (the children of nodes [16w, 16w + 16) of a level
-// are nodes [32w, 32w + 32) of the level below), so every node of every level
-// is computed as the level-by-level reduction computes it, and each is
-// written out.  One loop around one permutation call site covers all steps.
-constexpr uint64_t kClimbParents = 16384;
-constexpr int kClimbLevels = 5;
+// Levels where a permutation's latency, not the ALU pipe's throughput, sets the
+// time: up to kClimbLevels of them in one launch, one warp per node (coop.cuh).
+// Block b takes children [16b, 16b + 16) of the first level and all nodes above
+// them, up to one: 8 nodes, then 4, 2 and 1, handed on in shared memory; an odd
+// last node of a level is carried up.  The blocks' ranges nest (the parents of
+// nodes [16b, 16b + 16) are nodes [8b, 8b + 8) of the next level), so every node
+// is the one the level-by-level reduction gives, and each is written out.
+//
+// A node takes 1.6 us alone on its SM, more beside others (the warps of an SM share
+// its path to shared memory), where one thread per node took 4.5 whatever their
+// number.  Eight warps and four levels a launch measured best: 1000 leaves of 1001
+// bytes to the root 115 -> 47.9 us; 49.5 with four warps and three levels, 48.3 with
+// two and two, 70.7 with sixteen and five.  From kClimbPerSm parents per SM on down
+// this is the shorter way.
+constexpr int kClimbWarps = 8, kClimbLevels = 4;
+constexpr uint64_t kClimbPerSm = 16;
 
-__global__ void __launch_bounds__(kThreads) k_merkle_climb(const uint8_t *in, uint64_t count, uint8_t *out, int climb) {
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint64_t warp = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    uint64_t cnt = count;  // nodes of the level being reduced
-    const uint8_t *src = in;
-    uint8_t *dst = out;
-    uint32_t d[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int l = 0; l <= climb; ++l) {
+__global__ void __launch_bounds__(32 * kClimbWarps)
+    k_merkle_climb(const uint8_t *in, uint64_t count, uint8_t *out, int levels) {
+    __shared__ __align__(16) uint32_t mem[kClimbWarps][Coop::kWarpWords];
+    __shared__ __align__(16) uint32_t node[2][2 * kClimbWarps][8];  // digests of the level below and of this one
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const Coop c(mem[warp]);
+    uint64_t cnt = count;                            // nodes of the level below
+    uint64_t base = uint64_t(blockIdx.x) * 2 * kClimbWarps;  // this block's first of them
+    launch_wait();
+    if (threadIdx.x < 4 * kClimbWarps) {  // 16 bytes a thread; plain loads: an earlier launch wrote them
+        const uint64_t i = base + threadIdx.x / 2;
+        if (i < cnt)
+            *reinterpret_cast<uint4 *>(&node[0][threadIdx.x / 2][4 * (threadIdx.x & 1)]) =
+                reinterpret_cast<const uint4 *>(in)[2 * i + (threadIdx.x & 1)];
+    }
+    __syncthreads();
+    for (int l = 0; l < levels; ++l) {
+        const uint32_t (*child)[8] = node[l & 1];
         const uint64_t parents = cnt / 2 + (cnt & 1);
-        uint32_t lft[8], rgt[8];
-        uint64_t q;  // parent index
-        bool act;
-        if (l == 0) {
-            q = warp * 32 + lane;
-            act = q < parents;
+        if (l + 1 == levels) launch_next();
+        const uint64_t q = base / 2 + warp;  // this warp's parent, child[2 * warp] and the next
+        if (warp < uint32_t(kClimbWarps) >> l && q < parents) {
+            if (2 * q + 1 < cnt) {
+                // 0x01 || left || right, 65 bytes and their padding, in lanes 0..8 and 16.
+                const uint32_t *d = child[2 * warp];  // sixteen words: the two digests are neighbours
+                uint32_t a[2];
 #pragma unroll
-            for (int t = 0; t < 8; ++t) lft[t] = rgt[t] = 0;
-            if (act) {
-                const uint4 *c = reinterpret_cast<const uint4 *>(src + 64 * q);
-                const uint4 a = c[0], b = c[1];
-                lft[0] = a.x, lft[1] = a.y, lft[2] = a.z, lft[3] = a.w;
-                lft[4] = b.x, lft[5] = b.y, lft[6] = b.z, lft[7] = b.w;
-                if (2 * q + 1 < cnt) {
-                    const uint4 e = c[2], f = c[3];
-                    rgt[0] = e.x, rgt[1] = e.y, rgt[2] = e.z, rgt[3] = e.w;
-                    rgt[4] = f.x, rgt[5] = f.y, rgt[6] = f.z, rgt[7] = f.w;
+                for (int s = 0; s < 2; ++s) {
+                    const int k = c.lane(s);
+                    uint32_t lo = 0, hi = 0;
+                    if (k < 8) {
+                        lo = __funnelshift_l(k ? d[2 * k - 1] : 0x01000000u, d[2 * k], 8);
+                        hi = __funnelshift_l(d[2 * k], d[2 * k + 1], 8);
+                    } else if (k == 8) {
+                        lo = (d[15] >> 24) | (uint32_t(kDomain) << 8);
+                    } else if (k == kRate / 8 - 1) {
+                        hi = 0x80000000u;
+                    }
+                    a[s] = c.on && k < kRate / 8 ? c.half(lo, hi) : 0u;
                 }
+                c.permute(a, [] {});
+                const uint32_t w = c.unhalf(a[0]);
+                if (c.on && c.p == 0 && c.x < 4) {
+                    node[(l & 1) ^ 1][warp][2 * c.x + c.h] = w;
+                    reinterpret_cast<uint32_t *>(out + 32 * q)[2 * c.x + c.h] = w;
+                }
+            } else if (lane < 8) {
+                const uint32_t w = child[2 * warp][lane];
+                node[(l & 1) ^ 1][warp][lane] = w;
+                reinterpret_cast<uint32_t *>(out + 32 * q)[lane] = w;
             }
-        } else {
-            const uint32_t step = 1u << (l - 1);
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                lft[t] = d[t];
-                rgt[t] = __shfl_down_sync(0xFFFFFFFFu, d[t], step);
-            }
-            const uint64_t c = warp * (32u >> (l - 1)) + (lane >> (l - 1));  // this lane's node: the left child
-            act = (lane & (2 * step - 1)) == 0 && c < cnt;
-            q = c >> 1;
         }
-        if (act) {
-            if (2 * q + 1 < cnt) node_digest(lft, rgt, d);
-            else {
-#pragma unroll
-                for (int t = 0; t < 8; ++t) d[t] = lft[t];  // odd last node: carried up
-            }
-            uint4 *o = reinterpret_cast<uint4 *>(dst + 32 * q);
-            o[0] = make_uint4(d[0], d[1], d[2], d[3]);
-            o[1] = make_uint4(d[4], d[5], d[6], d[7]);
-        }
-        src = dst;
-        dst += 32 * parents;
+        __syncthreads();
+        out += 32 * parents;
         cnt = parents;
+        base /= 2;
     }
 }
 
@@ -432,43 +447,49 @@ uint64_t merkle_nodes(uint64_t n_leaves) {
 
 namespace {
 
-int launch_leaves(const uint8_t *buf, uint64_t n_leaves, uint64_t leaf_bytes, uint8_t *out, cudaStream_t stream) {
+int launch_leaves(const uint8_t *buf, uint64_t n_leaves, uint64_t leaf_bytes, uint8_t *out, cudaStream_t stream,
+                  const DeviceInfo &dev) {
     if (n_leaves == 0) return KB_OK;
+    const uint64_t sms = uint64_t(dev.sm_count > 0 ? dev.sm_count : 1);
+    const uint64_t few = leaf_bytes + 1 < uint64_t(kRate) ? kCoopOnePerSm : kCoopPerSm;
+    if (n_leaves <= few * sms)
+        return cuda_status(
+            launch_overlapped(k_merkle_leaves_coop, unsigned(n_leaves), 32, 0, stream, buf, leaf_bytes, out));
     const bool a8 = ((reinterpret_cast<uintptr_t>(buf) | leaf_bytes) & 7) == 0 && leaf_bytes > 0;
     // One thread per leaf and as many blocks as that takes: a leaf is a long
     // chain of permutations, and the block scheduler's dynamic placement
     // balances the last wave better than a fixed grid-stride split (measured
     // 5% faster on 4 GiB of 8 KiB leaves).
     const uint64_t grid = std::min<uint64_t>((n_leaves + kThreads - 1) / kThreads, uint64_t(INT32_MAX));
-    if (a8) k_merkle_leaves_a8<<<unsigned(grid), kThreads, 0, stream>>>(buf, n_leaves, leaf_bytes, out);
-    else k_merkle_leaves_any<<<unsigned(grid), kThreads, 0, stream>>>(buf, n_leaves, leaf_bytes, out);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_overlapped(a8 ? k_merkle_leaves_a8 : k_merkle_leaves_any, unsigned(grid), kThreads, 0,
+                                         stream, buf, n_leaves, leaf_bytes, out));
 }
 
 // Every level above the n leaf digests at `nodes`, written after them: one
-// launch per level while a level has more than kClimbParents parents (there
-// the ALU pipe's throughput sets the time), then climbing launches of up to
-// kClimbLevels + 1 levels each.
+// launch per level while a level has more than kClimbPerSm parents per SM (there
+// a thread per parent is as quick or the ALU pipe's throughput sets the time),
+// then climbing launches of up to kClimbLevels levels each.
 int launch_upper_levels(uint8_t *nodes, uint64_t n, cudaStream_t stream, const DeviceInfo &dev) {
     uint8_t *level = nodes;
     while (n > 1) {
         const uint64_t parents = n / 2 + (n & 1);
-        if (parents > kClimbParents) {
+        if (parents > kClimbPerSm * uint64_t(dev.sm_count > 0 ? dev.sm_count : 1)) {
             const uint64_t grid =
                 persistent_grid(reinterpret_cast<const void *>(&k_merkle_level), kThreads, 0, parents, dev);
-            k_merkle_level<<<unsigned(grid), kThreads, 0, stream>>>(level, n, level + 32 * n);
-            if (cudaGetLastError() != cudaSuccess) return KB_ERR_CUDA;
+            if (launch_overlapped(k_merkle_level, unsigned(grid), kThreads, 0, stream, level, n, level + 32 * n) !=
+                cudaSuccess)
+                return KB_ERR_CUDA;
             level += 32 * n;
             n = parents;
             continue;
         }
-        int climb = 0;
-        for (uint64_t m = parents; climb < kClimbLevels && m > 1; m = m / 2 + (m & 1)) ++climb;
-        const uint64_t threads = (parents + 31) / 32 * 32;
-        const uint64_t blocks = (threads + kThreads - 1) / kThreads;
-        k_merkle_climb<<<unsigned(blocks), kThreads, 0, stream>>>(level, n, level + 32 * n, climb);
-        if (cudaGetLastError() != cudaSuccess) return KB_ERR_CUDA;
-        for (int l = 0; l <= climb; ++l) {
+        int levels = 0;
+        for (uint64_t m = n; levels < kClimbLevels && m > 1; m = m / 2 + (m & 1)) ++levels;
+        const uint64_t blocks = (n + 2 * kClimbWarps - 1) / (2 * kClimbWarps);
+        if (launch_overlapped(k_merkle_climb, unsigned(blocks), 32 * kClimbWarps, 0, stream, level, n, level + 32 * n,
+                              levels) != cudaSuccess)
+            return KB_ERR_CUDA;
+        for (int l = 0; l < levels; ++l) {
             level += 32 * n;
             n = n / 2 + (n & 1);
         }
@@ -480,7 +501,7 @@ int launch_upper_levels(uint8_t *nodes, uint64_t n, cudaStream_t stream, const D
 
 int launch_merkle_levels(const uint8_t *buf, uint64_t n_leaves, uint64_t leaf_bytes, uint8_t *nodes,
                          cudaStream_t stream, const DeviceInfo &dev) {
-    int rc = launch_leaves(buf, n_leaves, leaf_bytes, nodes, stream);
+    int rc = launch_leaves(buf, n_leaves, leaf_bytes, nodes, stream, dev);
     if (rc != KB_OK) return rc;
     return launch_upper_levels(nodes, n_leaves, stream, dev);
 }
@@ -511,12 +532,11 @@ int launch_merkle_message(const uint8_t *msg, uint64_t len, uint64_t chunk_bytes
                           cudaStream_t stream, const DeviceInfo &dev) {
     const uint64_t n = merkle_message_leaves(len, chunk_bytes);
     const uint64_t full = len / chunk_bytes;
-    int rc = launch_leaves(msg, full, chunk_bytes, nodes, stream);
+    int rc = launch_leaves(msg, full, chunk_bytes, nodes, stream, dev);
     if (rc != KB_OK) return rc;
     if (full < n) {  // the short (or empty) last chunk
         const uint64_t last = len - full * chunk_bytes;
-        k_merkle_leaves_any<<<1, kThreads, 0, stream>>>(msg + full * chunk_bytes, 1, last, nodes + 32 * full);
-        if (cudaGetLastError() != cudaSuccess) return KB_ERR_CUDA;
+        if ((rc = launch_leaves(msg + full * chunk_bytes, 1, last, nodes + 32 * full, stream, dev)) != KB_OK) return rc;
     }
     return launch_upper_levels(nodes, n, stream, dev);
 }

@@ -18,6 +18,7 @@
 #include <cstdint>
 
 #include "keccak_core.cuh"
+#include "runtime.cuh"
 #include "sponge.cuh"
 
 namespace kb {
@@ -143,6 +144,7 @@ __device__ __forceinline__ void pair_sponge(bool active, const uint8_t *p, uint6
             }
             if (i + 1 < nfull) fetch(i + 1);
         } else if (i == nfull) {
+            launch_next();  // not before: the next kernel's blocks would crowd some SMs
 #pragma unroll
             for (int k = 0; k < kWords; ++k) {
                 const uint32_t at = 8 * k + 4 * h;

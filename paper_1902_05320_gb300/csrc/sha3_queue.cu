@@ -87,7 +87,6 @@ __global__ void __launch_bounds__(32)
                        const uint32_t *__restrict__ out_lens, uint8_t *__restrict__ digests, unsigned int *status) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     const uint32_t i = blockIdx.x, lane = threadIdx.x;
-    launch_next();
     const Coop c(mem);
     launch_wait();
     const int v = variants[i];
@@ -103,7 +102,7 @@ __global__ void __launch_bounds__(32)
         if (lane == 0) atomicOr(status, v > 5 ? KB_DEV_BAD_VARIANT : KB_DEV_BAD_OUTLEN);
         return;
     }
-    coop_sponge(c, p, len, v, digests + before, dlen);
+    coop_sponge<-1, true>(c, p, len, v, digests + before, dlen);
 }
 
 namespace {

@@ -18,18 +18,16 @@ __global__ void __launch_bounds__(32)
     k_sha3_uniform_coop(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len, int variant,
                         uint8_t *__restrict__ out, uint32_t out_len) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
-    launch_next();
     const Coop c(mem);
     const uint64_t m = blockIdx.x;
     launch_wait();
-    coop_sponge(c, msgs + m * stride, len, variant, out + m * out_len, out_len);
+    coop_sponge<-1, true>(c, msgs + m * stride, len, variant, out + m * out_len, out_len);
 }
 
 template <int V>
 __global__ void __launch_bounds__(kThreads)
     k_sha3_uniform_pair(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len, uint8_t *__restrict__ out,
                         uint32_t out_len, uint64_t n) {
-    launch_next();
     const uint64_t m = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 1;
     launch_wait();
     pair_sponge<Variant<V>::rate, Variant<V>::domain>(m < n, msgs + m * stride, len, out + m * out_len, out_len);

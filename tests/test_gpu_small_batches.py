@@ -160,3 +160,42 @@ def test_ragged_split_between_warps_and_threads(cuda_lib, n, long_len, long_ever
     for noalloc in (False, True):
         got, err = run_ragged(cuda_lib, b, noalloc)
         assert err == 0 and got.tobytes() == want_ragged(b)
+
+
+def tree_nodes(leaves):
+    nodes = level = [hashlib.sha3_256(b"\x00" + leaf).digest() for leaf in leaves]
+    while len(level) > 1:
+        up = [hashlib.sha3_256(b"\x01" + level[i] + level[i + 1]).digest() for i in range(0, len(level) - 1, 2)]
+        level = up + level[len(level) & ~1:]
+        nodes = nodes + level
+    return b"".join(nodes)
+
+
+@pytest.mark.parametrize("leaf_bytes", [1, 6, 7, 8, 127, 128, 134, 135, 136, 143, 144, 271, 272, 407, 1001])
+@pytest.mark.parametrize("n", [1, 2, 3, 15, 16, 17, 33, 255, 257, 1303])
+def test_merkle_small_trees_every_node(cuda_lib, n, leaf_bytes):
+    import torch
+
+    shift = (n + leaf_bytes) % 5
+    data = np.random.default_rng(n * 2000 + leaf_bytes).integers(0, 256, size=n * leaf_bytes, dtype=np.uint8)
+    raw = torch.zeros(data.size + 16, dtype=torch.uint8, device="cuda")
+    raw[shift:shift + data.size] = torch.from_numpy(data).cuda()
+    nodes = torch.empty(32 * cuda_lib.merkle_node_count(n), dtype=torch.uint8, device="cuda")
+    cuda_lib.merkle_sha3_256_levels(raw.data_ptr() + shift, n, leaf_bytes, nodes)
+    blob = data.tobytes()
+    assert nodes.cpu().numpy().tobytes() == tree_nodes([blob[i * leaf_bytes:(i + 1) * leaf_bytes] for i in range(n)])
+
+
+@pytest.mark.parametrize("per_sm", [12, 16, 32])  # the lines of the leaves and of the levels
+@pytest.mark.parametrize("leaf_bytes", [137, 200])
+def test_merkle_trees_around_the_lines(cuda_lib, per_sm, leaf_bytes):
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for n in (per_sm * sms, per_sm * sms + 1):
+        data = np.random.default_rng(n).integers(0, 256, size=n * leaf_bytes, dtype=np.uint8)
+        nodes = torch.empty(32 * cuda_lib.merkle_node_count(n), dtype=torch.uint8, device="cuda")
+        cuda_lib.merkle_sha3_256_levels(torch.from_numpy(data).cuda(), n, leaf_bytes, nodes)
+        blob = data.tobytes()
+        want_nodes = tree_nodes([blob[i * leaf_bytes:(i + 1) * leaf_bytes] for i in range(n)])
+        assert nodes.cpu().numpy().tobytes() == want_nodes
