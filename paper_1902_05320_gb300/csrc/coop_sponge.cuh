@@ -51,6 +51,58 @@ __device__ __forceinline__ void pad_raw(const RawWord &r, uint32_t o, int64_t le
     if (end) hi ^= 0x80000000u;
 }
 
+// The part of a sponge whose next block is a full one too: `count` times, XORs the
+// halves in e into the state and permutes, while the next block's words arrive and
+// become the new e.  `next`: the first byte of the block after the one in e.  Nothing
+// is padded here, and a thread's two addresses move on by a block each time
+// (rate % 4 == 0).
+__device__ __forceinline__ void coop_full_blocks(const Coop &c, uint32_t (&a)[2], uint32_t (&e)[2], uintptr_t next,
+                                                 uint32_t rate, uint64_t count) {
+    const int nwords = int(rate / 8);
+    const bool have0 = c.on && c.lane(0) < nwords, have1 = c.on && c.lane(1) < nwords;
+    const uint32_t *q0 = reinterpret_cast<const uint32_t *>((next + 8u * uint32_t(c.lane(0))) & ~uintptr_t(3));
+    const uint32_t *q1 = reinterpret_cast<const uint32_t *>((next + 8u * uint32_t(c.lane(1))) & ~uintptr_t(3));
+    const uint32_t sh = 8 * uint32_t(next & 3), step = rate / 4;
+    RawWord r0{0, 0, 0}, r1{0, 0, 0};
+    for (; count; --count) {
+        a[0] ^= e[0];
+        a[1] ^= e[1];
+        if (have0) {
+            r0.w0 = __ldg(q0);
+            r0.w1 = __ldg(q0 + 1);
+            if (sh) r0.w2 = __ldg(q0 + 2);
+        }
+        if (have1) {
+            r1.w0 = __ldg(q1);
+            r1.w1 = __ldg(q1 + 1);
+            if (sh) r1.w2 = __ldg(q1 + 2);
+        }
+        q0 += step;
+        q1 += step;
+        c.permute(a, [&] {
+            e[0] = c.half(__funnelshift_r(r0.w0, r0.w1, sh), __funnelshift_r(r0.w1, r0.w2, sh));
+            e[1] = c.half(__funnelshift_r(r1.w0, r1.w1, sh), __funnelshift_r(r1.w1, r1.w2, sh));
+        });
+    }
+}
+
+// Writes bytes [0, take) of the state's rate part to dst.  Every thread of the warp
+// calls it.
+__device__ __forceinline__ void coop_squeeze(const Coop &c, const uint32_t (&a)[2], uint8_t *dst, uint32_t take) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const uint32_t w = c.unhalf(a[s]);
+        const uint32_t at = 8u * uint32_t(c.lane(s)) + 4u * uint32_t(c.h);
+        if (c.on && at < take) {
+            uint8_t *q = dst + at;
+            const uint32_t nb = take - at < 4 ? take - at : 4;
+            if (nb == 4 && (reinterpret_cast<uintptr_t>(q) & 3) == 0) *reinterpret_cast<uint32_t *>(q) = w;
+            else
+                for (uint32_t b = 0; b < nb; ++b) q[b] = uint8_t(w >> (8 * b));
+        }
+    }
+}
+
 // One sponge: the message of len bytes at p (PREFIX >= 0: that byte comes before
 // it), dlen output bytes to dst.  Every thread of the warp calls it with the same
 // arguments.  ONLY: the kernel hashes nothing else and has one such warp a block;
@@ -114,34 +166,8 @@ __device__ __forceinline__ void coop_sponge(const Coop &c, const uint8_t *p, uin
     convert(0);
     uint64_t i = 0;
     if (nfull > 2) {
-        // Blocks whose successor is a full block too: nothing to pad, and the
-        // thread's two addresses move on by a block each time (rate % 4 == 0).
-        const bool have0 = c.on && c.lane(0) < nwords, have1 = c.on && c.lane(1) < nwords;
-        const uintptr_t first = reinterpret_cast<uintptr_t>(p) + rate - kShift;  // block 1
-        const uint32_t *q0 = reinterpret_cast<const uint32_t *>((first + 8u * uint32_t(c.lane(0))) & ~uintptr_t(3));
-        const uint32_t *q1 = reinterpret_cast<const uint32_t *>((first + 8u * uint32_t(c.lane(1))) & ~uintptr_t(3));
-        const uint32_t sh = 8 * o, step = rate / 4;
-        RawWord r0{0, 0, 0}, r1{0, 0, 0};
-        for (; i + 1 < nfull; ++i) {
-            a[0] ^= e[0];
-            a[1] ^= e[1];
-            if (have0) {
-                r0.w0 = __ldg(q0);
-                r0.w1 = __ldg(q0 + 1);
-                if (sh) r0.w2 = __ldg(q0 + 2);
-            }
-            if (have1) {
-                r1.w0 = __ldg(q1);
-                r1.w1 = __ldg(q1 + 1);
-                if (sh) r1.w2 = __ldg(q1 + 2);
-            }
-            q0 += step;
-            q1 += step;
-            c.permute(a, [&] {
-                e[0] = c.half(__funnelshift_r(r0.w0, r0.w1, sh), __funnelshift_r(r0.w1, r0.w2, sh));
-                e[1] = c.half(__funnelshift_r(r1.w0, r1.w1, sh), __funnelshift_r(r1.w1, r1.w2, sh));
-            });
-        }
+        coop_full_blocks(c, a, e, reinterpret_cast<uintptr_t>(p) + rate - kShift, rate, nfull - 1);
+        i = nfull - 1;
     }
     for (; i < total; ++i) {
         a[0] ^= e[0];
@@ -155,19 +181,7 @@ __device__ __forceinline__ void coop_sponge(const Coop &c, const uint8_t *p, uin
         });
         if (i >= nfull) {  // output block i - nfull
             const uint32_t base = uint32_t(i - nfull) * rate;
-            const uint32_t take = dlen - base < rate ? dlen - base : rate;
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                const uint32_t w = c.unhalf(a[s]);
-                const uint32_t at = 8u * uint32_t(c.lane(s)) + 4u * uint32_t(c.h);
-                if (c.on && at < take) {
-                    uint8_t *q = dst + base + at;
-                    const uint32_t nb = take - at < 4 ? take - at : 4;
-                    if (nb == 4 && (reinterpret_cast<uintptr_t>(q) & 3) == 0) *reinterpret_cast<uint32_t *>(q) = w;
-                    else
-                        for (uint32_t b = 0; b < nb; ++b) q[b] = uint8_t(w >> (8 * b));
-                }
-            }
+            coop_squeeze(c, a, dst + base, dlen - base < rate ? dlen - base : rate);
         }
     }
 }

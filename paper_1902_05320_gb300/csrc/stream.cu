@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <climits>
 
+#include "coop_sponge.cuh"
 #include "keccak_core.cuh"
 #include "runtime.cuh"
 #include "sponge.cuh"
@@ -117,6 +118,8 @@ __device__ __forceinline__ void pad_open_block(uint32_t (&A)[25], uint32_t (&B)[
 
 __global__ void __launch_bounds__(kThreads) k_stream_init(uint8_t *states, const uint8_t *variants, uint64_t n,
                                                           unsigned int *status) {
+    launch_next();
+    launch_wait();
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += step) {
         uint8_t *st = states + i * kStateBytes;
@@ -141,6 +144,8 @@ __global__ void __launch_bounds__(kThreads, 3)
                   const uint32_t *__restrict__ out_lens, const uint64_t *__restrict__ out_off,
                   uint8_t *__restrict__ digests, uint64_t n, unsigned int *status) {
     const uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    launch_next();
+    launch_wait();
     if (i >= n) return;
     uint8_t *st = states + i * kStateBytes;
     uint32_t *pending_field = reinterpret_cast<uint32_t *>(st + kNbufOff);
@@ -251,6 +256,151 @@ __global__ void __launch_bounds__(kThreads, 3)
     if (INIT || lens[i]) store_lanes(st, A, B);
 }
 
+// The same step for few messages: one warp per message (coop.cuh), which takes a
+// third of the time for a piece's chain of permutations, and in the final step sums
+// the output sizes before its message for the digest's place.  The piece is seen
+// as bytes [pending, pending + len) of a run of blocks that starts `pending` bytes
+// before it, so its head, whole blocks, tail and padding are one loop.  msgs may be
+// null in a final step: no piece.
+template <bool INIT, bool FINAL>
+__global__ void __launch_bounds__(32)
+    k_stream_step_coop(uint8_t *states, const uint8_t *__restrict__ init_variants, const uint8_t *__restrict__ msgs,
+                       const uint64_t *__restrict__ offsets, const uint64_t *__restrict__ lens,
+                       const uint32_t *__restrict__ out_lens, uint8_t *__restrict__ digests, unsigned int *status) {
+    __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
+    const Coop c(mem);
+    const uint32_t i = blockIdx.x, lane = threadIdx.x;
+    if (gridDim.x <= kFewBlocks) launch_next();
+    launch_wait();
+    uint8_t *st = states + uint64_t(i) * kStateBytes;
+    uint32_t *pending_field = reinterpret_cast<uint32_t *>(st + kNbufOff);
+    uint64_t *total_field = reinterpret_cast<uint64_t *>(st + kTotalOff);
+    const uint64_t len = msgs ? lens[i] : 0;
+    const int v = INIT ? init_variants[i] : st[kVarOff];
+    const bool done = !INIT && st[kDoneOff];
+    const uint32_t pending = INIT ? 0u : *pending_field;
+    const uint64_t total_in = INIT ? 0u : *total_field;
+    uint32_t dlen = 0;
+    uint64_t before = 0;
+    if constexpr (FINAL) {
+        dlen = out_lens[i];
+#pragma unroll 8
+        for (uint32_t j = lane; j < i; j += 32) before += out_lens[j];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    }
+    uint32_t a[2] = {0, 0};
+    auto store_state = [&] {
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const uint32_t w = c.unhalf(a[s]);
+            if (c.on && c.lane(s) < 25) reinterpret_cast<uint32_t *>(st)[2 * c.lane(s) + c.h] = w;
+        }
+    };
+    const uint32_t bad = v > 5 ? KB_DEV_BAD_VARIANT
+                         : done || (FINAL && v < 4 && dlen != uint32_t(variant_digest(v))) ? KB_DEV_BAD_OUTLEN : 0u;
+    __syncwarp();  // every thread has read the fields
+    if (INIT && lane == 0) {
+        st[kVarOff] = uint8_t(v);
+        st[kDoneOff] = 0;
+    }
+    if (bad) {
+        // Refused: a fresh state is left empty, an older one as it is.  An absorb of
+        // nothing into a finalised state is not an error.
+        if (lane == 0 && (INIT || FINAL || len)) atomicOr(status, bad);
+        if (INIT) {
+            if (lane == 0) {
+                *pending_field = 0;
+                *total_field = 0;
+            }
+            store_state();
+        }
+        return;
+    }
+    if constexpr (!INIT) {
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+            if (c.on && c.lane(s) < 25) {
+                const uint2 w = reinterpret_cast<const uint2 *>(st)[c.lane(s)];
+                a[s] = c.half(w.x, w.y);
+            }
+    }
+    const uint32_t rate = uint32_t(variant_rate(v));
+    const int nwords = int(rate / 8);
+    const uint32_t domain = rt_domain(v);
+    const uint64_t vlen = pending + len;  // the open block's bytes and the piece's
+    const uint64_t nfull = vlen / rate;
+    const uint32_t rem = uint32_t(vlen - nfull * rate);
+    if (lane == 0) {
+        *total_field = total_in + len;
+        if (FINAL) st[kDoneOff] = 1;
+        else *pending_field = rem;
+    }
+    const uintptr_t first = (msgs ? reinterpret_cast<uintptr_t>(msgs + offsets[i]) : uintptr_t(0)) - pending;
+    const uint32_t sh = 8 * uint32_t(first & 3);
+    // Halves of this thread's words of block b: the piece's bytes in it, and the
+    // padding where a final step ends.  Only aligned words that hold a byte of the
+    // piece are read.
+    auto block_halves = [&](uint64_t b, uint32_t (&e)[2]) {
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const int k = c.lane(s);
+            uint32_t lo = 0, hi = 0;
+            if (c.on && k < nwords) {
+                const uint64_t at = b * rate + 8u * uint32_t(k);
+                const int64_t skip = int64_t(pending) - int64_t(at);  // bytes of the word before the piece
+                const uint32_t from = skip <= 0 ? 0u : skip < 8 ? uint32_t(skip) : 8u;
+                const uint32_t to = vlen <= at ? 0u : vlen - at < 8 ? uint32_t(vlen - at) : 8u;
+                if (from < to) {
+                    const uint32_t o = sh / 8;
+                    const uint32_t *q = reinterpret_cast<const uint32_t *>((first + at) & ~uintptr_t(3));
+                    uint32_t w[3];
+#pragma unroll
+                    for (uint32_t j = 0; j < 3; ++j)  // bytes [4j, 4j + 4) from q on; the piece's are [o + from, o + to)
+                        w[j] = 4 * j < o + to && 4 * j + 4 > o + from ? __ldg(q + j) : 0u;
+                    lo = __funnelshift_r(w[0], w[1], sh) & low_bits(8 * int(to)) & ~low_bits(8 * int(from));
+                    hi = __funnelshift_r(w[1], w[2], sh) & low_bits(8 * int(to) - 32) & ~low_bits(8 * int(from) - 32);
+                }
+                if (FINAL && b == nfull) {
+                    if (uint32_t(k) == rem / 8) {
+                        const uint32_t ps = 8 * (rem % 8);
+                        if (ps < 32) lo ^= domain << ps;
+                        else hi ^= domain << (ps - 32);
+                    }
+                    if (k == nwords - 1) hi ^= 0x80000000u;
+                }
+            }
+            e[s] = c.half(lo, hi);
+        }
+    };
+    uint32_t e[2];
+    block_halves(0, e);
+    uint64_t b = 0;
+    if (nfull > 2) {
+        coop_full_blocks(c, a, e, first + rate, rate, nfull - 1);
+        b = nfull - 1;
+    }
+    for (; b < nfull; ++b) {
+        a[0] ^= e[0];
+        a[1] ^= e[1];
+        c.permute(a, [] {});
+        block_halves(b + 1, e);
+    }
+    a[0] ^= e[0];  // the open block: the tail, and the padding of a final step
+    a[1] ^= e[1];
+    if (gridDim.x > kFewBlocks) launch_next();
+    if constexpr (FINAL) {
+        uint8_t *dst = digests + before;
+        const uint32_t nsq = dlen > rate ? (dlen - 1) / rate : 0;
+        for (uint32_t j = 0; j <= nsq; ++j) {
+            c.permute(a, [] {});
+            coop_squeeze(c, a, dst + uint64_t(j) * rate, j < nsq ? rate : dlen - nsq * rate);
+        }
+    } else if (INIT || len) {
+        store_state();
+    }
+}
+
 // One thread per message and as many blocks as that takes (the block
 // scheduler balances the last wave; a grid-stride split would give some
 // threads one message more than others).
@@ -260,13 +410,20 @@ unsigned grid_for(uint64_t n) { return unsigned(std::min<uint64_t>((n + kThreads
 
 int launch_stream_init(uint8_t *states, const uint8_t *variants, uint64_t n, cudaStream_t stream,
                        const DeviceInfo &dev) {
-    k_stream_init<<<grid_for(n), kThreads, 0, stream>>>(states, variants, n, dev.d_status);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(
+        launch_overlapped(k_stream_init, grid_for(n), kThreads, 0, stream, states, variants, n, dev.d_status));
 }
 
 int launch_stream_step(bool init, bool final_, uint8_t *states, const uint8_t *variants, const uint8_t *msgs,
                        const uint64_t *offsets, const uint64_t *lens, const uint32_t *out_lens, uint8_t *digests,
                        uint64_t n, cudaStream_t stream, const DeviceInfo &dev) {
+    if (init && final_) return KB_ERR_INVALID;  // one whole message per state: keccak_batch
+    if (n <= kCoopPerSm * uint64_t(dev.sm_count > 0 ? dev.sm_count : 1))
+        return cuda_status(launch_overlapped(init     ? k_stream_step_coop<true, false>
+                                             : final_ ? k_stream_step_coop<false, true>
+                                                      : k_stream_step_coop<false, false>,
+                                             unsigned(n), 32, 0, stream, states, variants, msgs, offsets, lens,
+                                             out_lens, digests, dev.d_status));
     uint64_t *out_off = nullptr;
     uint64_t *zeros = nullptr;
     if (final_) {
@@ -285,18 +442,11 @@ int launch_stream_step(bool init, bool final_, uint8_t *states, const uint8_t *v
         }
         if ((err = launch_digest_offsets(out_lens, n, out_off, out_off + n, stream)) != KB_OK) return err;
     }
-    const unsigned g = grid_for(n);
-    if (init && final_) return KB_ERR_INVALID;  // one whole message per state: keccak_batch
-    if (init)
-        k_stream_step<true, false><<<g, kThreads, 0, stream>>>(states, variants, msgs, offsets, lens, out_lens,
-                                                               out_off, digests, n, dev.d_status);
-    else if (final_)
-        k_stream_step<false, true><<<g, kThreads, 0, stream>>>(states, variants, msgs, offsets, lens, out_lens,
-                                                               out_off, digests, n, dev.d_status);
-    else
-        k_stream_step<false, false><<<g, kThreads, 0, stream>>>(states, variants, msgs, offsets, lens, out_lens,
-                                                                out_off, digests, n, dev.d_status);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_overlapped(init     ? k_stream_step<true, false>
+                                         : final_ ? k_stream_step<false, true>
+                                                  : k_stream_step<false, false>,
+                                         grid_for(n), kThreads, 0, stream, states, variants, msgs, offsets, lens,
+                                         out_lens, out_off, digests, n, dev.d_status));
 }
 
 int launch_stream_absorb(uint8_t *states, const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens,

@@ -199,3 +199,81 @@ def test_merkle_trees_around_the_lines(cuda_lib, per_sm, leaf_bytes):
         blob = data.tobytes()
         want_nodes = tree_nodes([blob[i * leaf_bytes:(i + 1) * leaf_bytes] for i in range(n)])
         assert nodes.cpu().numpy().tobytes() == want_nodes
+
+
+@pytest.mark.parametrize("fused", [False, True])
+@pytest.mark.parametrize("per_sm,more", [(0, 1), (3, 7), (12, 0), (12, 1)])  # the line between warps and threads
+def test_stream_around_the_line(cuda_lib, per_sm, more, fused):
+    """Pieces of 0, 1, a few and many bytes, opening blocks at every offset, through either form of every step."""
+    import torch
+
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + more
+    rng = np.random.default_rng(17 * n + fused)
+    dev = lambda a: torch.from_numpy(a.view({8: np.int64, 4: np.int32, 1: np.uint8}[a.itemsize])).cuda()  # noqa: E731
+    variants = rng.integers(0, 6, size=n).astype(np.uint8)
+    out_lens = np.array([W.DIGEST_BYTES[v] or rng.integers(0, 400) for v in variants], dtype=np.uint32)
+    d_var, d_out = dev(variants), dev(out_lens)
+    states = torch.full((n * cuda_lib.KB_STATE_BYTES,), 0xA5, dtype=torch.uint8, device="cuda")
+    out = torch.full((int(out_lens.sum()) + 16,), 0xEE, dtype=torch.uint8, device="cuda")
+    messages = [b""] * n
+    cuda_lib.keccak_last_error()
+    steps = 5
+    for step in range(steps):
+        lens = np.where(rng.random(n) < 0.3, rng.integers(0, 9, size=n), rng.integers(0, 900, size=n)).astype(np.uint64)
+        gaps = rng.integers(0, 4, size=n).astype(np.uint64)
+        ends = np.cumsum(lens + gaps, dtype=np.uint64)
+        data = rng.integers(0, 256, size=int(ends[-1]) + 1, dtype=np.uint8)
+        blob = data.tobytes()
+        messages = [m + blob[int(e - k):int(e)] for m, e, k in zip(messages, ends, lens)]
+        args = (dev(data), dev(ends - lens), dev(lens))
+        if step == 0 and fused:
+            cuda_lib.keccak_stream_init_absorb(states, d_var, *args, n)
+        elif step == steps - 1 and fused:
+            cuda_lib.keccak_stream_absorb_final(states, *args, d_out, out, n)
+        else:
+            if step == 0:
+                cuda_lib.keccak_stream_init(states, d_var, n)
+            cuda_lib.keccak_stream_absorb(states, *args, n)
+        torch.cuda.synchronize()
+    if not fused:
+        cuda_lib.keccak_stream_final(states, d_out, out, n)
+    assert cuda_lib.keccak_last_error() == 0
+    got = out.cpu().numpy()
+    assert (got[int(out_lens.sum()):] == 0xEE).all()
+    assert got[:int(out_lens.sum())].tobytes() == b"".join(want(int(v), m, int(d))
+                                                           for v, m, d in zip(variants, messages, out_lens))
+
+
+def test_stream_refusals_in_both_forms(cuda_lib):
+    """An unknown function, a wrong digest size and a finalised state: the same status bits and untouched outputs
+    from the warp form and the thread form."""
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    seen = []
+    for n in (40, 12 * sms + 40):
+        variants = torch.ones(n, dtype=torch.uint8, device="cuda")
+        variants[5] = 9
+        states = torch.zeros(n * cuda_lib.KB_STATE_BYTES, dtype=torch.uint8, device="cuda")
+        data = torch.arange(100 * n, device="cuda").to(torch.uint8)
+        offsets = torch.arange(n, device="cuda") * 100
+        lens = torch.full((n,), 100, dtype=torch.int64, device="cuda")
+        out_lens = torch.full((n,), 32, dtype=torch.int32, device="cuda")
+        out_lens[7] = 31
+        out = torch.full((32 * n,), 0xEE, dtype=torch.uint8, device="cuda")
+        errs = []
+        cuda_lib.keccak_last_error()
+        cuda_lib.keccak_stream_init_absorb(states, variants, data, offsets, lens, n)
+        errs.append(cuda_lib.keccak_last_error())
+        cuda_lib.keccak_stream_absorb_final(states, data, offsets, lens, out_lens, out, n)
+        errs.append(cuda_lib.keccak_last_error())
+        mine = 32 * 40 - 1  # the outputs of the first 40 messages, one of them 31 bytes
+        first = out.cpu().numpy()[:mine].copy()
+        cuda_lib.keccak_stream_absorb(states, data, offsets, lens, n)  # finalised states refuse more
+        errs.append(cuda_lib.keccak_last_error())
+        cuda_lib.keccak_stream_absorb(states, data, offsets, torch.zeros_like(lens), n)
+        errs.append(cuda_lib.keccak_last_error())
+        cuda_lib.keccak_stream_final(states, out_lens, out, n)
+        errs.append(cuda_lib.keccak_last_error())
+        seen.append((errs, first.tobytes(), out.cpu().numpy()[:mine].tobytes()))
+    assert seen[0] == seen[1] and seen[0][0][0] == cuda_lib.KB_DEV_BAD_VARIANT
