@@ -111,7 +111,6 @@ __device__ __forceinline__ void coop_squeeze(const Coop &c, const uint32_t (&a)[
 // kernel's still stand and would crowd some SMs, where such warps slow one another
 // (1824 leaves of 1000 bytes a call: 63 to 96 us from run to run set up at once,
 // 57.5 late; 200 ragged messages 14.4 at once, 16.8 late).
-constexpr uint32_t kFewBlocks = 600;  // four per SM
 template <int PREFIX = -1, bool ONLY = false>
 __device__ __forceinline__ void coop_sponge(const Coop &c, const uint8_t *p, uint64_t len, int variant, uint8_t *dst,
                                             uint32_t dlen) {

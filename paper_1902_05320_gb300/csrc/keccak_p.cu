@@ -10,6 +10,7 @@
 // lanes serves all widths and all round indices.
 #include <cuda_runtime.h>
 
+#include "coop.cuh"
 #include "keccak_core.cuh"
 #include "runtime.cuh"
 
@@ -115,6 +116,8 @@ __device__ __forceinline__ void run_tiles(uint64_t *states, uint64_t n, uint2 *s
             asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sdst + 8 * j), "l"(src + j) : "memory");
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
+    launch_next();
+    launch_wait();
     if (tile >= ntiles) return;
     load(sbase, tile);
     for (uint32_t b = 0; tile < ntiles; tile += nwarps, b ^= 1u) {
@@ -216,6 +219,8 @@ __global__ void __launch_bounds__(kThreads) k_keccak_p_1600(uint64_t *states, in
             for (int k = 0; k < 25; ++k) s[k] = make_uint2(L[k], H[k]);
         });
     } else {
+        launch_next();
+        launch_wait();
         const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
         for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += step) {
             uint2 *s = reinterpret_cast<uint2 *>(states + 25 * i);
@@ -233,6 +238,36 @@ __global__ void __launch_bounds__(kThreads) k_keccak_p_1600(uint64_t *states, in
     }
 }
 
+// Few states of width 64 and rounds within Keccak-f[1600]'s 24: a warp each
+// (coop.cuh), a third of the time of one thread's chain of rounds.
+__global__ void __launch_bounds__(32) k_keccak_p_1600_coop(uint64_t *states, int first_ir, int nr) {
+    __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
+    const Coop c(mem);
+    if (gridDim.x <= kFewBlocks) launch_next();
+    launch_wait();
+    uint2 *st = reinterpret_cast<uint2 *>(states + 25 * uint64_t(blockIdx.x));
+    uint32_t a[2] = {0, 0};
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+        if (c.on && c.lane(s) < 25) {
+            const uint2 w = st[c.lane(s)];
+            a[s] = c.half(w.x, w.y);
+        }
+    int r = first_ir;
+    const int end = first_ir + nr;
+#pragma unroll 1
+    for (; r + 2 <= end; r += 2) {
+        c.round<0>(a, r);
+        c.round<1>(a, r + 1);
+    }
+    if (r < end) c.round<0>(a, r);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const uint32_t w = c.unhalf(a[s]);
+        if (c.on && c.lane(s) < 25) reinterpret_cast<uint32_t *>(st)[2 * c.lane(s) + c.h] = w;
+    }
+}
+
 // Launches a tiled kernel with its two tile buffers (above the 48 KB a block
 // gets without opting in).
 template <class K>
@@ -241,8 +276,7 @@ int launch_tiled(K kernel, uint64_t *states, int first_ir, int nr, uint64_t n, c
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTileSmem)) != cudaSuccess)
         return cuda_status(cudaGetLastError());
     const uint64_t g = persistent_grid(reinterpret_cast<const void *>(kernel), kThreads, kTileSmem, n, dev);
-    kernel<<<unsigned(g), kThreads, kTileSmem, stream>>>(states, first_ir, nr, n);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_overlapped(kernel, unsigned(g), kThreads, kTileSmem, stream, states, first_ir, nr, n));
 }
 
 template <int W>
@@ -266,14 +300,17 @@ int launch_keccak_p(uint64_t *states, int b, int nr, uint64_t n, cudaStream_t st
         case 4: return launch_small<16>(states, first_ir, nr, n, stream, dev);
         case 5: return launch_small<32>(states, first_ir, nr, n, stream, dev);
         default: {
+            if (first_ir >= 0 && n <= kCoopPerSm * uint64_t(dev.sm_count > 0 ? dev.sm_count : 1))
+                return cuda_status(
+                    launch_overlapped(k_keccak_p_1600_coop, unsigned(n), 32, 0, stream, states, first_ir, nr));
             // Staged through shared memory below 16 rounds (measured on 2^24
             // states: 12 rounds 2.53 ms read directly, 2.15 ms staged; 24
             // rounds 3.84 ms directly, 4.02 ms staged).
             if (nr < 16) return launch_tiled(k_keccak_p_1600<true>, states, first_ir, nr, n, stream, dev);
             const uint64_t g =
                 persistent_grid(reinterpret_cast<const void *>(&k_keccak_p_1600<false>), kThreads, 0, n, dev);
-            k_keccak_p_1600<false><<<unsigned(g), kThreads, 0, stream>>>(states, first_ir, nr, n);
-            return cuda_status(cudaGetLastError());
+            return cuda_status(
+                launch_overlapped(k_keccak_p_1600<false>, unsigned(g), kThreads, 0, stream, states, first_ir, nr, n));
         }
     }
 }

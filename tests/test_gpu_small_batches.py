@@ -277,3 +277,25 @@ def test_stream_refusals_in_both_forms(cuda_lib):
         errs.append(cuda_lib.keccak_last_error())
         seen.append((errs, first.tobytes(), out.cpu().numpy()[:mine].tobytes()))
     assert seen[0] == seen[1] and seen[0][0][0] == cuda_lib.KB_DEV_BAD_VARIANT
+
+
+@pytest.mark.parametrize("nr", [1, 2, 11, 12, 24, 25])
+@pytest.mark.parametrize("per_sm,more", [(0, 1), (0, 5), (12, 0), (12, 1)])
+def test_keccak_p_around_the_line(cuda_lib, per_sm, more, nr):
+    """Few states (a warp each) against many (a thread each), and 24 rounds against hashlib."""
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = per_sm * sms + more
+    states = np.random.default_rng(n + nr).integers(0, 2**63, size=(n, 25), dtype=np.int64)
+    # Row 0 holds the padded one-block message of SHA3-256("abc").
+    states[0] = 0
+    states[0].view(np.uint8)[:4] = np.frombuffer(b"abc\x06", np.uint8)
+    states[0].view(np.uint8)[135] = 0x80
+    few = torch.from_numpy(states).cuda()
+    cuda_lib.keccak_p_batch(few, 1600, nr, n)
+    many = torch.from_numpy(np.tile(states, (12 * sms // n + 2, 1))).cuda()
+    cuda_lib.keccak_p_batch(many, 1600, nr, many.shape[0])
+    assert torch.equal(few, many[:n])
+    if nr == 24:
+        assert few[0].cpu().numpy().tobytes()[:32] == hashlib.sha3_256(b"abc").digest()
