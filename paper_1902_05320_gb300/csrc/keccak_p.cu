@@ -116,7 +116,6 @@ __device__ __forceinline__ void run_tiles(uint64_t *states, uint64_t n, uint2 *s
             asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sdst + 8 * j), "l"(src + j) : "memory");
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    launch_next();
     launch_wait();
     if (tile >= ntiles) return;
     load(sbase, tile);
@@ -219,7 +218,6 @@ __global__ void __launch_bounds__(kThreads) k_keccak_p_1600(uint64_t *states, in
             for (int k = 0; k < 25; ++k) s[k] = make_uint2(L[k], H[k]);
         });
     } else {
-        launch_next();
         launch_wait();
         const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
         for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += step) {

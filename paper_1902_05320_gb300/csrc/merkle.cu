@@ -93,7 +93,6 @@ __device__ __forceinline__ void leaf_state_a8(const uint8_t *p, uint64_t leaf_by
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_merkle_leaves_a8(const uint8_t *__restrict__ buf, uint64_t n_leaves, uint64_t leaf_bytes,
                        uint8_t *__restrict__ out) {
-    launch_next();
     launch_wait();
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n_leaves; i += step) {
@@ -167,7 +166,6 @@ __device__ __forceinline__ void absorb_leaf_block_any(uint32_t (&A)[25], uint32_
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_merkle_leaves_any(const uint8_t *__restrict__ buf, uint64_t n_leaves, uint64_t leaf_bytes,
                         uint8_t *__restrict__ out) {
-    launch_next();
     launch_wait();
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
     const uint64_t vlen = leaf_bytes + 1;
@@ -224,7 +222,6 @@ __device__ __forceinline__ void merkle_parent(const uint8_t *in, uint64_t count,
 // One level, one thread per parent.
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_merkle_level(const uint8_t *in, uint64_t count, uint8_t *out) {
-    launch_next();
     launch_wait();
     const uint64_t parents = count / 2 + (count & 1);
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;

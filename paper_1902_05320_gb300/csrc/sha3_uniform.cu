@@ -39,7 +39,6 @@ __global__ void __launch_bounds__(kThreads, LEN == -1 ? kMinBlocks : kOneBlockMi
     k_sha3_uniform(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len_rt,
                    uint8_t *__restrict__ out, uint32_t out_len, uint64_t n) {
     using P = Variant<V>;
-    launch_next();
     launch_wait();
     const uint64_t len = LEN >= 0 ? uint64_t(LEN) : len_rt;
     const uint32_t dlen = P::digest ? uint32_t(P::digest) : out_len;
@@ -121,7 +120,6 @@ __global__ void __launch_bounds__(kThreads, kOneBlockMinBlocks)
         bulk_copy_g2s(buf[b], msgs + first * 64, bytes, &bar[b]);
         ++uses[b];
     };
-    launch_next();
     if (threadIdx.x == 0) {
         mbar_init(&bar[0], 1);
         mbar_init(&bar[1], 1);

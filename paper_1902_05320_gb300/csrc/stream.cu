@@ -118,7 +118,6 @@ __device__ __forceinline__ void pad_open_block(uint32_t (&A)[25], uint32_t (&B)[
 
 __global__ void __launch_bounds__(kThreads) k_stream_init(uint8_t *states, const uint8_t *variants, uint64_t n,
                                                           unsigned int *status) {
-    launch_next();
     launch_wait();
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += step) {
@@ -144,7 +143,6 @@ __global__ void __launch_bounds__(kThreads, 3)
                   const uint32_t *__restrict__ out_lens, const uint64_t *__restrict__ out_off,
                   uint8_t *__restrict__ digests, uint64_t n, unsigned int *status) {
     const uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    launch_next();
     launch_wait();
     if (i >= n) return;
     uint8_t *st = states + i * kStateBytes;
