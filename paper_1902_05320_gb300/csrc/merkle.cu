@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n_leaves; i += step) {
         uint32_t A[25], B[25];
         leaf_state_a8(buf + i * leaf_bytes, leaf_bytes, A, B);
-        squeeze<kRate, PlainRep>(A, B, out + 32 * i, 32);
+        squeeze<kRate, PlainRep, 32>(A, B, out + 32 * i, 32);
     }
 }
 
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
             absorb_leaf_block_any(A, B, p, b, nfull, rem);
             PlainRep::permute<false>(A, B);
         }
-        squeeze<kRate, PlainRep>(A, B, out + 32 * i, 32);
+        squeeze<kRate, PlainRep, 32>(A, B, out + 32 * i, 32);
     }
 }
 
@@ -216,7 +216,7 @@ __device__ __forceinline__ void merkle_parent(const uint8_t *in, uint64_t count,
     PlainRep::set_word(A[8], B[8], vlo, vhi);
     B[kRate / 8 - 1] ^= 0x80000000u;
     PlainRep::permute<true>(A, B);
-    squeeze<kRate, PlainRep>(A, B, out + 32 * j, 32);
+    squeeze<kRate, PlainRep, 32>(A, B, out + 32 * j, 32);
 }
 
 // One level, one thread per parent.

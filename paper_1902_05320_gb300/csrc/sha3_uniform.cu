@@ -24,22 +24,24 @@
 namespace kb {
 namespace {
 
-// Blocks per SM the one-block kernels are compiled for.  With rotations on the
-// multiply pipe more warps are wanted to keep both pipes fed: 2^24 64-byte
-// messages take 3.31 ms at a budget of 4 (5 blocks fit), 3.29 at 5, 3.24 at 6.
-// The multi-block kernels stay at kMinBlocks (2^18 messages of 1023 bytes
-// 820 us at 4; 837 at 5 and 851 at 6, which spill).
-constexpr int kOneBlockMinBlocks = 6;
+// Blocks per SM a kernel is compiled for.  With rotations on the multiply pipe more
+// warps are wanted to keep both pipes fed: 2^24 64-byte messages take 3.31 ms at a
+// budget of 4 (5 blocks fit), 3.29 at 5, 3.24 at 6; 2^22 messages of 32 bytes 855 us
+// at 4, 848 at 5, 840 at 6 (loop of two rounds; of four: 915, 901, 893).  The
+// multi-block kernel stays at kMinBlocks (2^18 messages of 1023 bytes 820 us; 837 at
+// 5, 851 at 6, spilling).
+constexpr int min_blocks(int len) { return len == -1 ? kMinBlocks : 6; }
 
 // LEN >= 0: compile-time message length; -1: runtime; -2: runtime, below the
 // rate, with at most one block of output.  A8: base and stride are multiples
 // of 8 (16 when LEN == 64).
 template <int V, int LEN, bool A8, class Rep>
-__global__ void __launch_bounds__(kThreads, LEN == -1 ? kMinBlocks : kOneBlockMinBlocks)
+__global__ void __launch_bounds__(kThreads, min_blocks(LEN))
     k_sha3_uniform(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len_rt,
                    uint8_t *__restrict__ out, uint32_t out_len, uint64_t n) {
     using P = Variant<V>;
     launch_wait();
+    constexpr int kOut = P::digest ? P::digest : P::rate;
     const uint64_t len = LEN >= 0 ? uint64_t(LEN) : len_rt;
     const uint32_t dlen = P::digest ? uint32_t(P::digest) : out_len;
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
@@ -69,7 +71,7 @@ __global__ void __launch_bounds__(kThreads, LEN == -1 ? kMinBlocks : kOneBlockMi
                 if (i > 0) squeeze<P::rate, Rep>(A, B, dst + uint64_t(i - 1) * P::rate, P::rate);
                 Rep::template permute<true>(A, B);
             }
-            squeeze<P::rate, Rep>(A, B, dst + uint64_t(nsq) * P::rate, dlen - nsq * P::rate);
+            squeeze<P::rate, Rep, kOut>(A, B, dst + uint64_t(nsq) * P::rate, dlen - nsq * P::rate);
         } else if constexpr (LEN == -2) {
             // A runtime length below the rate and at most one output block:
             // the message is the padded last block and one permutation,
@@ -77,11 +79,11 @@ __global__ void __launch_bounds__(kThreads, LEN == -1 ? kMinBlocks : kOneBlockMi
             uint32_t A[25], B[25];
 #pragma unroll
             for (int i = 0; i < 25; ++i) A[i] = B[i] = 0;
-            absorb_last<P::rate, P::domain, A8, Rep>(A, B, p, uint32_t(len));
-            Rep::template permute<true>(A, B);
-            squeeze<P::rate, Rep>(A, B, dst, dlen);
+            absorb_last_same<P::rate, P::domain, A8, Rep>(A, B, p, uint32_t(len));
+            keccak_f1600_plain<true, 23, 2>(A, B);
+            squeeze<P::rate, Rep, kOut>(A, B, dst, dlen);
         } else {
-            sponge<P::rate, P::domain, A8, Rep>(p, len, dst, dlen);
+            sponge<P::rate, P::domain, A8, Rep, true>(p, len, dst, dlen);
         }
     }
 }
@@ -101,11 +103,12 @@ constexpr uint32_t kTileBytes = kThreads * 64;  // 8 KiB
 constexpr uint64_t kWaitNs = 1000000000ull;     // 1 s
 
 template <int V, class Rep>
-__global__ void __launch_bounds__(kThreads, kOneBlockMinBlocks)
+__global__ void __launch_bounds__(kThreads, min_blocks(64))
     k_sha3_uniform64_tma(const uint8_t *__restrict__ msgs, uint8_t *__restrict__ out, uint32_t out_len, uint64_t n,
                          unsigned int *status) {
     using P = Variant<V>;
     static_assert(64 < P::rate, "a 64-byte message is one block for every variant");
+    constexpr int kOut = P::digest ? P::digest : P::rate;
     __shared__ __align__(128) uint8_t buf[2][kTileBytes];
     __shared__ __align__(8) uint64_t bar[2];
     const uint64_t ntiles = (n + kThreads - 1) / kThreads;
@@ -177,7 +180,7 @@ __global__ void __launch_bounds__(kThreads, kOneBlockMinBlocks)
                 if (i > 0) squeeze<P::rate, Rep>(A, B, dst + uint64_t(i - 1) * P::rate, P::rate);
                 Rep::template permute<true>(A, B);
             }
-            squeeze<P::rate, Rep>(A, B, dst + uint64_t(nsq) * P::rate, dlen - nsq * P::rate);
+            squeeze<P::rate, Rep, kOut>(A, B, dst + uint64_t(nsq) * P::rate, dlen - nsq * P::rate);
         }
     }
 }

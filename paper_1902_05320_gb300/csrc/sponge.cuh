@@ -76,9 +76,54 @@ __device__ __forceinline__ void absorb_full(uint32_t (&A)[25], uint32_t (&B)[25]
     }
 }
 
+// Writes bytes [0, nbytes) of the rate part of the state (0 < nbytes <= 168)
+// to dst at any alignment.  Output byte b lands in the aligned 32-bit word
+// (b + o) / 4, o = dst mod 4, so aligned word j is a funnel shift of state
+// words j-1 and j.  Words wholly inside the output take one 32-bit store;
+// the partial words at either end are written byte by byte, so no byte
+// outside [dst, dst + nbytes) is touched.
+template <class Rep>
+__device__ __forceinline__ void squeeze_rt(const uint32_t (&A)[25], const uint32_t (&B)[25], uint8_t *dst,
+                                           uint32_t nbytes) {
+    const uintptr_t d = reinterpret_cast<uintptr_t>(dst);
+    const uint32_t o = uint32_t(d & 3);
+    uint32_t *al = reinterpret_cast<uint32_t *>(d & ~uintptr_t(3));
+    const uint32_t sh = 8 * o;
+    const uint32_t end = nbytes + o;    // output end, in bytes from al
+    const uint32_t jl = (end - 1) >> 2;  // last aligned word touched
+    const uint32_t jfull_lo = o ? 1u : 0u;
+    const uint32_t jfull_hi = (end & 3) ? jl : jl + 1;  // full words: [jfull_lo, jfull_hi)
+    uint32_t prev = 0, first = 0, last = 0;
+#pragma unroll
+    for (int j = 0; j <= 42; ++j) {
+        if (uint32_t(j) > jl) break;
+        uint32_t s = 0;
+        if (j < 42) {
+            uint32_t lo, hi;
+            Rep::get_word(A[j / 2], B[j / 2], lo, hi);
+            s = (j & 1) ? hi : lo;
+        }
+        const uint32_t v = __funnelshift_l(prev, s, sh);
+        prev = s;
+        if (uint32_t(j) >= jfull_lo && uint32_t(j) < jfull_hi) al[j] = v;
+        if (j == 0) first = v;
+        if (uint32_t(j) == jl) last = v;
+    }
+    uint8_t *b = reinterpret_cast<uint8_t *>(al);
+    if (o) {  // head: bytes o .. min(4, end) - 1 of word 0
+        const uint32_t hend = end < 4 ? end : 4u;
+        for (uint32_t i = o; i < hend; ++i) b[i] = uint8_t(first >> (8 * i));
+    }
+    if ((end & 3) && !(jl == 0 && o)) {  // tail: bytes 0 .. (end & 3) - 1 of word jl
+        for (uint32_t i = 0; i < (end & 3); ++i) b[4 * jl + i] = uint8_t(last >> (8 * i));
+    }
+}
+
 // Writes bytes [0, nbytes) of the rate part of the state to dst
-// (nbytes <= RATE), with the widest stores dst's alignment allows.
-template <int RATE, class Rep>
+// (nbytes <= RATE), with the widest stores dst's alignment allows.  (An output at no
+// alignment used to go out byte by byte: 13.8 M SHAKE128 outputs of 499 bytes took
+// 48 ms, where the permutations take 9.)  nbytes <= MAXB.
+template <int RATE, class Rep, int MAXB = RATE>
 __device__ __forceinline__ void squeeze(const uint32_t (&A)[25], const uint32_t (&B)[25], uint8_t *dst,
                                         uint32_t nbytes) {
     const uintptr_t d = reinterpret_cast<uintptr_t>(dst);
@@ -111,9 +156,12 @@ __device__ __forceinline__ void squeeze(const uint32_t (&A)[25], const uint32_t 
                 if (uint32_t(8 * k + 4) < nbytes) *reinterpret_cast<uint32_t *>(dst + 8 * k + 4) = hi;
             }
         }
-    } else {
+    } else if constexpr (MAXB < RATE) {
+        // A fixed digest at an address that is no multiple of 4: byte by byte (the
+        // funnel-shifted words below cost the 64-byte kernel, which has no such
+        // address in earnest, 1%).
 #pragma unroll
-        for (int k = 0; k < RATE / 8; ++k) {
+        for (int k = 0; 8 * k < MAXB; ++k) {
             if (uint32_t(8 * k) < nbytes) {
                 uint32_t lo, hi;
                 Rep::get_word(A[k], B[k], lo, hi);
@@ -122,6 +170,8 @@ __device__ __forceinline__ void squeeze(const uint32_t (&A)[25], const uint32_t 
                 for (uint32_t b = 0; b < nb; ++b) dst[8 * k + b] = uint8_t(w >> (8 * b));
             }
         }
+    } else if (nbytes) {
+        squeeze_rt<Rep>(A, B, dst, nbytes);
     }
 }
 
@@ -207,10 +257,44 @@ __device__ __forceinline__ void absorb_last(uint32_t (&A)[25], uint32_t (&B)[25]
     absorb_last_rt<A8, Rep>(A, B, p, rem, RATE / 8, uint32_t(DOMAIN));
 }
 
-// One complete sponge for a message of len bytes at p, writing dlen output
-// bytes to dst.  The permutation has a single call site, so its code appears
-// once.
+// The same where every thread of the warp has the same rem: a word is taken whole,
+// in part (with the padding behind it) or not at all, by branches that do not
+// diverge, where the form above masks and tests every word of the rate (12
+// instructions a word: 2^22 messages of 10 to 100 bytes 940-957 us, now 840-878).
 template <int RATE, int DOMAIN, bool A8, class Rep>
+__device__ __forceinline__ void absorb_last_same(uint32_t (&A)[25], uint32_t (&B)[25], const uint8_t *p, uint32_t rem) {
+    const uintptr_t start = reinterpret_cast<uintptr_t>(p);
+    const uint32_t *a = reinterpret_cast<const uint32_t *>(A8 ? start : start & ~uintptr_t(3));
+    const uint32_t o = A8 ? 0u : uint32_t(start & 3), sh = 8 * o;
+#pragma unroll
+    for (int k = 0; k < RATE / 8; ++k) {
+        if (uint32_t(8 * k + 8) <= rem) {
+            uint32_t lo, hi;
+            if constexpr (A8) {
+                ld_word_a8(p + 8 * k, lo, hi);
+            } else {
+                const uint32_t w0 = __ldg(a + 2 * k), w1 = __ldg(a + 2 * k + 1);
+                const uint32_t w2 = o ? __ldg(a + 2 * k + 2) : 0u;
+                lo = __funnelshift_r(w0, w1, sh);
+                hi = __funnelshift_r(w1, w2, sh);
+            }
+            Rep::xor_word(A[k], B[k], lo, hi);
+        } else if (uint32_t(8 * k) <= rem) {
+            const uint32_t n = rem - 8 * k;  // 0..7 message bytes, then the domain byte
+            uint32_t lo = 0, hi = 0;
+            if (n) ld_word_any(p + 8 * k, n, lo, hi);
+            if (n < 4) lo ^= uint32_t(DOMAIN) << (8 * n);
+            else hi ^= uint32_t(DOMAIN) << (8 * (n - 4));
+            Rep::xor_word(A[k], B[k], lo, hi);
+        }
+    }
+    Rep::xor_word(A[RATE / 8 - 1], B[RATE / 8 - 1], 0u, 0x80000000u);
+}
+
+// One complete sponge for a message of len bytes at p, writing dlen output
+// bytes to dst.  SAME: len is the same for every thread of the warp.  The permutation has a single call site, so its code appears
+// once.
+template <int RATE, int DOMAIN, bool A8, class Rep, bool SAME = false>
 __device__ __forceinline__ void sponge(const uint8_t *p, uint64_t len, uint8_t *dst, uint32_t dlen) {
     uint32_t A[25], B[25];
 #pragma unroll
@@ -221,54 +305,12 @@ __device__ __forceinline__ void sponge(const uint8_t *p, uint64_t len, uint8_t *
     const uint64_t total = nfull + 1 + nsq;
     for (uint64_t i = 0; i < total; ++i) {
         if (i < nfull) absorb_full<RATE, A8, Rep>(A, B, p + i * RATE);
+        else if (i == nfull && SAME) absorb_last_same<RATE, DOMAIN, A8, Rep>(A, B, p + nfull * RATE, rem);
         else if (i == nfull) absorb_last<RATE, DOMAIN, A8, Rep>(A, B, p + nfull * RATE, rem);
         else squeeze<RATE, Rep>(A, B, dst + (i - nfull - 1) * RATE, RATE);
         Rep::template permute<false>(A, B);
     }
     squeeze<RATE, Rep>(A, B, dst + uint64_t(nsq) * RATE, dlen - nsq * RATE);
-}
-
-// Writes bytes [0, nbytes) of the rate part of the state (0 < nbytes <= 168)
-// to dst at any alignment.  Output byte b lands in the aligned 32-bit word
-// (b + o) / 4, o = dst mod 4, so aligned word j is a funnel shift of state
-// words j-1 and j.  Words wholly inside the output take one 32-bit store;
-// the partial words at either end are written byte by byte, so no byte
-// outside [dst, dst + nbytes) is touched.
-template <class Rep>
-__device__ __forceinline__ void squeeze_rt(const uint32_t (&A)[25], const uint32_t (&B)[25], uint8_t *dst,
-                                           uint32_t nbytes) {
-    const uintptr_t d = reinterpret_cast<uintptr_t>(dst);
-    const uint32_t o = uint32_t(d & 3);
-    uint32_t *al = reinterpret_cast<uint32_t *>(d & ~uintptr_t(3));
-    const uint32_t sh = 8 * o;
-    const uint32_t end = nbytes + o;    // output end, in bytes from al
-    const uint32_t jl = (end - 1) >> 2;  // last aligned word touched
-    const uint32_t jfull_lo = o ? 1u : 0u;
-    const uint32_t jfull_hi = (end & 3) ? jl : jl + 1;  // full words: [jfull_lo, jfull_hi)
-    uint32_t prev = 0, first = 0, last = 0;
-#pragma unroll
-    for (int j = 0; j <= 42; ++j) {
-        if (uint32_t(j) > jl) break;
-        uint32_t s = 0;
-        if (j < 42) {
-            uint32_t lo, hi;
-            Rep::get_word(A[j / 2], B[j / 2], lo, hi);
-            s = (j & 1) ? hi : lo;
-        }
-        const uint32_t v = __funnelshift_l(prev, s, sh);
-        prev = s;
-        if (uint32_t(j) >= jfull_lo && uint32_t(j) < jfull_hi) al[j] = v;
-        if (j == 0) first = v;
-        if (uint32_t(j) == jl) last = v;
-    }
-    uint8_t *b = reinterpret_cast<uint8_t *>(al);
-    if (o) {  // head: bytes o .. min(4, end) - 1 of word 0
-        const uint32_t hend = end < 4 ? end : 4u;
-        for (uint32_t i = o; i < hend; ++i) b[i] = uint8_t(first >> (8 * i));
-    }
-    if ((end & 3) && !(jl == 0 && o)) {  // tail: bytes 0 .. (end & 3) - 1 of word jl
-        for (uint32_t i = 0; i < (end & 3); ++i) b[4 * jl + i] = uint8_t(last >> (8 * i));
-    }
 }
 
 template <bool A8, class Rep>
