@@ -196,10 +196,13 @@ __device__ __forceinline__ uint32_t shl_pair_mul(uint32_t lo, uint32_t hi) {
 // five register reads a word and still pay (335 -> 328), 12 and 13 lose
 // (336), all up to 15 more (339); bit reversals on the otherwise idle XU pipe
 // for the offsets near 32 lose as well (330 -> 334..347).
-template <int N>
+// MUL = false keeps to funnel shifts: for a warp alone on its sub-partition the
+// multiplies' longer chains cost more than the ALU time they save (17,800 messages
+// of 23,907 bytes 966 us against 885).
+template <int N, bool MUL>
 __device__ __forceinline__ void rotl64_round(uint32_t lo, uint32_t hi, uint32_t &nl, uint32_t &nh) {
     constexpr int M = N & 31;
-    if constexpr (M >= 1 && M <= 11) {
+    if constexpr (MUL && M >= 1 && M <= 11) {
         nl = N < 32 ? shl_pair_mul<M>(hi, lo) : shl_pair_mul<M>(lo, hi);
         nh = N < 32 ? shl_pair_mul<M>(lo, hi) : shl_pair_mul<M>(hi, lo);
     } else {
@@ -209,7 +212,7 @@ __device__ __forceinline__ void rotl64_round(uint32_t lo, uint32_t hi, uint32_t 
 
 // theta's column terms for the source lane of (X, Y), then rho; pi is the
 // choice of source: Eq. 6, A'[x,y] = A[(x+3y) mod 5, x].
-template <int X, int Y>
+template <int X, int Y, bool MUL>
 __device__ __forceinline__ void plain_theta_rho_pi(const uint32_t (&L)[25], const uint32_t (&H)[25],
                                                    const uint32_t (&CL)[5], const uint32_t (&CH)[5],
                                                    const uint32_t (&RL)[5], const uint32_t (&RH)[5],
@@ -219,19 +222,19 @@ __device__ __forceinline__ void plain_theta_rho_pi(const uint32_t (&L)[25], cons
     // Eq. 4 with D[x] = C[x-1] ^ rot(C[x+1], 1) (Eq. 3).
     const uint32_t tl = xor3(L[SRC], CL[(SX + 4) % 5], RL[(SX + 1) % 5]);
     const uint32_t th = xor3(H[SRC], CH[(SX + 4) % 5], RH[(SX + 1) % 5]);
-    rotl64_round<rho_offset(SRC)>(tl, th, bl, bh);
+    rotl64_round<rho_offset(SRC), MUL>(tl, th, bl, bh);
 }
 
-template <int Y>
+template <int Y, bool MUL>
 __device__ __forceinline__ void plain_row(const uint32_t (&L)[25], const uint32_t (&H)[25], const uint32_t (&CL)[5],
                                           const uint32_t (&CH)[5], const uint32_t (&RL)[5], const uint32_t (&RH)[5],
                                           uint32_t (&NL)[25], uint32_t (&NH)[25]) {
     uint32_t BL[5], BH[5];
-    plain_theta_rho_pi<0, Y>(L, H, CL, CH, RL, RH, BL[0], BH[0]);
-    plain_theta_rho_pi<1, Y>(L, H, CL, CH, RL, RH, BL[1], BH[1]);
-    plain_theta_rho_pi<2, Y>(L, H, CL, CH, RL, RH, BL[2], BH[2]);
-    plain_theta_rho_pi<3, Y>(L, H, CL, CH, RL, RH, BL[3], BH[3]);
-    plain_theta_rho_pi<4, Y>(L, H, CL, CH, RL, RH, BL[4], BH[4]);
+    plain_theta_rho_pi<0, Y, MUL>(L, H, CL, CH, RL, RH, BL[0], BH[0]);
+    plain_theta_rho_pi<1, Y, MUL>(L, H, CL, CH, RL, RH, BL[1], BH[1]);
+    plain_theta_rho_pi<2, Y, MUL>(L, H, CL, CH, RL, RH, BL[2], BH[2]);
+    plain_theta_rho_pi<3, Y, MUL>(L, H, CL, CH, RL, RH, BL[3], BH[3]);
+    plain_theta_rho_pi<4, Y, MUL>(L, H, CL, CH, RL, RH, BL[4], BH[4]);
 #pragma unroll
     for (int x = 0; x < 5; ++x) {  // Eq. 7
         NL[x + 5 * Y] = chi3(BL[x], BL[(x + 1) % 5], BL[(x + 2) % 5]);
@@ -240,6 +243,7 @@ __device__ __forceinline__ void plain_row(const uint32_t (&L)[25], const uint32_
 }
 
 // One round without iota; the caller XORs the round constant into lane 0.
+template <bool MUL = true>
 __device__ __forceinline__ void plain_round_body(uint32_t (&L)[25], uint32_t (&H)[25], uint32_t (&NL)[25],
                                                  uint32_t (&NH)[25]) {
     uint32_t CL[5], CH[5], RL[5], RH[5];
@@ -249,18 +253,19 @@ __device__ __forceinline__ void plain_round_body(uint32_t (&L)[25], uint32_t (&H
         CH[x] = xor3(xor3(H[x], H[x + 5], H[x + 10]), H[x + 15], H[x + 20]);
     }
 #pragma unroll
-    for (int x = 0; x < 5; ++x) rotl64_round<1>(CL[x], CH[x], RL[x], RH[x]);
-    plain_row<0>(L, H, CL, CH, RL, RH, NL, NH);
-    plain_row<1>(L, H, CL, CH, RL, RH, NL, NH);
-    plain_row<2>(L, H, CL, CH, RL, RH, NL, NH);
-    plain_row<3>(L, H, CL, CH, RL, RH, NL, NH);
-    plain_row<4>(L, H, CL, CH, RL, RH, NL, NH);
+    for (int x = 0; x < 5; ++x) rotl64_round<1, MUL>(CL[x], CH[x], RL[x], RH[x]);
+    plain_row<0, MUL>(L, H, CL, CH, RL, RH, NL, NH);
+    plain_row<1, MUL>(L, H, CL, CH, RL, RH, NL, NH);
+    plain_row<2, MUL>(L, H, CL, CH, RL, RH, NL, NH);
+    plain_row<3, MUL>(L, H, CL, CH, RL, RH, NL, NH);
+    plain_row<4, MUL>(L, H, CL, CH, RL, RH, NL, NH);
 }
 
 // Round i_r with its constant read from the __constant__ table.
+template <bool MUL = true>
 __device__ __forceinline__ void plain_round_rt(uint32_t (&L)[25], uint32_t (&H)[25], int ir) {
     uint32_t NL[25], NH[25];
-    plain_round_body(L, H, NL, NH);
+    plain_round_body<MUL>(L, H, NL, NH);
     NL[0] ^= c_rc.w[2 * ir];  // Eq. 9
     NH[0] += c_rc.w[2 * ir + 1];  // bit 31 alone or nothing, so the sum is the XOR (off the ALU pipe)
 #pragma unroll

@@ -94,14 +94,17 @@ int tuning_set(int key, int64_t value);
 // Launchers (one per translation unit of kernels).
 int launch_uniform(const uint8_t *msgs, uint64_t stride, uint64_t len, int variant, uint32_t out_len,
                    uint8_t *digests, uint64_t n, cudaStream_t stream, const DeviceInfo &dev);
-// Fixed-stride batches below kPairPerSm messages per SM (sha3_small.cu): true when
+// Fixed-stride batches of up to kThinPerSm messages per SM (sha3_small.cu): true when
 // one of its kernels took the batch (*rc is the launch's status).
 //
 // The lines between the forms, in messages per SM, from us a permutation on a
 // GB300 of 152 SMs: thirty threads a message 1.55 at 0.4, 1.80 at 8 and 2.58 at
 // 12; two threads 2.82 up to 64 (one warp per sub-partition) and 4.97 beyond; a
-// thread each 4.47.
-constexpr uint64_t kCoopOnePerSm = 8, kCoopPerSm = 12, kPairPerSm = 64;
+// thread each 4.5 up to 128 (the same).  Up to 256 the kernel that loads the next
+// block ahead (k_sha3_uniform_thin) beats the general one: 23,907 bytes a message,
+// 17,800 messages 754 us against 966, 38,912 1384 against 1535; beyond, with three
+// warps a sub-partition, it does not (1000 bytes: 102 us either way).
+constexpr uint64_t kCoopOnePerSm = 8, kCoopPerSm = 12, kPairPerSm = 64, kThinPerSm = 256;
 bool launch_uniform_small(const uint8_t *msgs, uint64_t stride, uint64_t len, int variant, uint32_t out_len,
                           uint8_t *digests, uint64_t n, cudaStream_t stream, const DeviceInfo &dev, int *rc);
 int launch_ragged(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens, const uint8_t *variants,

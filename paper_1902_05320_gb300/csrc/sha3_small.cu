@@ -33,6 +33,65 @@ __global__ void __launch_bounds__(kThreads)
     pair_sponge<Variant<V>::rate, Variant<V>::domain>(m < n, msgs + m * stride, len, out + m * out_len, out_len);
 }
 
+// A thread per message where that gives a sub-partition one warp or two: few warps
+// do not hide each other's loads, so each thread's next block is loaded into
+// registers before the permutation, which for a lone warp keeps to funnel shifts
+// (keccak_core.cuh).
+template <int V, bool MUL>
+__global__ void __launch_bounds__(kThreads, 2)
+    k_sha3_uniform_thin(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len, uint8_t *__restrict__ out,
+                        uint32_t out_len, uint64_t n) {
+    using P = Variant<V>;
+    constexpr int kWords = P::rate / 4;
+    const uint64_t m = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    launch_wait();
+    if (m >= n) return;
+    const uint8_t *p = msgs + m * stride;
+    const uint32_t dlen = P::digest ? uint32_t(P::digest) : out_len;
+    uint8_t *dst = out + m * dlen;
+    const uint64_t nfull = len / P::rate;
+    const uint32_t nsq = dlen > uint32_t(P::rate) ? (dlen - 1) / P::rate : 0;
+    const uint32_t sh = uint32_t(reinterpret_cast<uintptr_t>(p) & 3) * 8;  // the same for every block (rate % 4 == 0)
+    uint32_t A[25], B[25], w[kWords + 1];
+#pragma unroll
+    for (int k = 0; k < 25; ++k) A[k] = B[k] = 0;
+    auto fetch = [&](uint64_t i) {
+        const uint32_t *a = reinterpret_cast<const uint32_t *>((reinterpret_cast<uintptr_t>(p) & ~uintptr_t(3)) +
+                                                               i * P::rate);
+#pragma unroll
+        for (int k = 0; k < kWords; ++k) w[k] = __ldg(a + k);
+        w[kWords] = sh ? __ldg(a + kWords) : 0u;
+    };
+    if (nfull) fetch(0);
+    for (uint64_t i = 0; i <= nfull + nsq; ++i) {
+        if (i < nfull) {
+#pragma unroll
+            for (int k = 0; k < P::rate / 8; ++k)
+                PlainRep::xor_word(A[k], B[k], __funnelshift_r(w[2 * k], w[2 * k + 1], sh),
+                                   __funnelshift_r(w[2 * k + 1], w[2 * k + 2], sh));
+            if (i + 1 < nfull) fetch(i + 1);
+        } else if (i == nfull) {
+            absorb_last_same<P::rate, P::domain, false, PlainRep>(A, B, p + nfull * P::rate,
+                                                                  uint32_t(len - nfull * P::rate));
+        } else {
+            squeeze<P::rate, PlainRep>(A, B, dst + (i - nfull - 1) * P::rate, P::rate);
+        }
+#pragma unroll 1
+        for (int r = 0; r < 24; r += 4) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) plain_round_rt<MUL>(A, B, r + j);
+        }
+    }
+    squeeze<P::rate, PlainRep>(A, B, dst + uint64_t(nsq) * P::rate, dlen - nsq * P::rate);
+}
+
+template <int V, bool MUL>
+int launch_thin(const uint8_t *msgs, uint64_t stride, uint64_t len, uint32_t out_len, uint8_t *digests, uint64_t n,
+                cudaStream_t stream) {
+    return cuda_status(launch_overlapped(k_sha3_uniform_thin<V, MUL>, unsigned((n + kThreads - 1) / kThreads), kThreads, 0,
+                                         stream, msgs, stride, len, digests, out_len, n));
+}
+
 template <int V>
 int launch_pair(const uint8_t *msgs, uint64_t stride, uint64_t len, uint32_t out_len, uint8_t *digests, uint64_t n,
                 cudaStream_t stream) {
@@ -55,16 +114,23 @@ bool launch_uniform_small(const uint8_t *msgs, uint64_t stride, uint64_t len, in
                                             digests, out_len));
         return true;
     }
-    if (one || n > kPairPerSm * sms) return false;
+    if (one || n > kThinPerSm * sms) return false;
+    const bool pair = n <= kPairPerSm * sms, lone = n <= kThinPerSm / 2 * sms;
+#define KB_FEW(V) \
+    *rc = pair   ? launch_pair<V>(msgs, stride, len, out_len, digests, n, stream) \
+          : lone ? launch_thin<V, false>(msgs, stride, len, out_len, digests, n, stream) \
+                 : launch_thin<V, true>(msgs, stride, len, out_len, digests, n, stream); \
+    return true
     switch (variant) {
-        case 0: *rc = launch_pair<0>(msgs, stride, len, out_len, digests, n, stream); return true;
-        case 1: *rc = launch_pair<1>(msgs, stride, len, out_len, digests, n, stream); return true;
-        case 2: *rc = launch_pair<2>(msgs, stride, len, out_len, digests, n, stream); return true;
-        case 3: *rc = launch_pair<3>(msgs, stride, len, out_len, digests, n, stream); return true;
-        case 4: *rc = launch_pair<4>(msgs, stride, len, out_len, digests, n, stream); return true;
-        case 5: *rc = launch_pair<5>(msgs, stride, len, out_len, digests, n, stream); return true;
+        case 0: KB_FEW(0);
+        case 1: KB_FEW(1);
+        case 2: KB_FEW(2);
+        case 3: KB_FEW(3);
+        case 4: KB_FEW(4);
+        case 5: KB_FEW(5);
         default: return false;
     }
+#undef KB_FEW
 }
 
 }  // namespace kb

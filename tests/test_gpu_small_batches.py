@@ -36,7 +36,7 @@ def run_uniform(cuda_lib, data, shift, stride, length, variant, out_len, n):
 
 @pytest.mark.parametrize("shift", [0, 1, 2, 3, 4, 7])
 @pytest.mark.parametrize("variant", range(6))
-@pytest.mark.parametrize("per_sm", [0, 13])  # thirty threads a message; two threads
+@pytest.mark.parametrize("per_sm", [0, 13, 70, 130])  # thirty threads a message; two; one, a warp or two a sub-partition
 def test_lengths_and_alignments(cuda_lib, variant, shift, per_sm):
     import torch
 
@@ -57,7 +57,7 @@ def test_lengths_and_alignments(cuda_lib, variant, shift, per_sm):
 
 
 @pytest.mark.parametrize("blocks", [1, 3])
-@pytest.mark.parametrize("edge", [8, 12, 64])  # the lines between the forms, in messages per SM
+@pytest.mark.parametrize("edge", [8, 12, 64, 128, 256])  # the lines between the forms, in messages per SM
 def test_batch_sizes_around_the_lines(cuda_lib, edge, blocks):
     import torch
 
