@@ -10,17 +10,17 @@
 // warp's 32 messages normally share one rate and the absorb can use the
 // rate's compile-time form.  The work order lists the buckets longest first.
 //   1. k_prep: digest-offset tile sums and a bucket histogram;
-//   2. k_plan: one block scans the tile sums, lays the buckets out longest
-//      first and sets the queue heads;
-//   3. k_scatter: digest offsets, and each message's slot in the work order;
-//   4. k_sha3_queue: a persistent grid; each warp takes a group of 32
+//   2. k_scatter: lays the buckets out longest first, digest offsets, and each
+//      message's slot in the work order; its first block splits the order between
+//      the next two kernels;
+//   3. k_sha3_queue: a persistent grid; each warp takes a group of 32
 //      consecutive entries of the order with one atomic and hashes one
 //      message per thread.  Warps run messages of nearly equal cost.  The
 //      queue has two ends: on every SM sub-partition the warp in the lowest
 //      hardware slot takes groups from the costly end (the longest chains
 //      start first), the others from the cheap end.
 //   k_sha3_lanes runs the first K entries of the order (the K costliest
-//   messages; K from k_plan, or given) one warp per message, concurrently with
+//   messages; K from the plan, or given) one warp per message, concurrently with
 //   the queue kernel, which covers the entries from K on: it is launched first and
 //   lets the queue kernel start as soon as its own blocks have.
 //
@@ -92,7 +92,7 @@ constexpr uint32_t kSlotWords = 48;  // SMs told apart: 192 (beyond, they share 
 
 struct Control {
     uint32_t count[kBuckets];        // messages per bucket
-    uint32_t cursor[kBuckets];       // next free slot of each bucket in the order
+    uint32_t cursor[kBuckets];       // slots of each bucket in the order that are taken
     unsigned long long head;         // warp-per-message schedule: next entry of the order
     unsigned long long lane_head;    // hybrid: next of the first K entries (one warp each)
     unsigned long long ends;         // queue: groups taken from the back (high 32 bits) and front (low)
@@ -149,19 +149,56 @@ __device__ __forceinline__ uint64_t bucket_cost(int b) {
 constexpr uint64_t kThreadChain = 4800000, kWarpChain = 1700000, kThreadWork = 215, kWarpWork = 3000;
 constexpr uint64_t kAutoSplit = ~uint64_t(0);
 
-// One block: exclusive scan of the tile sums, bucket starts in descending order
-// (bucket kBuckets-1 first), and the queue kernel's first entry: `split`, or for
-// kAutoSplit the number of messages that are better off with a warp each.  With W
-// permutations in all, w(b) of them in buckets above b and c(b) the cost of bucket
-// b, the batch lasts about max(c(b) kThreadChain, W kThreadWork, w(b) kWarpWork,
-// c_max kWarpChain) when the buckets above b go to warps; the first term falls
-// with b, the third rises, so the split is the first b where the first is no
-// longer the largest.  (A batch big enough to fill the GPU for its longest chain's
-// time splits off nothing.)
-static __global__ void __launch_bounds__(kScanThreads)
-    k_plan(uint64_t *tile_sums, uint64_t ntiles, Control *ctl, uint64_t split) {
-    constexpr int kPer = (kBuckets + kScanThreads - 1) / kScanThreads;  // buckets per thread
+// The queue kernel's first entry where the plan chooses it: the number of messages
+// that are better off with a warp each.  With W permutations in all, w(b) of them in
+// buckets above b and c(b) the cost of bucket b, the batch lasts about
+// max(c(b) kThreadChain, W kThreadWork, w(b) kWarpWork, c_max kWarpChain) when the
+// buckets above b go to warps; the first term falls with b, the third rises, so the
+// split is the first b where the first is no longer the largest.  (A batch big
+// enough to fill the GPU for its longest chain's time splits off nothing.)  Called
+// by a whole block; thread t holds the counts of buckets kBuckets-1 - (kPer t + j) and
+// `before`, the messages in buckets above them.
+constexpr int kPer = (kBuckets + kScanThreads - 1) / kScanThreads;
+__device__ __forceinline__ uint64_t plan_split(const uint32_t (&count)[kPer], uint64_t before) {
     __shared__ unsigned long long first_cut, cost_max;
+    if (threadIdx.x == 0) {
+        first_cut = ~0ull;
+        cost_max = 0;
+    }
+    uint64_t work = 0, top = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+        if (b >= 0 && count[j]) {
+            const uint64_t c = bucket_cost(b);
+            work += count[j] * c;
+            if (top == 0) top = c;  // buckets come in descending order of cost
+        }
+    }
+    uint64_t w;
+    const uint64_t all = block_exclusive_scan(work, w);  // (its barriers cover the lines above)
+    if (top) atomicMax(&cost_max, (unsigned long long)top);
+    __syncthreads();
+    uint64_t m = before;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+        if (b >= 0 && count[j]) {
+            const uint64_t c = bucket_cost(b), chain = c * kThreadChain;
+            if (chain <= all * kThreadWork || chain <= w * kWarpWork || chain <= cost_max * kWarpChain)
+                atomicMin(&first_cut, (unsigned long long)m);
+            m += count[j];
+            w += count[j] * c;
+        }
+    }
+    __syncthreads();
+    return first_cut;  // where no bucket met the condition, every message gets a warp
+}
+
+// Tile sums to the messages' exclusive sums, for batches of so many tiles that each
+// block of k_scatter would take long to add up those before its own.
+constexpr uint64_t kSumTiles = 4096;
+static __global__ void __launch_bounds__(kScanThreads) k_plan_tiles(uint64_t *tile_sums, uint64_t ntiles) {
     launch_next();
     launch_wait();
     uint64_t carry = 0;
@@ -173,61 +210,20 @@ static __global__ void __launch_bounds__(kScanThreads)
         if (i < ntiles) tile_sums[i] = carry + excl;
         carry += total;
     }
-    if (threadIdx.x == 0) {
-        first_cut = ~0ull;
-        cost_max = 0;
-    }
-    uint32_t count[kPer];
-    uint64_t messages = 0, work = 0;
-#pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
-        count[j] = b >= 0 ? ctl->count[b] : 0u;
-        messages += count[j];
-        if (b >= 0) work += count[j] * bucket_cost(b);
-    }
-    uint64_t m0, w0;
-    block_exclusive_scan(messages, m0);
-    const uint64_t all = block_exclusive_scan(work, w0);
-    if (split == kAutoSplit) {
-#pragma unroll
-        for (int j = kPer - 1; j >= 0; --j) {
-            const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
-            if (b >= 0 && count[j]) atomicMax(&cost_max, (unsigned long long)bucket_cost(b));
-        }
-        __syncthreads();
-        uint64_t m = m0, w = w0;
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
-            if (b < 0) break;
-            const uint64_t chain = bucket_cost(b) * kThreadChain;
-            if (count[j] && (chain <= all * kThreadWork || chain <= w * kWarpWork || chain <= cost_max * kWarpChain))
-                atomicMin(&first_cut, (unsigned long long)m);
-            m += count[j];
-            w += count[j] * bucket_cost(b);
-        }
-        __syncthreads();
-    }
-    uint64_t m = m0;
-#pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
-        if (b >= 0) ctl->cursor[b] = uint32_t(m);
-        m += count[j];
-    }
-    // No bucket met the condition: every message gets a warp.
-    if (threadIdx.x == 0) ctl->queue_start = split == kAutoSplit ? first_cut : split;
 }
 
+// Digest offsets, and each message's slot in the work order.  Every block lays the
+// buckets out by itself, in descending order (bucket kBuckets-1 first), and block 0
+// chooses the queue kernel's first entry (`split`, or by plan_split for kAutoSplit): a
+// launch of one block for that in between took 9 to 11 us.
 template <bool BY_VARIANT>
 __global__ void __launch_bounds__(kScanThreads)
     k_scatter(const uint64_t *__restrict__ lens, const uint8_t *__restrict__ variants,
               const uint32_t *__restrict__ out_lens, uint64_t n, const uint64_t *__restrict__ tile_sums,
-              uint64_t *__restrict__ out_off, uint32_t *__restrict__ order, Control *ctl) {
+              uint64_t ntiles, uint64_t *__restrict__ out_off, uint32_t *__restrict__ order, Control *ctl,
+              uint64_t split) {
     __shared__ uint32_t hist[kBuckets];
     __shared__ uint32_t start[kBuckets];
-    launch_next();
     for (int b = threadIdx.x; b < kBuckets; b += blockDim.x) hist[b] = 0;
     __syncthreads();
     launch_wait();
@@ -247,21 +243,47 @@ __global__ void __launch_bounds__(kScanThreads)
         }
         s += d[j];
     }
-    uint64_t excl;
+    // Bytes of output before this block's messages.
+    uint64_t tile = 0, excl;
+    if (ntiles > kSumTiles) {
+        tile = tile_sums[blockIdx.x];  // k_plan_tiles has added them up
+    } else {
+        uint64_t mine = 0;
+        for (uint64_t t = threadIdx.x; t < blockIdx.x; t += kScanThreads) mine += tile_sums[t];
+        tile = block_exclusive_scan(mine, excl);
+    }
     block_exclusive_scan(s, excl);
-    uint64_t acc = tile_sums[blockIdx.x] + excl;
+    uint64_t acc = tile + excl;
 #pragma unroll
     for (int j = 0; j < kScanItems; ++j) {
         if (base + j < n) out_off[base + j] = acc;
         acc += d[j];
     }
-    __syncthreads();
-    for (int b = threadIdx.x; b < kBuckets; b += blockDim.x)
-        start[b] = hist[b] ? atomicAdd(&ctl->cursor[b], hist[b]) : 0u;
+    // The buckets' first slots.
+    uint32_t count[kPer];
+    uint64_t messages = 0, m0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+        count[j] = b >= 0 ? ctl->count[b] : 0u;
+        messages += count[j];
+    }
+    block_exclusive_scan(messages, m0);
+    uint32_t m = uint32_t(m0);
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+        if (b >= 0) start[b] = m + (hist[b] ? atomicAdd(&ctl->cursor[b], hist[b]) : 0u);
+        m += count[j];
+    }
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < kScanItems; ++j)
         if (base + j < n) order[start[key[j]] + rank[j]] = uint32_t(base + j);
+    if (blockIdx.x == 0) {
+        const uint64_t first = split == kAutoSplit ? plan_split(count, m0) : split;
+        if (threadIdx.x == 0) ctl->queue_start = first;
+    }
 }
 
 // The persistent queue kernel: one thread per message, 32 messages per

@@ -19,7 +19,7 @@ struct QueueConfig {
     int blocks_per_sm = 0;      // blocks per SM of the launch (0: as many as fit)
     int stage = 2 | 4;          // how message blocks are read: registers, looped permutation (kStageRegs | kLooped)
     int64_t warp_messages = 0;  // the K costliest messages run one warp each, unless auto_split
-    bool auto_split = true;     // K from the batch's costs (k_plan)
+    bool auto_split = true;     // K from the batch's costs (plan_split)
     bool lanes = false;         // control: every message one warp
     bool per_variant = false;   // control: one launch per variant, unsorted
     float ms = 0;               // the autotuner's time for this configuration

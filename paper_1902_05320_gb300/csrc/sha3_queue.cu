@@ -3,7 +3,7 @@
 // autotuner, plus the direct-load instances of the queue kernel and the two
 // control schedules.
 //
-// The six operations of a call (a memset and five kernels, the last two side by
+// The five operations of a call (a memset and four kernels, the last two side by
 // side) are captured once per call signature into a CUDA graph and replayed
 // afterwards.
 // A control schedule groups the messages by variant instead and hashes each
@@ -53,6 +53,7 @@ __global__ void __launch_bounds__(32)
                  const uint32_t *__restrict__ order, uint8_t *__restrict__ digests, uint64_t n, bool all, Control *ctl,
                  unsigned int *status) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
+    launch_wait();
     const uint64_t limit = all || ctl->queue_start > n ? n : ctl->queue_start;
     unsigned long long *head = all ? &ctl->head : &ctl->lane_head;
     if (limit == 0) return;
@@ -118,7 +119,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
                    const uint64_t *__restrict__ out_off, const uint32_t *__restrict__ order,
                    uint8_t *__restrict__ digests, const Control *ctl, unsigned int *status) {
     using P = Variant<V>;
-    const uint64_t end = ctl->cursor[V], begin = end - ctl->count[V];
+    uint64_t begin = 0;  // the order lists the higher variants (6: invalid ones) first
+    for (int b = V + 1; b <= 6; ++b) begin += ctl->count[b];
+    const uint64_t end = begin + ctl->count[V];
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t k = begin + uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < end; k += step) {
         const uint32_t i = order[k];
@@ -219,11 +222,19 @@ int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *le
     const uint64_t ntiles = digest_offsets_tiles(n);
     const Buffers bf = carve(scratch, n, ntiles);
     if (cudaMemsetAsync(bf.ctl, 0, sizeof(Control), stream) != cudaSuccess) return KB_ERR_CUDA;
+    // Bookkeeping: the buckets' counts, then offsets and order.
+    auto book = [&](auto prep, auto scatter, uint64_t split) -> int {
+        prep<<<unsigned(ntiles), kScanThreads, 0, stream>>>(lens, variants, out_lens, n, bf.tile_sums, bf.ctl);
+        if (cudaGetLastError() != cudaSuccess) return KB_ERR_CUDA;
+        if (ntiles > kSumTiles &&
+            launch_overlapped(k_plan_tiles, 1, kScanThreads, 0, stream, bf.tile_sums, ntiles) != cudaSuccess)
+            return KB_ERR_CUDA;
+        return cuda_status(launch_overlapped(scatter, unsigned(ntiles), kScanThreads, 0, stream, lens, variants,
+                                             out_lens, n, bf.tile_sums, ntiles, bf.out_off, bf.order, bf.ctl, split));
+    };
+    int rc = KB_OK;
     if (cfg.per_variant) {
-        k_prep<true><<<unsigned(ntiles), kScanThreads, 0, stream>>>(lens, variants, out_lens, n, bf.tile_sums, bf.ctl);
-        k_plan<<<1, kScanThreads, 0, stream>>>(bf.tile_sums, ntiles, bf.ctl, 0);
-        k_scatter<true><<<unsigned(ntiles), kScanThreads, 0, stream>>>(lens, variants, out_lens, n, bf.tile_sums,
-                                                                       bf.out_off, bf.order, bf.ctl);
+        if ((rc = book(k_prep<true>, k_scatter<true>, 0)) != KB_OK) return rc;
         const unsigned g = unsigned(grid);
         k_sha3_variant<0><<<g, kThreads, 0, stream>>>(msgs, offsets, lens, out_lens, bf.out_off, bf.order, digests, bf.ctl, status);
         k_sha3_variant<1><<<g, kThreads, 0, stream>>>(msgs, offsets, lens, out_lens, bf.out_off, bf.order, digests, bf.ctl, status);
@@ -235,24 +246,20 @@ int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *le
         return cuda_status(cudaGetLastError());
     }
     // The warp-per-message share: the costliest messages (the order's first
-    // entries), as many as k_plan finds or a fixed number.
+    // entries), as many as the plan finds or a fixed number.
     const uint64_t fixed = std::min<uint64_t>(uint64_t(cfg.warp_messages), n);
     const uint64_t split = cfg.lanes ? 0 : cfg.auto_split ? kAutoSplit : fixed;
-    k_prep<false><<<unsigned(ntiles), kScanThreads, 0, stream>>>(lens, variants, out_lens, n, bf.tile_sums, bf.ctl);
-    if (launch_overlapped(k_plan, 1, kScanThreads, 0, stream, bf.tile_sums, ntiles, bf.ctl, split) != cudaSuccess ||
-        launch_overlapped(k_scatter<false>, unsigned(ntiles), kScanThreads, 0, stream, lens, variants, out_lens, n,
-                          bf.tile_sums, bf.out_off, bf.order, bf.ctl) != cudaSuccess)
-        return KB_ERR_CUDA;
+    if ((rc = book(k_prep<false>, k_scatter<false>, split)) != KB_OK) return rc;
     if (cfg.lanes) {
-        k_sha3_lanes<<<unsigned(grid), 32, 0, stream>>>(msgs, offsets, lens, variants, out_lens, bf.out_off, bf.order,
-                                                       digests, n, true, bf.ctl, status);
-        return cuda_status(cudaGetLastError());
+        return cuda_status(launch_overlapped(k_sha3_lanes, unsigned(grid), 32, 0, stream, msgs, offsets, lens, variants,
+                                             out_lens, bf.out_off, bf.order, digests, n, true, bf.ctl, status));
     }
     if (split != 0) {
         const uint64_t most = kLanesPerSm * uint64_t(sm_count > 0 ? sm_count : 1);
-        k_sha3_lanes<<<unsigned(std::min(cfg.auto_split ? n : fixed, most)), 32, 0, stream>>>(
-            msgs, offsets, lens, variants, out_lens, bf.out_off, bf.order, digests, n, false, bf.ctl, status);
-        if (cudaGetLastError() != cudaSuccess) return KB_ERR_CUDA;
+        if (launch_overlapped(k_sha3_lanes, unsigned(std::min(cfg.auto_split ? n : fixed, most)), 32, 0, stream, msgs,
+                              offsets, lens, variants, out_lens, bf.out_off, bf.order, digests, n, false, bf.ctl,
+                              status) != cudaSuccess)
+            return KB_ERR_CUDA;
     }
     if (!cfg.auto_split && fixed == n) return KB_OK;  // every message has a warp
     const void *fn = queue_kernel(cfg.minb, cfg.stage);
@@ -260,8 +267,8 @@ int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *le
     Control *ctl = bf.ctl;
     void *args[] = {&msgs, &offsets, &lens, &variants, &out_lens, const_cast<uint64_t **>(&bf.out_off),
                     const_cast<uint32_t **>(&bf.order), &digests, &n, &ctl, &status};
-    // Beside k_sha3_lanes: both need k_scatter alone, which had ended before the
-    // first block of k_sha3_lanes started.
+    // Beside k_sha3_lanes: both need k_scatter alone, and the blocks of k_sha3_lanes
+    // let this kernel start (or exit) only after they have seen that end.
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
