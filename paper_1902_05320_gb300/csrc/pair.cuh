@@ -51,30 +51,37 @@ __device__ __forceinline__ void pair_row(const uint32_t (&S)[25], const uint32_t
     for (int x = 0; x < 5; ++x) N[x + 5 * Y] = chi3(B[x], B[(x + 1) % 5], B[(x + 2) % 5]);
 }
 
+// Round ir; lo_mask = h - 1 (all ones on the threads with the low words).
+__device__ __forceinline__ void pair_round(uint32_t (&S)[25], uint32_t h, uint32_t lo_mask, int ir) {
+    uint32_t C[5], R[5], N[25];
+#pragma unroll
+    for (int x = 0; x < 5; ++x) C[x] = xor3(xor3(S[x], S[x + 5], S[x + 10]), S[x + 15], S[x + 20]);
+#pragma unroll
+    for (int x = 0; x < 5; ++x) R[x] = pair_rotl<1>(C[x]);
+    pair_row<0>(S, C, R, N);
+    pair_row<1>(S, C, R, N);
+    pair_row<2>(S, C, R, N);
+    pair_row<3>(S, C, R, N);
+    pair_row<4>(S, C, R, N);
+    // The constant's high word is bit 31 alone or nothing: a sum will do.
+    N[0] = (N[0] ^ (c_rc.w[2 * ir] & lo_mask)) + c_rc.w[2 * ir + 1] * h;
+#pragma unroll
+    for (int i = 0; i < 25; ++i) S[i] = N[i];
+}
+
 // Keccak-f[1600]; every thread of the warp calls it.  h: which word of the lanes
-// this thread holds (its lane number's last bit).
+// this thread holds (its lane number's last bit).  TAIL: rounds [TAIL, 24) are
+// unrolled, so that the last one keeps only the lanes that are used.
+template <int TAIL = 24, int UNROLL = 4>
 __device__ __forceinline__ void pair_permute(uint32_t (&S)[25], uint32_t h) {
     const uint32_t lo_mask = h - 1u;
 #pragma unroll 1
-    for (int r = 0; r < 24; r += 4) {
+    for (int r = 0; r < TAIL; r += UNROLL) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            uint32_t C[5], R[5], N[25];
-#pragma unroll
-            for (int x = 0; x < 5; ++x) C[x] = xor3(xor3(S[x], S[x + 5], S[x + 10]), S[x + 15], S[x + 20]);
-#pragma unroll
-            for (int x = 0; x < 5; ++x) R[x] = pair_rotl<1>(C[x]);
-            pair_row<0>(S, C, R, N);
-            pair_row<1>(S, C, R, N);
-            pair_row<2>(S, C, R, N);
-            pair_row<3>(S, C, R, N);
-            pair_row<4>(S, C, R, N);
-            // The constant's high word is bit 31 alone or nothing: a sum will do.
-            N[0] = (N[0] ^ (c_rc.w[2 * (r + j)] & lo_mask)) + c_rc.w[2 * (r + j) + 1] * h;
-#pragma unroll
-            for (int i = 0; i < 25; ++i) S[i] = N[i];
-        }
+        for (int j = 0; j < UNROLL; ++j) pair_round(S, h, lo_mask, r + j);
     }
+#pragma unroll
+    for (int r = TAIL; r < 24; ++r) pair_round(S, h, lo_mask, r);
 }
 
 // Bytes [p, p + nvalid) as a little-endian 32-bit word, nvalid <= 4, any
@@ -88,6 +95,51 @@ __device__ __forceinline__ uint32_t ld_u32_any(const uint8_t *p, uint32_t nvalid
     const uint32_t w1 = o + nvalid > 4 ? __ldg(a + 1) : 0u;
     const uint32_t v = __funnelshift_r(w0, w1, 8 * o);
     return nvalid < 4 ? v & ((1u << (8 * nvalid)) - 1u) : v;
+}
+
+// Writes bytes [0, nbytes) of the rate part to dst.
+template <int RATE>
+__device__ __forceinline__ void pair_squeeze(const uint32_t (&S)[25], bool active, uint32_t h, uint8_t *dst,
+                                             uint32_t nbytes) {
+    const bool whole = ((reinterpret_cast<uintptr_t>(dst) | nbytes) & 3) == 0;
+#pragma unroll
+    for (int k = 0; k < RATE / 8; ++k) {
+        const uint32_t at = 8 * k + 4 * h;
+        if (!active || at >= nbytes) continue;
+        if (whole) {
+            *reinterpret_cast<uint32_t *>(dst + at) = S[k];
+        } else {
+            const uint32_t nb = nbytes - at < 4 ? nbytes - at : 4;
+            for (uint32_t b = 0; b < nb; ++b) dst[at + b] = uint8_t(S[k] >> (8 * b));
+        }
+    }
+}
+
+// A message of one block (len < RATE, dlen <= RATE; dlen <= 8 OUT lanes).  Words are
+// taken whole, in part or not at all by branches on the common length.
+template <int RATE, int DOMAIN, int OUT>
+__device__ __forceinline__ void pair_one_block(bool active, const uint8_t *p, uint32_t len, uint8_t *dst,
+                                               uint32_t dlen) {
+    const uint32_t h = threadIdx.x & 1u;
+    uint32_t S[25];
+    const uintptr_t q = reinterpret_cast<uintptr_t>(p) + 4 * h;
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(q & ~uintptr_t(3));
+    const uint32_t o = uint32_t(q & 3);
+#pragma unroll
+    for (int k = 0; k < 25; ++k) {
+        S[k] = 0;
+        if (k >= RATE / 8) continue;
+        if (uint32_t(8 * k + 8) <= len) {
+            if (active) S[k] = __funnelshift_r(__ldg(w + 2 * k), o ? __ldg(w + 2 * k + 1) : 0u, 8 * o);
+        } else if (uint32_t(8 * k) <= len) {
+            const uint32_t at = 8 * k + 4 * h, left = len > at ? len - at : 0;
+            if (active) S[k] = ld_u32_any(p + at, left < 4 ? left : 4u);
+            if (len / 4 == at / 4) S[k] ^= uint32_t(DOMAIN) << (8 * (len & 3));
+        }
+        if (k == RATE / 8 - 1) S[k] ^= h << 31;
+    }
+    pair_permute<22, 2>(S, h);
+    pair_squeeze<8 * OUT>(S, active, h, dst, dlen);
 }
 
 // One sponge in the pair: the message of len bytes at p, dlen output bytes to dst.
@@ -113,20 +165,6 @@ __device__ __forceinline__ void pair_sponge(bool active, const uint8_t *p, uint6
 #pragma unroll
         for (int k = 0; k < kWords; ++k) w[k] = active ? __ldg(q + 2 * k) : 0u;
         w[kWords] = active && sh && h == 0 ? __ldg(q + 2 * kWords) : 0u;
-    };
-    auto squeeze_block = [&](uint8_t *o, uint32_t nbytes) {
-        const bool whole = ((reinterpret_cast<uintptr_t>(o) | nbytes) & 3) == 0;
-#pragma unroll
-        for (int k = 0; k < kWords; ++k) {
-            const uint32_t at = 8 * k + 4 * h;
-            if (!active || at >= nbytes) continue;
-            if (whole) {
-                *reinterpret_cast<uint32_t *>(o + at) = S[k];
-            } else {
-                const uint32_t nb = nbytes - at < 4 ? nbytes - at : 4;
-                for (uint32_t b = 0; b < nb; ++b) o[at + b] = uint8_t(S[k] >> (8 * b));
-            }
-        }
     };
     const bool unaligned = __any_sync(0xffffffffu, sh != 0);
     if (nfull) fetch(0);
@@ -155,11 +193,11 @@ __device__ __forceinline__ void pair_sponge(bool active, const uint8_t *p, uint6
                 S[k] ^= v;
             }
         } else {
-            squeeze_block(dst + (i - nfull - 1) * RATE, RATE);
+            pair_squeeze<RATE>(S, active, h, dst + (i - nfull - 1) * RATE, RATE);
         }
         pair_permute(S, h);
     }
-    squeeze_block(dst + uint64_t(nsq) * RATE, dlen - nsq * RATE);
+    pair_squeeze<RATE>(S, active, h, dst + uint64_t(nsq) * RATE, dlen - nsq * RATE);
 }
 
 }  // namespace kb

@@ -33,6 +33,20 @@ __global__ void __launch_bounds__(kThreads)
     pair_sponge<Variant<V>::rate, Variant<V>::domain>(m < n, msgs + m * stride, len, out + m * out_len, out_len);
 }
 
+// The same for messages of one block, which need no loop over blocks and only the
+// output's lanes of the last round.
+template <int V>
+__global__ void __launch_bounds__(kThreads)
+    k_sha3_uniform_pair_one(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len, uint8_t *__restrict__ out,
+                            uint32_t out_len, uint64_t n) {
+    using P = Variant<V>;
+    const uint64_t m = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 1;
+    launch_wait();
+    launch_next();
+    pair_one_block<P::rate, P::domain, P::digest ? (P::digest + 7) / 8 : P::rate / 8>(
+        m < n, msgs + m * stride, uint32_t(len), out + m * out_len, out_len);
+}
+
 // A thread per message where that gives a sub-partition one warp or two: few warps
 // do not hide each other's loads, so each thread's next block is loaded into
 // registers before the permutation, which for a lone warp keeps to funnel shifts
@@ -96,7 +110,8 @@ template <int V>
 int launch_pair(const uint8_t *msgs, uint64_t stride, uint64_t len, uint32_t out_len, uint8_t *digests, uint64_t n,
                 cudaStream_t stream) {
     const uint64_t per_block = kThreads / 2;
-    return cuda_status(launch_overlapped(k_sha3_uniform_pair<V>, unsigned((n + per_block - 1) / per_block), kThreads, 0,
+    const bool one = len < uint64_t(Variant<V>::rate) && out_len <= uint32_t(Variant<V>::rate);
+    return cuda_status(launch_overlapped(one ? k_sha3_uniform_pair_one<V> : k_sha3_uniform_pair<V>, unsigned((n + per_block - 1) / per_block), kThreads, 0,
                                          stream, msgs, stride, len, digests, out_len, n));
 }
 
@@ -105,8 +120,6 @@ int launch_pair(const uint8_t *msgs, uint64_t stride, uint64_t len, uint32_t out
 bool launch_uniform_small(const uint8_t *msgs, uint64_t stride, uint64_t len, int variant, uint32_t out_len,
                           uint8_t *digests, uint64_t n, cudaStream_t stream, const DeviceInfo &dev, int *rc) {
     const uint64_t sms = uint64_t(dev.sm_count > 0 ? dev.sm_count : 1);
-    // A message of one permutation: a thread each folds round 0 and most of the
-    // last, and beats two threads (6.1 against 6.5 us a launch).
     const uint32_t rate = uint32_t(variant_rate(variant));
     const bool one = len < rate && out_len <= rate;
     if (n <= (one ? kCoopOnePerSm : kCoopPerSm) * sms) {
@@ -114,7 +127,11 @@ bool launch_uniform_small(const uint8_t *msgs, uint64_t stride, uint64_t len, in
                                             digests, out_len));
         return true;
     }
-    if (one || n > kThinPerSm * sms) return false;
+    // One-block messages: a thread each folds round 0 and most of the last, so two
+    // threads gain less, and lose where their many 4-byte loads queue ahead of the
+    // shuffles (4096 messages, us a call: 10 bytes 4.68 against 5.83, 64 bytes 5.04
+    // against 5.64, 135 bytes 7.04 against 5.82).
+    if (n > (one ? kPairPerSm : kThinPerSm) * sms || (one && len > 72)) return false;
     const bool pair = n <= kPairPerSm * sms, lone = n <= kThinPerSm / 2 * sms;
 #define KB_FEW(V) \
     *rc = pair   ? launch_pair<V>(msgs, stride, len, out_len, digests, n, stream) \
