@@ -49,7 +49,9 @@ ROUND_OPS_NO_IOTA = 20 + 5 + 50 + 47 + 50
 # SMs x 32-bit integer lanes per SM per clock x maximum SM clock: the ALU
 # issue roofline.  LOP3 and SHF run on the ALU pipe, which takes one warp
 # instruction per SM sub-partition every two cycles (ncu's pipe counters on
-# the hashing kernel), i.e. 16 lanes per sub-partition and 64 per SM.
+# the hashing kernel), i.e. 16 lanes per sub-partition and 64 per SM.  The
+# kernels run part of the rotations on the multiply pipe beside it, so a
+# fraction of this peak can pass 1.
 SM_COUNT_GB300 = 152
 INT_LANES_PER_SM_CLK = 64
 SM_MAX_MHZ = 2070.0
@@ -371,7 +373,8 @@ def main() -> None:
                      "frac": achieved / peak, "traffic": traffic,
                      "ops_per_hash": ops_perm,
                      "peak_basis": f"{SM_COUNT_GB300} SMs x {INT_LANES_PER_SM_CLK} int32 lanes/clk x "
-                                   f"{SM_MAX_MHZ:.0f} MHz max SM clock",
+                                   f"{SM_MAX_MHZ:.0f} MHz max SM clock (the ALU pipe; part of the rotations run on "
+                                   "the multiply pipe beside it, so frac can pass 1)",
                      "kernel": "k_sha3_uniform64_tma<SHA3-256> (64-byte messages staged by bulk copies)"},
         "e2e": e2e,
         "gpu_launches": args.steps,

@@ -7,7 +7,7 @@
 //  * PlainRep (the default): lane i is (L[i], H[i]) = its low and high 32-bit
 //    halves, i.e. the little-endian message words themselves.  A 64-bit
 //    rotation by n is two SHF funnel shifts (none for n = 0, a register swap
-//    for n = 32).
+//    for n = 32), or for small n two shifts by a multiplication (below).
 //  * InterleavedRep: lane i is (E[i], O[i]) = its even and odd bits.  A 64-bit
 //    rotation becomes two 32-bit rotations, which saves 6 SHF per round
 //    (theta's rotation by 1 and rho's offset-1 lane need one SHF instead of
@@ -16,7 +16,7 @@
 //    outweighs the saving for every message size, so this form is kept as the
 //    measured control.
 //
-// Round function (Eq. 10), per 32-bit word, written as LOP3 and SHF:
+// Round function (Eq. 10), per 32-bit word, written as LOP3, SHF and IMAD:
 //   theta (Eq. 2-4): column parities C (two 3-input XORs per word), the
 //     rotated parity rot(C[x+1], 1), then A ^ C[x-1] ^ rot(C[x+1], 1) in one
 //     3-input LOP3 per word;
@@ -24,15 +24,16 @@
 //     and a compile-time renaming of registers (pi costs nothing);
 //   chi (Eq. 7): a ^ (~b & c), one LOP3 per word;
 //   iota (Eq. 8-9, the paper's "zeta"): XOR of the round constant into lane 0.
-// Plain form: 20 + 10 + 50 + 48 + 50 + 2 = 180 instructions per round.
+// Plain form: 20 + 10 + 50 + 48 + 50 + 2 = 180 instructions per round, all on the
+// ALU pipe; with the rotations of plain_round_rt on the multiply pipe, fewer there.
 //
-// Round structure: the first rounds run in a loop of four rounds per
-// iteration that reads the round constants from a __constant__ table (the
-// placement Section 4.2 uses) -- a fully unrolled 24-round body is larger
-// than the instruction cache serves well; the last four rounds are unrolled
-// with the constants as immediates, so when only a few output lanes are used
-// the compiler drops the rest of the final round.  Round 0 can be peeled the
-// same way when most of the input state is known to be zero.
+// Round structure: the rounds run in a loop of a few rounds per iteration that
+// reads the round constants from a __constant__ table (the placement Section
+// 4.2 uses) -- a fully unrolled 24-round body is larger than the instruction
+// cache serves well.  One-block kernels peel round 0, since most of the input
+// state is known to be zero there, and unroll the last rounds with the
+// constants as immediates, so that the compiler drops what the output does not
+// use of the final round; kernels that absorb several blocks loop over all 24.
 #pragma once
 
 #include <cstdint>

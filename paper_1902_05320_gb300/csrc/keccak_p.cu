@@ -10,6 +10,9 @@
 // lanes serves all widths and all round indices.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <climits>
+
 #include "coop.cuh"
 #include "keccak_core.cuh"
 #include "runtime.cuh"
@@ -305,8 +308,7 @@ int launch_keccak_p(uint64_t *states, int b, int nr, uint64_t n, cudaStream_t st
             // states: 12 rounds 2.53 ms read directly, 2.15 ms staged; 24
             // rounds 3.84 ms directly, 4.02 ms staged).
             if (nr < 16) return launch_tiled(k_keccak_p_1600<true>, states, first_ir, nr, n, stream, dev);
-            const uint64_t g =
-                persistent_grid(reinterpret_cast<const void *>(&k_keccak_p_1600<false>), kThreads, 0, n, dev);
+            const uint64_t g = std::min<uint64_t>((n + kThreads - 1) / kThreads, uint64_t(INT32_MAX));
             return cuda_status(
                 launch_overlapped(k_keccak_p_1600<false>, unsigned(g), kThreads, 0, stream, states, first_ir, nr, n));
         }

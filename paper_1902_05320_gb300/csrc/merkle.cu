@@ -10,9 +10,9 @@
 // Kernels: one thread per leaf (the prefixed message is read through a
 // one-byte funnel shift of the leaf's aligned words), then the levels above
 // (0x01 || left || right is exactly one 65-byte block at rate 136), one thread
-// per parent node: one launch per level while a level has more than 16384
-// parents, and above that climbing launches that reduce up to six levels
-// each, the upper ones inside each warp through shuffles.
+// per parent node: one launch per level while a level has more than kClimbPerSm
+// parents per SM, and above that climbing launches that reduce up to four
+// levels each with a warp per node.  Few leaves take a warp each as well.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -471,8 +471,7 @@ int launch_upper_levels(uint8_t *nodes, uint64_t n, cudaStream_t stream, const D
     while (n > 1) {
         const uint64_t parents = n / 2 + (n & 1);
         if (parents > kClimbPerSm * uint64_t(dev.sm_count > 0 ? dev.sm_count : 1)) {
-            const uint64_t grid =
-                persistent_grid(reinterpret_cast<const void *>(&k_merkle_level), kThreads, 0, parents, dev);
+            const uint64_t grid = std::min<uint64_t>((parents + kThreads - 1) / kThreads, uint64_t(INT32_MAX));
             if (launch_overlapped(k_merkle_level, unsigned(grid), kThreads, 0, stream, level, n, level + 32 * n) !=
                 cudaSuccess)
                 return KB_ERR_CUDA;

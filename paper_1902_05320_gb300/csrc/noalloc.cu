@@ -8,7 +8,7 @@
 // budget, a plugin or real-time host whose rules forbid cudaMalloc (it can
 // synchronise the whole device and stall unrelated work), or code that must
 // know its memory footprint before it runs.  This entry point runs the same
-// cost-bucketed queue (its prep, plan, scatter and hashing kernels, in the
+// cost-bucketed queue (its prep, scatter and hashing kernels, in the
 // built-in configuration, launched directly without a graph) with the
 // scratch in a fixed, file-scope device array instead: every GPU that loads
 // the library holds that array until the process exits, and no call here

@@ -4,7 +4,7 @@
 //
 // Three schedules, chosen by KB_TUNE_RAGGED_SCHEDULE:
 //  * the cost-bucketed persistent work queue of sha3_queue.cu (default), with
-//    one thread per message or, in its lane-parallel form, one warp per
+//    one thread per message or, in its other form, one warp per
 //    message;
 //  * input order, kept as the plain one-launch control: digest offsets by an
 //    exclusive prefix sum of out_lens (three small kernels), then one thread

@@ -8,8 +8,9 @@
 // block, round 0 on zero capacity lanes), and a general runtime length; the
 // runtime forms with 8-byte aligned loads or at any alignment.  The state representation is
 // a template parameter: plain 32-bit halves by default, bit-interleaved
-// halves as the measured control for SHA3-256.  A grid of (occupancy x SMs)
-// blocks strides over the messages.
+// halves as the measured control for SHA3-256.  A thread takes one message, and the
+// grid as many blocks as that takes.  Batches that give an SM sub-partition two warps or fewer
+// go to sha3_small.cu first.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -25,12 +26,14 @@ namespace kb {
 namespace {
 
 // Blocks per SM a kernel is compiled for.  With rotations on the multiply pipe more
-// warps are wanted to keep both pipes fed: 2^24 64-byte messages take 3.31 ms at a
-// budget of 4 (5 blocks fit), 3.29 at 5, 3.24 at 6; 2^22 messages of 32 bytes 855 us
-// at 4, 848 at 5, 840 at 6 (loop of two rounds; of four: 915, 901, 893).  The
-// multi-block kernel stays at kMinBlocks (2^18 messages of 1023 bytes 820 us; 837 at
-// 5, 851 at 6, spilling).
-constexpr int min_blocks(int len) { return len == -1 ? kMinBlocks : 6; }
+// warps keep both pipes fed, as long as nothing spills: 2^24 64-byte messages staged
+// by bulk copies 3143 us at 5, 3179 at 6, 3135 at 7; 2^22 messages of 32 bytes 824 at 4,
+// 815 at 5 and 6, 805 at 7, of 135 bytes 861, 842, 840 and 830 (at 8 these spill: 3355,
+// 867 and 893).  The 64-byte kernel that loads directly takes 868 at 6 and 908 at 7, the
+// multi-block kernel is best at kMinBlocks (2^18 messages of 1023 bytes 820; 837 at 5,
+// 851 at 6, spilling).
+constexpr int min_blocks(int len) { return len == -1 ? kMinBlocks : len == -2 ? 7 : 6; }
+constexpr int kStagedMinBlocks = 7;
 
 // LEN >= 0: compile-time message length; -1: runtime; -2: runtime, below the
 // rate, with at most one block of output.  A8: base and stride are multiples
@@ -88,113 +91,84 @@ __global__ void __launch_bounds__(kThreads, min_blocks(LEN))
     }
 }
 
-// The 64-byte form with its messages staged through shared memory by bulk
-// asynchronous copies (cp.async.bulk, completed on an mbarrier): a block takes
-// tiles of kThreads consecutive messages (8 KiB, one copy issued by thread 0),
-// two buffers deep, so the next tile arrives while the current one is hashed.
-// Each thread reads its message from shared memory; once every thread has
-// read the buffer (a proxy fence, then a block barrier) thread 0 refills it
-// with the tile after next, and the hashing runs while that copy is in
-// flight.  Needs stride 64 and a 16-byte aligned base in device memory.  A
-// wait that outlasts kWaitNs sets KB_DEV_TIMEOUT; the block then waits
-// (bounded) for its copies in flight and stops without writing the rest of
-// its digests.
+// The 64-byte form with its messages staged through shared memory by a bulk
+// asynchronous copy (cp.async.bulk, completed on an mbarrier): a block takes one
+// tile of kThreads consecutive messages (8 KiB, copied by thread 0) and ends; the
+// other blocks of its SM hash while its copy is in flight.  Needs stride 64 and a
+// 16-byte aligned base in device memory.  A wait that outlasts kWaitNs sets
+// KB_DEV_TIMEOUT; the thread then waits (bounded) once more for the copy and stops
+// without writing its digest.
+//
+// What bounds it is the round (keccak_core.cuh); why one tile a block: the warp in
+// a sub-partition's lowest slot issues first, so blocks with equal shares of the
+// tiles finish one after the other and leave the last alone, with too few warps to
+// fill the pipes, while blocks that take a tile at a time are replaced until the
+// tiles run out.  2^24 messages: 3258 us with 912 blocks that share all tiles and
+// load two ahead, 3173 with 16 tiles a block, 3164 with 4 and 3169 with 1; 119,040
+// messages 41.3, 82.3, 41.2 and 35.5.
 constexpr uint32_t kTileBytes = kThreads * 64;  // 8 KiB
 constexpr uint64_t kWaitNs = 1000000000ull;     // 1 s
 
 template <int V, class Rep>
-__global__ void __launch_bounds__(kThreads, min_blocks(64))
+__global__ void __launch_bounds__(kThreads, kStagedMinBlocks)
     k_sha3_uniform64_tma(const uint8_t *__restrict__ msgs, uint8_t *__restrict__ out, uint32_t out_len, uint64_t n,
                          unsigned int *status) {
     using P = Variant<V>;
     static_assert(64 < P::rate, "a 64-byte message is one block for every variant");
     constexpr int kOut = P::digest ? P::digest : P::rate;
-    __shared__ __align__(128) uint8_t buf[2][kTileBytes];
-    __shared__ __align__(8) uint64_t bar[2];
-    const uint64_t ntiles = (n + kThreads - 1) / kThreads;
-    const uint32_t dlen = P::digest ? uint32_t(P::digest) : out_len;
-    const uint64_t stride = gridDim.x;
-    // Thread 0 issues the copies; uses[b] counts the copies issued into buffer b.
-    uint32_t uses[2] = {0, 0};
-    auto issue = [&](uint64_t tile, int b) {
-        const uint64_t first = tile * kThreads;
-        const uint32_t bytes = uint32_t(n - first < kThreads ? n - first : uint64_t(kThreads)) * 64;
-        mbar_arrive_expect_tx(&bar[b], bytes);
-        bulk_copy_g2s(buf[b], msgs + first * 64, bytes, &bar[b]);
-        ++uses[b];
-    };
+    __shared__ __align__(128) uint8_t buf[kTileBytes];
+    __shared__ __align__(8) uint64_t bar;
+    const uint64_t first = uint64_t(blockIdx.x) * kThreads;
     if (threadIdx.x == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
+        mbar_init(&bar, 1);
         fence_barrier_init();
+        launch_wait();
+        const uint32_t bytes = uint32_t(n - first < kThreads ? n - first : uint64_t(kThreads)) * 64;
+        mbar_arrive_expect_tx(&bar, bytes);
+        bulk_copy_g2s(buf, msgs + first * 64, bytes, &bar);
     }
     __syncthreads();
     launch_wait();
-    if (threadIdx.x == 0) {
-        if (blockIdx.x < ntiles) issue(blockIdx.x, 0);
-        if (blockIdx.x + stride < ntiles) issue(blockIdx.x + stride, 1);
+    if (!mbar_wait_bounded(&bar, 0, kWaitNs)) {
+        atomicOr(status, KB_DEV_TIMEOUT);
+        mbar_wait_bounded(&bar, 0, kWaitNs);  // the copy may still land: not into another block's memory
+        return;
     }
-    uint32_t k = 0;
-    for (uint64_t tile = blockIdx.x; tile < ntiles; tile += stride, ++k) {
-        const int b = int(k & 1);
-        const bool ok = mbar_wait_bounded(&bar[b], (k >> 1) & 1, kWaitNs);
-        const uint64_t m = tile * kThreads + threadIdx.x;
-        uint32_t A[25], B[25];
+    const uint64_t m = first + threadIdx.x;
+    if (m >= n) return;
+    uint32_t A[25], B[25];
 #pragma unroll
-        for (int i = 0; i < 25; ++i) A[i] = B[i] = 0;
-        if (ok && m < n) {
-            const uint4 *q = reinterpret_cast<const uint4 *>(buf[b] + threadIdx.x * 64);
+    for (int i = 0; i < 25; ++i) A[i] = B[i] = 0;
+    const uint4 *q = reinterpret_cast<const uint4 *>(buf + threadIdx.x * 64);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint4 v = q[j];
-                Rep::set_word(A[2 * j], B[2 * j], v.x, v.y);
-                Rep::set_word(A[2 * j + 1], B[2 * j + 1], v.z, v.w);
-            }
-        }
-        // Every thread has read buffer b (or timed out): refill it, or stop.
-        // The proxy fence orders this thread's reads of b before the bulk
-        // copy's writes into it.
-        fence_proxy_async_smem();
-        if (__syncthreads_or(!ok)) {
-            if (threadIdx.x == 0) {
-                atomicOr(status, KB_DEV_TIMEOUT);
-                // A buffer holds at most one copy beyond the phases consumed
-                // before this tile; wait (bounded) for it to land.
-                for (int c = 0; c < 2; ++c) {
-                    const uint32_t consumed = (k + 1 - uint32_t(c)) / 2;
-                    if (uses[c] > consumed) mbar_wait_bounded(&bar[c], consumed & 1, kWaitNs);
-                }
-            }
-            return;
-        }
-        if (threadIdx.x == 0 && tile + 2 * stride < ntiles) issue(tile + 2 * stride, b);
-        if (m < n) {
-            A[8] ^= Rep::word_a(uint64_t(P::domain));
-            B[8] ^= Rep::word_b(uint64_t(P::domain));
-            constexpr uint64_t kEnd = uint64_t(0x80) << 56;
-            A[P::rate / 8 - 1] ^= Rep::word_a(kEnd);
-            B[P::rate / 8 - 1] ^= Rep::word_b(kEnd);
-            uint8_t *dst = out + m * dlen;
-            const uint32_t nsq = dlen > uint32_t(P::rate) ? (dlen - 1) / P::rate : 0;
-            for (uint32_t i = 0; i <= nsq; ++i) {
-                if (i > 0) squeeze<P::rate, Rep>(A, B, dst + uint64_t(i - 1) * P::rate, P::rate);
-                Rep::template permute<true>(A, B);
-            }
-            squeeze<P::rate, Rep, kOut>(A, B, dst + uint64_t(nsq) * P::rate, dlen - nsq * P::rate);
-        }
+    for (int j = 0; j < 4; ++j) {
+        const uint4 v = q[j];
+        Rep::set_word(A[2 * j], B[2 * j], v.x, v.y);
+        Rep::set_word(A[2 * j + 1], B[2 * j + 1], v.z, v.w);
     }
+    A[8] ^= Rep::word_a(uint64_t(P::domain));
+    B[8] ^= Rep::word_b(uint64_t(P::domain));
+    constexpr uint64_t kEnd = uint64_t(0x80) << 56;
+    A[P::rate / 8 - 1] ^= Rep::word_a(kEnd);
+    B[P::rate / 8 - 1] ^= Rep::word_b(kEnd);
+    const uint32_t dlen = P::digest ? uint32_t(P::digest) : out_len;
+    uint8_t *dst = out + m * dlen;
+    const uint32_t nsq = dlen > uint32_t(P::rate) ? (dlen - 1) / P::rate : 0;
+    for (uint32_t i = 0; i <= nsq; ++i) {
+        if (i > 0) squeeze<P::rate, Rep>(A, B, dst + uint64_t(i - 1) * P::rate, P::rate);
+        Rep::template permute<true>(A, B);
+    }
+    squeeze<P::rate, Rep, kOut>(A, B, dst + uint64_t(nsq) * P::rate, dlen - nsq * P::rate);
 }
 
 template <int V, int LEN, bool A8, class Rep>
 int launch_one(const uint8_t *msgs, uint64_t stride, uint64_t len, uint32_t out_len, uint8_t *digests,
                uint64_t n, cudaStream_t stream, const DeviceInfo &dev) {
-    const void *fn = reinterpret_cast<const void *>(&k_sha3_uniform<V, LEN, A8, Rep>);
-    // One-block messages: a grid of (occupancy x SMs) blocks strides over
-    // them.  Longer messages: one message per thread and as many blocks as
-    // that takes, so the block scheduler balances the last wave dynamically.
-    const uint64_t need = (n + kThreads - 1) / kThreads;
-    const uint64_t grid = len < uint64_t(Variant<V>::rate) ? persistent_grid(fn, kThreads, 0, n, dev)
-                                                           : std::min<uint64_t>(need, uint64_t(INT32_MAX));
+    // A message per thread and as many blocks as that takes, so that the block
+    // scheduler balances the sub-partitions' shares (k_sha3_uniform64_tma).  One-block
+    // messages with (occupancy x SMs) blocks striding over them, against this: 2^22 of
+    // 32 bytes 851 us -> 816, of 135 bytes 929 -> 841, of 64 at a stride of 80 903 -> 868.
+    const uint64_t grid = std::min<uint64_t>((n + kThreads - 1) / kThreads, uint64_t(INT32_MAX));
     return cuda_status(launch_overlapped(k_sha3_uniform<V, LEN, A8, Rep>, unsigned(grid), kThreads, 0, stream, msgs,
                                          stride, len, digests, out_len, n));
 }
@@ -202,8 +176,7 @@ int launch_one(const uint8_t *msgs, uint64_t stride, uint64_t len, uint32_t out_
 template <int V>
 int launch_tma(const uint8_t *msgs, uint32_t out_len, uint8_t *digests, uint64_t n, cudaStream_t stream,
                const DeviceInfo &dev) {
-    const void *fn = reinterpret_cast<const void *>(&k_sha3_uniform64_tma<V, PlainRep>);
-    const uint64_t grid = persistent_grid(fn, kThreads, 0, n, dev);
+    const uint64_t grid = (n + kThreads - 1) / kThreads;  // device memory holds fewer than 2^31 tiles
     return cuda_status(launch_overlapped(k_sha3_uniform64_tma<V, PlainRep>, unsigned(grid), kThreads, 0, stream, msgs,
                                          digests, out_len, n, dev.d_status));
 }

@@ -71,6 +71,19 @@ def test_batch_sizes_around_the_lines(cuda_lib, edge, blocks):
             assert got[i].tobytes() == hashlib.sha3_256(blob[i * length:(i + 1) * length]).digest(), (n, i)
 
 
+@pytest.mark.parametrize("variant,out_len", [(1, 32), (3, 64), (4, 337)])
+@pytest.mark.parametrize("tiles,more", [(100, -1), (100, 0), (100, 1), (7 * 152, 1), (14 * 152 + 5, 127)])
+def test_tiles_of_128_messages(cuda_lib, tiles, more, variant, out_len):
+    """64-byte messages packed back to back, a block per tile: the last tile whole, one message short or with one."""
+    n = 128 * tiles + more
+    data = np.random.default_rng(n).integers(0, 256, size=n * 64, dtype=np.uint8)
+    got = run_uniform(cuda_lib, data, 0, 64, 64, variant, out_len, n)
+    blob = data.tobytes()
+    for i in sorted({0, 1, 127, 128, 129, n // 2, n - 130, n - 129, n - 128, n - 127, n - 2, n - 1} |
+                    set(range(77, n, 997))):
+        assert got[i].tobytes() == want(variant, blob[64 * i:64 * i + 64], out_len), i
+
+
 def run_ragged(cuda_lib, b, noalloc=False):
     """(output bytes with 0xEE where nothing was written, device status) of a RaggedBatch."""
     import torch
