@@ -16,24 +16,29 @@
 //   3. k_sha3_queue: a persistent grid; each warp takes a group of 32
 //      consecutive entries of the order with one atomic and hashes one
 //      message per thread.  Warps run messages of nearly equal cost.  The
-//      queue has two ends: on every SM sub-partition the warp in the lowest
-//      hardware slot takes groups from the costly end (the longest chains
-//      start first), the others from the cheap end.
+//      queue has two parts of equal work: on every SM sub-partition the warp in
+//      the lowest hardware slot starts with the costlier (the longest chains
+//      start first), the others with the cheaper; either goes on to the other's
+//      part when its own is handed out.  Both parts run longest first.
 //   k_sha3_lanes runs the first K entries of the order (the K costliest
 //   messages; K from the plan, or given) one warp per message, concurrently with
 //   the queue kernel, which covers the entries from K on: it is launched first and
 //   lets the queue kernel start as soon as its own blocks have.
 //
-// Why two ends.  Measured on GB300: when two warps of one sub-partition both
+// Why two parts.  Measured on GB300: when two warps of one sub-partition both
 // have ALU work ready, the one in the lower hardware warp slot (%warpid)
 // issues, and once blocks are prefetched a warp rarely stalls, so the other
-// warp only runs in its partner's gaps.  With one queue end, a long chain of
+// warp only runs in its partner's gaps.  With one queue, a long chain of
 // permutations that landed in a higher slot waited behind its partner's
 // stream of groups and finished milliseconds after everything else.  With two
-// ends the long chains go to the slots that issue first, and a warp in a
-// higher slot only ever holds a cheap group, which it can finish late without
-// a tail.  The order of the slots affects only speed: every group is taken
-// exactly once, whichever warp takes it.
+// parts the long chains go to the slots that issue first, a warp in a higher
+// slot starts with chains of half the work's median at most, and what is handed
+// out last, by then to every warp, is the cheapest, so the warps end together.
+// (With the higher slots going up from the cheapest group instead, the two met
+// in groups of middling cost: 2^20 messages log-uniform to 64 KiB 11.60 ms
+// against 11.21, 300,000 4.24 against 4.11.)  Three warps a sub-partition take
+// 11.28 and 4.66 ms, the chains of each being slower.  The order of the slots
+// affects only speed: every group is taken exactly once, whichever warp takes it.
 #pragma once
 
 #include <cstdint>
@@ -95,8 +100,9 @@ struct Control {
     uint32_t cursor[kBuckets];       // slots of each bucket in the order that are taken
     unsigned long long head;         // warp-per-message schedule: next entry of the order
     unsigned long long lane_head;    // hybrid: next of the first K entries (one warp each)
-    unsigned long long ends;         // queue: groups taken from the back (high 32 bits) and front (low)
+    unsigned long long ends;         // queue: groups taken from the cheaper part (high 32 bits) and the costlier (low)
     unsigned long long queue_start;  // queue: first entry of the order it covers (K)
+    unsigned long long queue_mid;    // queue: first entry of its cheaper part
     uint32_t slots[kSlotWords];      // queue: a byte per SM, a bit per group of four hardware warp slots in use
 };
 
@@ -195,6 +201,54 @@ __device__ __forceinline__ uint64_t plan_split(const uint32_t (&count)[kPer], ui
     return first_cut;  // where no bucket met the condition, every message gets a warp
 }
 
+// The entry where the queue kernel's cheaper part begins: entries [first, mid) have
+// half of the permutations of [first, n).  Where the line lies matters little between
+// 3/8 and 5/8 (2^20 messages log-uniform to 64 KiB 11.21 ms at each, 2^19 5.63 ms); at
+// 1/4 and 3/4 2^19 messages take 5.89, at 3/4 and 7/8 2^20 take 11.47 and 11.35.
+// Called as plan_split.
+__device__ __forceinline__ uint64_t plan_mid(const uint32_t (&count)[kPer], uint64_t before, uint64_t first) {
+    __shared__ unsigned long long skipped, mid;
+    if (threadIdx.x == 0) {
+        skipped = 0;
+        mid = first;
+    }
+    uint64_t work = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+        if (b >= 0) work += count[j] * bucket_cost(b);
+    }
+    uint64_t w;
+    const uint64_t all = block_exclusive_scan(work, w);
+    uint64_t m = before, u = w;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+        if (b >= 0 && count[j]) {
+            const uint64_t c = bucket_cost(b);
+            if (first > m && first <= m + count[j]) skipped = u + (first - m) * c;
+            m += count[j];
+            u += count[j] * c;
+        }
+    }
+    __syncthreads();
+    const uint64_t target = skipped + (all - skipped) / 2;
+    m = before;
+    u = w;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+        if (b >= 0 && count[j]) {
+            const uint64_t c = bucket_cost(b);
+            if (c && target > u && target <= u + count[j] * c) mid = m + (target - u + c - 1) / c;
+            m += count[j];
+            u += count[j] * c;
+        }
+    }
+    __syncthreads();
+    return mid;
+}
+
 // Tile sums to the messages' exclusive sums, for batches of so many tiles that each
 // block of k_scatter would take long to add up those before its own.
 constexpr uint64_t kSumTiles = 4096;
@@ -282,7 +336,11 @@ __global__ void __launch_bounds__(kScanThreads)
         if (base + j < n) order[start[key[j]] + rank[j]] = uint32_t(base + j);
     if (blockIdx.x == 0) {
         const uint64_t first = split == kAutoSplit ? plan_split(count, m0) : split;
-        if (threadIdx.x == 0) ctl->queue_start = first;
+        const uint64_t mid = plan_mid(count, m0, first);
+        if (threadIdx.x == 0) {
+            ctl->queue_start = first;
+            ctl->queue_mid = mid < first ? first : mid;
+        }
     }
 }
 
@@ -303,6 +361,7 @@ __global__ void __launch_bounds__(kThreads, MINB)
     const int lane = threadIdx.x & 31;
     const uint64_t start = ctl->queue_start;
     const unsigned long long ngroups = n > start ? (n - start + 31) / 32 : 0;
+    const unsigned long long nfront = min((unsigned long long)(ctl->queue_mid - start) / 32, ngroups);
     // Whether this warp is in the lowest hardware slot of its sub-partition that a
     // warp of this kernel holds: warps of k_sha3_lanes may sit below.
     bool front;
@@ -321,16 +380,18 @@ __global__ void __launch_bounds__(kThreads, MINB)
         }
         front = (__shfl_sync(0xffffffffu, held, 0) & 0xffu & (bit - 1)) == 0;
     }
-    for (;;) {
-        // One atomic on both ends: group g is taken at most once, from the
-        // front (g = f) or the back (g = ngroups - 1 - b), and the two ends
-        // never pass each other.
+    // One atomic per group; a warp that finds its part handed out goes on to the other.
+    for (int parts = 2; parts > 0;) {
         unsigned long long old = 0;
         if (lane == 0) old = atomicAdd(&ctl->ends, front ? 1ull : (1ull << 32));
         old = __shfl_sync(0xffffffffu, old, 0);
-        const unsigned long long f = old & 0xffffffffull, b = old >> 32;
-        if (f + b >= ngroups) break;
-        const uint64_t idx = start + (front ? f : ngroups - 1 - b) * 32 + lane;
+        const unsigned long long g = front ? old & 0xffffffffull : nfront + (old >> 32);
+        if (g >= (front ? nfront : ngroups)) {
+            front = !front;
+            --parts;
+            continue;
+        }
+        const uint64_t idx = start + g * 32 + lane;
         if (idx < n) {
             if constexpr (STAGE == kStageDirect) {
                 hash_ragged_message(msgs, offsets, lens, variants, out_lens, out_off, digests, order[idx], status);

@@ -175,6 +175,37 @@ def test_ragged_split_between_warps_and_threads(cuda_lib, n, long_len, long_ever
         assert err == 0 and got.tobytes() == want_ragged(b)
 
 
+@pytest.mark.parametrize("k", [-1, 0, 33, "most", "all"])  # messages that take a warp each; the queue has the rest
+@pytest.mark.parametrize("kind", ["equal", "empty", "one long", "one valid"])
+def test_queue_parts(cuda_lib, kind, k):
+    """The queue's costlier and cheaper part where costs tie, where one message is half of the work, and where most
+    messages have no cost."""
+    import torch
+
+    n = 21 * torch.cuda.get_device_properties(0).multi_processor_count + 7
+    lens = np.full(n, {"equal": 300, "one valid": 500}.get(kind, 0))
+    if kind == "one long":
+        lens[n // 3] = 50000
+    b = W.ragged_batch(n, seed=11, lens=lens, shake_out=(1, 90), gap=1)
+    if kind == "one valid":
+        b.variants[np.arange(n) != 1000] = 77
+    saved = cuda_lib.keccak_tune_get(cuda_lib.KB_TUNE_QUEUE_WARP_MESSAGES)
+    cuda_lib.keccak_tune_set(cuda_lib.KB_TUNE_QUEUE_WARP_MESSAGES, {"most": n - 31, "all": n}.get(k, k))
+    try:
+        got, err = run_ragged(cuda_lib, b)
+    finally:
+        cuda_lib.keccak_tune_set(cuda_lib.KB_TUNE_QUEUE_WARP_MESSAGES, saved)
+    if kind == "one valid":
+        assert err == cuda_lib.KB_DEV_BAD_VARIANT
+        at, size = int(b.out_offsets()[1000]), int(b.out_lens[1000])
+        o = int(b.offsets[1000])
+        assert got[at:at + size].tobytes() == want(int(b.variants[1000]), b.msgs.tobytes()[o:o + 500], size)
+        got[at:at + size] = 0xEE
+        assert (got == 0xEE).all()
+    else:
+        assert err == 0 and got.tobytes() == want_ragged(b)
+
+
 def tree_nodes(leaves):
     nodes = level = [hashlib.sha3_256(b"\x00" + leaf).digest() for leaf in leaves]
     while len(level) > 1:
