@@ -87,66 +87,48 @@ __device__ __forceinline__ void small_round(uint32_t (&A)[25], int ir) {
 // each warp takes tiles of 32 consecutive 200-byte states (6.4 KB), copied
 // with coalesced 8-byte accesses (the warp touches 256 contiguous bytes per
 // access), and each thread then reads its own state from shared memory.
-// Every warp has two tile buffers of its own: the next tile's copies
-// (cp.async, 8 bytes each) are issued before the current tile is permuted,
-// so a warp's loads overlap its own arithmetic, and warps synchronise only
-// among their own threads (tiles of 128 states per block, with block
-// barriers, measured 5-10% slower).  Reading the states straight from
-// global memory, each thread 25 accesses 200 bytes apart, left the
-// reduced-round runs waiting on memory.
+// A warp takes one tile and ends; the SM's other warps compute while its copies
+// (cp.async, 8 bytes each) are in flight, and warps synchronise only among their
+// own threads.  Reading the states straight from global memory, each thread 25
+// accesses 200 bytes apart, leaves the reduced rounds waiting on memory.  2^22
+// states: 12 rounds of width 1600 463 us, 4 rounds 250, 18 rounds of width 200 397;
+// with two buffers a warp in a grid that strides over the tiles, which is half the
+// warps per SM and equal shares (k_sha3_uniform64_tma says why those end late), 501,
+// 303 and 422.  What is left of the 4 rounds is HBM's (1.68 GB, 251 us at the
+// measured copy rate).
 constexpr uint32_t kWarpTile = 32;                                   // states per warp tile
 constexpr uint32_t kTileWords = kWarpTile * 25;                      // uint2 words of a tile (6.4 KB)
-constexpr size_t kTileSmem = size_t(kThreads / 32) * 2 * kTileWords * sizeof(uint2);  // per block
+constexpr size_t kTileSmem = size_t(kThreads / 32) * kTileWords * sizeof(uint2);  // per block
 
-// The warp tiles of this warp, one warp-stride apart over the grid, each
-// permuted state by state by f(uint2 *state) in shared memory and written
-// back in place.
+// This warp's tile, permuted state by state by f(uint2 *state) in shared memory
+// and written back in place.
 template <class F>
-__device__ __forceinline__ void run_tiles(uint64_t *states, uint64_t n, uint2 *sm, F f) {
+__device__ __forceinline__ void run_tile(uint64_t *states, uint64_t n, uint2 *sm, F f) {
     const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
-    const uint64_t ntiles = (n + kWarpTile - 1) / kWarpTile;
-    const uint64_t nwarps = uint64_t(gridDim.x) * (blockDim.x / 32);
-    uint64_t tile = uint64_t(blockIdx.x) * (blockDim.x / 32) + wib;
-    uint2 *mine = sm + wib * 2 * kTileWords;
-    const uint32_t sbase = static_cast<uint32_t>(__cvta_generic_to_shared(mine));
-    auto count = [&](uint64_t t) {
-        return uint32_t(n - t * kWarpTile < kWarpTile ? n - t * kWarpTile : uint64_t(kWarpTile));
-    };
-    auto load = [&](uint32_t sdst, uint64_t t) {
-        const uint2 *src = reinterpret_cast<const uint2 *>(states + 25 * t * kWarpTile);
-        const uint32_t words = count(t) * 25;
-        for (uint32_t j = lane; j < words; j += 32)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sdst + 8 * j), "l"(src + j) : "memory");
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
+    const uint64_t first = (uint64_t(blockIdx.x) * (blockDim.x / 32) + wib) * kWarpTile;
     launch_wait();
-    if (tile >= ntiles) return;
-    load(sbase, tile);
-    for (uint32_t b = 0; tile < ntiles; tile += nwarps, b ^= 1u) {
-        const uint64_t next = tile + nwarps;
-        // The other buffer was last read before the warp barrier that ended
-        // the previous pass, so the next tile may be copied into it now.
-        if (next < ntiles) load(sbase + (b ^ 1u) * kTileWords * 8u, next);
-        else asm volatile("cp.async.commit_group;" ::: "memory");  // an empty group keeps the count below uniform
-        asm volatile("cp.async.wait_group 1;" ::: "memory");         // this tile's copies have landed
-        __syncwarp();
-        uint2 *cur = mine + b * kTileWords;
-        const uint32_t cnt = count(tile);
-        if (lane < cnt) f(cur + 25 * lane);
-        __syncwarp();
-        uint2 *dst = reinterpret_cast<uint2 *>(states + 25 * tile * kWarpTile);
-        for (uint32_t j = lane; j < cnt * 25; j += 32) dst[j] = cur[j];
-        __syncwarp();
-    }
+    if (first >= n) return;
+    const uint32_t cnt = uint32_t(n - first < kWarpTile ? n - first : uint64_t(kWarpTile));
+    uint2 *mine = sm + wib * kTileWords;
+    uint2 *g = reinterpret_cast<uint2 *>(states + 25 * first);
+    const uint32_t sbase = static_cast<uint32_t>(__cvta_generic_to_shared(mine));
+    for (uint32_t j = lane; j < cnt * 25; j += 32)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sbase + 8 * j), "l"(g + j) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
     asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    if (lane < cnt) f(mine + 25 * lane);
+    __syncwarp();
+    for (uint32_t j = lane; j < cnt * 25; j += 32) g[j] = mine[j];
 }
 
+// (At 7 blocks per SM 18 rounds of width 200 take 397 us, 407 with registers to spare.)
 template <int W>
-__global__ void __launch_bounds__(kThreads) k_keccak_p_small(uint64_t *states, int first_ir, int nr, uint64_t n) {
+__global__ void __launch_bounds__(kThreads, 7) k_keccak_p_small(uint64_t *states, int first_ir, int nr, uint64_t n) {
     using L = SmallLanes<W>;
     extern __shared__ uint2 sm[];
     const int ir0 = ((first_ir % 255) + 255) % 255;  // rc has period 255 (Algorithm 5)
-    run_tiles(states, n, sm, [&](uint2 *s) {
+    run_tile(states, n, sm, [&](uint2 *s) {
         uint32_t A[25];
 #pragma unroll
         for (int k = 0; k < 25; ++k) A[k] = L::load(s[k].x);
@@ -167,7 +149,7 @@ __device__ __forceinline__ void p1600_round(uint32_t (&L)[25], uint32_t (&H)[25]
     plain_round_body(L, H, NL, NH);
     const uint64_t rc = c_rc255.v[ir];
     NL[0] ^= uint32_t(rc);
-    NH[0] ^= uint32_t(rc >> 32);
+    NH[0] += uint32_t(rc >> 32);  // bit 31 alone or nothing: the sum is the XOR, off the ALU pipe
 #pragma unroll
     for (int k = 0; k < 25; ++k) {
         L[k] = NL[k];
@@ -208,7 +190,7 @@ template <bool STAGED>
 __global__ void __launch_bounds__(kThreads) k_keccak_p_1600(uint64_t *states, int first_ir, int nr, uint64_t n) {
     if constexpr (STAGED) {
         extern __shared__ uint2 sm[];
-        run_tiles(states, n, sm, [&](uint2 *s) {
+        run_tile(states, n, sm, [&](uint2 *s) {
             uint32_t L[25], H[25];
 #pragma unroll
             for (int k = 0; k < 25; ++k) {
@@ -269,20 +251,15 @@ __global__ void __launch_bounds__(32) k_keccak_p_1600_coop(uint64_t *states, int
     }
 }
 
-// Launches a tiled kernel with its two tile buffers (above the 48 KB a block
-// gets without opting in).
 template <class K>
-int launch_tiled(K kernel, uint64_t *states, int first_ir, int nr, uint64_t n, cudaStream_t stream,
-                 const DeviceInfo &dev) {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTileSmem)) != cudaSuccess)
-        return cuda_status(cudaGetLastError());
-    const uint64_t g = persistent_grid(reinterpret_cast<const void *>(kernel), kThreads, kTileSmem, n, dev);
-    return cuda_status(launch_overlapped(kernel, unsigned(g), kThreads, kTileSmem, stream, states, first_ir, nr, n));
+int launch_tiled(K kernel, uint64_t *states, int first_ir, int nr, uint64_t n, cudaStream_t stream) {
+    const uint64_t grid = (n + kThreads - 1) / kThreads;  // 2^31 blocks would be 55 TB of states
+    return cuda_status(launch_overlapped(kernel, unsigned(grid), kThreads, kTileSmem, stream, states, first_ir, nr, n));
 }
 
 template <int W>
 int launch_small(uint64_t *states, int first_ir, int nr, uint64_t n, cudaStream_t stream, const DeviceInfo &dev) {
-    return launch_tiled(k_keccak_p_small<W>, states, first_ir, nr, n, stream, dev);
+    return launch_tiled(k_keccak_p_small<W>, states, first_ir, nr, n, stream);
 }
 
 }  // namespace
@@ -304,10 +281,10 @@ int launch_keccak_p(uint64_t *states, int b, int nr, uint64_t n, cudaStream_t st
             if (first_ir >= 0 && n <= kCoopPerSm * uint64_t(dev.sm_count > 0 ? dev.sm_count : 1))
                 return cuda_status(
                     launch_overlapped(k_keccak_p_1600_coop, unsigned(n), 32, 0, stream, states, first_ir, nr));
-            // Staged through shared memory below 16 rounds (measured on 2^24
-            // states: 12 rounds 2.53 ms read directly, 2.15 ms staged; 24
-            // rounds 3.84 ms directly, 4.02 ms staged).
-            if (nr < 16) return launch_tiled(k_keccak_p_1600<true>, states, first_ir, nr, n, stream, dev);
+            // Staged through shared memory below 16 rounds (2^22 states: 12 rounds
+            // 574 us read directly, 463 staged; 14 rounds 560 and 532; 18 rounds
+            // 647 and 669; 24 rounds 839 and 875).
+            if (nr < 16) return launch_tiled(k_keccak_p_1600<true>, states, first_ir, nr, n, stream);
             const uint64_t g = std::min<uint64_t>((n + kThreads - 1) / kThreads, uint64_t(INT32_MAX));
             return cuda_status(
                 launch_overlapped(k_keccak_p_1600<false>, unsigned(g), kThreads, 0, stream, states, first_ir, nr, n));

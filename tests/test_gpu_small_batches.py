@@ -323,6 +323,30 @@ def test_stream_refusals_in_both_forms(cuda_lib):
     assert seen[0] == seen[1] and seen[0][0][0] == cuda_lib.KB_DEV_BAD_VARIANT
 
 
+@pytest.mark.parametrize("b,nr", [(25, 12), (200, 18), (800, 22), (1600, 3)])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 127, 129, 7 * 128 * 152 + 33])
+def test_keccak_p_tiles(cuda_lib, b, nr, n):
+    """The staged kernels at the edges of a warp's and a block's tile: the same results in reverse order (so every state
+    at another place), the first and the last against the oracle, and the state past the last one untouched."""
+    import torch
+
+    import oracle
+
+    w = b // 25
+    given = np.random.default_rng(b + n).integers(0, 1 << 64, size=(n + 1, 25), dtype=np.uint64) >> np.uint64(64 - w)
+    states = torch.from_numpy(given.view(np.int64)).cuda()
+    turned = states[:n].flip(0).contiguous()
+    cuda_lib.keccak_p_batch(states, b, nr, n)
+    cuda_lib.keccak_p_batch(turned, b, nr, n)
+    assert torch.equal(states[:n], turned.flip(0))
+    got = states.cpu().numpy().view(np.uint64)
+    assert (got[n] == given[n]).all()
+    for i in {0, n - 1}:
+        bits = np.array([(int(v) >> z) & 1 for v in given[i] for z in range(w)], dtype=np.uint8)
+        lanes = oracle.keccak_p(b, nr, bits).reshape(25, w)
+        assert [sum(int(x) << z for z, x in enumerate(lane)) for lane in lanes] == [int(v) for v in got[i]], i
+
+
 @pytest.mark.parametrize("nr", [1, 2, 11, 12, 24, 25])
 @pytest.mark.parametrize("per_sm,more", [(0, 1), (0, 5), (12, 0), (12, 1)])
 def test_keccak_p_around_the_line(cuda_lib, per_sm, more, nr):
