@@ -518,9 +518,9 @@ void keccak_release(void);
 #define KB_HOST_PATH_ZERO_COPY 2
 /*   KB_TUNE_STAGING: how the fixed-stride kernel reads 64-byte messages packed
  *     back to back (stride 64, 16-byte aligned, device memory) --
- *     KB_STAGING_TMA (default: bulk asynchronous copies of 8 KiB tiles into
- *     shared memory, two deep, then each thread reads its message from there;
- *     measured ~0.8% faster) or KB_STAGING_DIRECT (each thread loads its
+ *     KB_STAGING_TMA (default: a bulk asynchronous copy of an 8 KiB tile
+ *     into shared memory per block, then each thread reads its message from
+ *     there; measured 9% faster) or KB_STAGING_DIRECT (each thread loads its
  *     message with four 16-byte loads; the measured control).  Other shapes,
  *     and host-mapped buffers, always load directly. */
 #define KB_TUNE_STAGING 7

@@ -191,9 +191,12 @@ __device__ __forceinline__ uint32_t shl_pair_mul(uint32_t lo, uint32_t hi) {
 // (theta's 1 and rho's 1, 2, 3, 6, 8, 10, 36, 39, 41 and 43), by funnel shifts
 // otherwise.  A round then has 149 ALU instructions and 96 multiplies instead
 // of 180 and none: 361 -> 328 cycles a warp and sub-partition in the looped
-// permutation.  It does not reach the ALU's 298: the register file's read
-// ports bind next (a multiply with two register operands beside three-operand
-// LOP3s costs 0.45 cycles).  So the line lies at 11: offsets of 9..11 cost
+// permutation (333 and 324 on a later build, with equal shares a warp and with work
+// handed out in small units).  It does not reach the ALU's 298: a multiply with two
+// register operands beside three-operand LOP3s costs 0.45 cycles of the register
+// file's read ports.  (Fewer reads for ten more instructions, theta's D computed once
+// and two-operand XORs, lose: 350, or 336 to 348 for some columns, against 331.)  So
+// the line lies at 11: offsets of 9..11 cost
 // five register reads a word and still pay (335 -> 328), 12 and 13 lose
 // (336), all up to 15 more (339); bit reversals on the otherwise idle XU pipe
 // for the offsets near 32 lose as well (330 -> 334..347).
