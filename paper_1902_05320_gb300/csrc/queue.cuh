@@ -104,7 +104,26 @@ struct Control {
     unsigned long long queue_start;  // queue: first entry of the order it covers (K)
     unsigned long long queue_mid;    // queue: first entry of its cheaper part
     uint32_t slots[kSlotWords];      // queue: a byte per SM, a bit per group of four hardware warp slots in use
+    uint32_t ready;                  // 1: k_sha3_lanes has seen the end of k_scatter
 };
+
+// The hand-off from k_scatter to a k_sha3_queue that starts beside k_sha3_lanes.
+// griddepcontrol.wait covers the kernel before (k_sha3_lanes), whose end the queue
+// kernel must not wait for; that kernel's own wait makes k_scatter's writes visible
+// to itself alone.  So a thread of k_sha3_lanes that has waited releases a flag and
+// every thread of the queue kernel acquires it.
+__device__ __forceinline__ void hand_over(uint32_t *flag) {
+    asm volatile("st.release.gpu.b32 [%0], %1;" ::"l"(flag), "r"(1u) : "memory");
+}
+// False where the flag is not seen within some tens of microseconds (it is set before
+// the last block of k_sha3_lanes lets the queue kernel start, so it is there or on its
+// way): the caller then waits for the whole of k_sha3_lanes.
+__device__ __forceinline__ bool taken_over(const uint32_t *flag) {
+    uint32_t v = 0;
+    for (int i = 0; i < 64 && v == 0; ++i)
+        asm volatile("ld.acquire.gpu.b32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
+    return v != 0;
+}
 
 template <bool BY_VARIANT>
 __global__ void __launch_bounds__(kScanThreads)
@@ -346,19 +365,21 @@ __global__ void __launch_bounds__(kScanThreads)
 
 // The persistent queue kernel: one thread per message, 32 messages per
 // dequeue.  STAGE picks how blocks are read and the permutation's form
-// (kStage* | kLooped).
+// (kStage* | kLooped).  `beside`: launched to run beside k_sha3_lanes.  No pointer is
+// __restrict__: loads of what k_scatter wrote stay behind the hand-off.
 template <int MINB, int STAGE>
 __global__ void __launch_bounds__(kThreads, MINB)
-    k_sha3_queue(const uint8_t *__restrict__ msgs, const uint64_t *__restrict__ offsets,
-                 const uint64_t *__restrict__ lens, const uint8_t *__restrict__ variants,
-                 const uint32_t *__restrict__ out_lens, const uint64_t *__restrict__ out_off,
-                 const uint32_t *__restrict__ order, uint8_t *__restrict__ digests, uint64_t n, Control *ctl,
-                 unsigned int *status) {
+    k_sha3_queue(const uint8_t *msgs, const uint64_t *offsets,
+                 const uint64_t *lens, const uint8_t *variants,
+                 const uint32_t *out_lens, const uint64_t *out_off,
+                 const uint32_t *order, uint8_t *digests, uint64_t n, Control *ctl,
+                 unsigned int *status, bool beside) {
     static_assert(kThreads == 128, "the stage layout assumes 128 threads per block");
     constexpr int kRead = STAGE & 3;
     constexpr bool kLoop = (STAGE & kLooped) != 0;
     __shared__ uint32_t stage_mem[kRead == kStageAsync ? 2 * kStageWords * kThreads : 1];
     const int lane = threadIdx.x & 31;
+    if (beside && !taken_over(&ctl->ready)) launch_wait();
     const uint64_t start = ctl->queue_start;
     const unsigned long long ngroups = n > start ? (n - start + 31) / 32 : 0;
     const unsigned long long nfront = min((unsigned long long)(ctl->queue_mid - start) / 32, ngroups);

@@ -54,6 +54,8 @@ __global__ void __launch_bounds__(32)
                  unsigned int *status) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     launch_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) hand_over(&ctl->ready);
+    __syncwarp();
     const uint64_t limit = all || ctl->queue_start > n ? n : ctl->queue_start;
     unsigned long long *head = all ? &ctl->head : &ctl->lane_head;
     if (limit == 0) return;
@@ -265,10 +267,11 @@ int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *le
     const void *fn = queue_kernel(cfg.minb, cfg.stage);
     if (!fn) return KB_ERR_INVALID;
     Control *ctl = bf.ctl;
+    bool beside = split != 0;
     void *args[] = {&msgs, &offsets, &lens, &variants, &out_lens, const_cast<uint64_t **>(&bf.out_off),
-                    const_cast<uint32_t **>(&bf.order), &digests, &n, &ctl, &status};
+                    const_cast<uint32_t **>(&bf.order), &digests, &n, &ctl, &status, &beside};
     // Beside k_sha3_lanes: both need k_scatter alone, and the blocks of k_sha3_lanes
-    // let this kernel start (or exit) only after they have seen that end.
+    // let this kernel start (or exit) only after they have seen that end (hand_over).
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -277,7 +280,7 @@ int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *le
     lc.blockDim = dim3(kThreads);
     lc.stream = stream;
     lc.attrs = &attr;
-    lc.numAttrs = split != 0 ? 1 : 0;
+    lc.numAttrs = beside ? 1 : 0;
     return cuda_status(cudaLaunchKernelExC(&lc, fn, args));
 }
 
