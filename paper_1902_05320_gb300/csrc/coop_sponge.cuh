@@ -26,9 +26,9 @@ __device__ __forceinline__ RawWord ld_raw(const uint8_t *q, int64_t left) {
     const uint32_t o = uint32_t(start & 3);
     const uint32_t n = left >= 8 ? 8u : left > 0 ? uint32_t(left) : 0u;
     RawWord r;
-    r.w0 = n ? __ldg(a) : 0u;
-    r.w1 = o + n > 4 ? __ldg(a + 1) : 0u;
-    r.w2 = o + n > 8 ? __ldg(a + 2) : 0u;
+    r.w0 = n ? *a : 0u;
+    r.w1 = o + n > 4 ? a[1] : 0u;
+    r.w2 = o + n > 8 ? a[2] : 0u;
     return r;
 }
 
@@ -68,14 +68,14 @@ __device__ __forceinline__ void coop_full_blocks(const Coop &c, uint32_t (&a)[2]
         a[0] ^= e[0];
         a[1] ^= e[1];
         if (have0) {
-            r0.w0 = __ldg(q0);
-            r0.w1 = __ldg(q0 + 1);
-            if (sh) r0.w2 = __ldg(q0 + 2);
+            r0.w0 = *q0;
+            r0.w1 = q0[1];
+            if (sh) r0.w2 = q0[2];
         }
         if (have1) {
-            r1.w0 = __ldg(q1);
-            r1.w1 = __ldg(q1 + 1);
-            if (sh) r1.w2 = __ldg(q1 + 2);
+            r1.w0 = *q1;
+            r1.w1 = q1[1];
+            if (sh) r1.w2 = q1[2];
         }
         q0 += step;
         q1 += step;

@@ -91,8 +91,8 @@ __device__ __forceinline__ void leaf_state_a8(const uint8_t *p, uint64_t leaf_by
 }
 
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
-    k_merkle_leaves_a8(const uint8_t *__restrict__ buf, uint64_t n_leaves, uint64_t leaf_bytes,
-                       uint8_t *__restrict__ out) {
+    k_merkle_leaves_a8(const uint8_t *buf, uint64_t n_leaves, uint64_t leaf_bytes,
+                       uint8_t *out) {
     launch_wait();
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n_leaves; i += step) {
@@ -132,11 +132,11 @@ __device__ __forceinline__ void absorb_leaf_block_any(uint32_t (&A)[25], uint32_
     const uint32_t *a = reinterpret_cast<const uint32_t *>(start & ~uintptr_t(3));
     const uint32_t sh = uint32_t(start & 3) * 8;
     if (full) {
-        uint32_t prev = __ldg(a);
+        uint32_t prev = *a;
 #pragma unroll
         for (int k = 1; k < kRate / 8; ++k) {
-            const uint32_t w1 = __ldg(a + 2 * k - 1);
-            const uint32_t w2 = (k + 1 < kRate / 8 || sh != 0) ? __ldg(a + 2 * k) : 0u;
+            const uint32_t w1 = a[2 * k - 1];
+            const uint32_t w2 = (k + 1 < kRate / 8 || sh != 0) ? a[2 * k] : 0u;
             PlainRep::xor_word(A[k], B[k], __funnelshift_r(prev, w1, sh), __funnelshift_r(w1, w2, sh));
             prev = w2;
         }
@@ -145,11 +145,11 @@ __device__ __forceinline__ void absorb_leaf_block_any(uint32_t (&A)[25], uint32_
         const uint32_t left = rem > 8 ? rem - 8 : 0u;
         const uint32_t nw = left ? uint32_t(((start + left - 1) >> 2) - (start >> 2)) + 1 : 0u;
         int rb = int(8 * rem) - 64;  // message bits still to come, from lane k on
-        uint32_t prev = nw ? __ldg(a) : 0u;
+        uint32_t prev = nw ? *a : 0u;
 #pragma unroll
         for (int k = 1; k < kRate / 8; ++k) {
-            const uint32_t w1 = uint32_t(2 * k - 1) < nw ? __ldg(a + 2 * k - 1) : 0u;
-            const uint32_t w2 = uint32_t(2 * k) < nw ? __ldg(a + 2 * k) : 0u;
+            const uint32_t w1 = uint32_t(2 * k - 1) < nw ? a[2 * k - 1] : 0u;
+            const uint32_t w2 = uint32_t(2 * k) < nw ? a[2 * k] : 0u;
             uint32_t vl = __funnelshift_r(prev, w1, sh), vh = __funnelshift_r(w1, w2, sh);
             prev = w2;
             vl &= __funnelshift_lc(0xFFFFFFFFu, 0u, uint32_t(max(rb, 0)));
@@ -164,8 +164,8 @@ __device__ __forceinline__ void absorb_leaf_block_any(uint32_t (&A)[25], uint32_
 }
 
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
-    k_merkle_leaves_any(const uint8_t *__restrict__ buf, uint64_t n_leaves, uint64_t leaf_bytes,
-                        uint8_t *__restrict__ out) {
+    k_merkle_leaves_any(const uint8_t *buf, uint64_t n_leaves, uint64_t leaf_bytes,
+                        uint8_t *out) {
     launch_wait();
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
     const uint64_t vlen = leaf_bytes + 1;
@@ -253,7 +253,7 @@ __device__ __forceinline__ void load_node_block(uint32_t (&A)[25], uint32_t (&B)
 // Few leaves: one warp each (coop_sponge.cuh), which takes a third of the time of a
 // thread for a leaf's chain of permutations.
 __global__ void __launch_bounds__(32)
-    k_merkle_leaves_coop(const uint8_t *__restrict__ buf, uint64_t leaf_bytes, uint8_t *__restrict__ out) {
+    k_merkle_leaves_coop(const uint8_t *buf, uint64_t leaf_bytes, uint8_t *out) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     const Coop c(mem);
     const uint64_t i = blockIdx.x;

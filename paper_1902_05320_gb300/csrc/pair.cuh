@@ -91,8 +91,8 @@ __device__ __forceinline__ uint32_t ld_u32_any(const uint8_t *p, uint32_t nvalid
     const uintptr_t start = reinterpret_cast<uintptr_t>(p);
     const uint32_t *a = reinterpret_cast<const uint32_t *>(start & ~uintptr_t(3));
     const uint32_t o = uint32_t(start & 3);
-    const uint32_t w0 = __ldg(a);
-    const uint32_t w1 = o + nvalid > 4 ? __ldg(a + 1) : 0u;
+    const uint32_t w0 = *a;
+    const uint32_t w1 = o + nvalid > 4 ? a[1] : 0u;
     const uint32_t v = __funnelshift_r(w0, w1, 8 * o);
     return nvalid < 4 ? v & ((1u << (8 * nvalid)) - 1u) : v;
 }
@@ -130,7 +130,7 @@ __device__ __forceinline__ void pair_one_block(bool active, const uint8_t *p, ui
         S[k] = 0;
         if (k >= RATE / 8) continue;
         if (uint32_t(8 * k + 8) <= len) {
-            if (active) S[k] = __funnelshift_r(__ldg(w + 2 * k), o ? __ldg(w + 2 * k + 1) : 0u, 8 * o);
+            if (active) S[k] = __funnelshift_r(w[2 * k], o ? w[2 * k + 1] : 0u, 8 * o);
         } else if (uint32_t(8 * k) <= len) {
             const uint32_t at = 8 * k + 4 * h, left = len > at ? len - at : 0;
             if (active) S[k] = ld_u32_any(p + at, left < 4 ? left : 4u);
@@ -163,8 +163,8 @@ __device__ __forceinline__ void pair_sponge(bool active, const uint8_t *p, uint6
         const uint32_t *q = reinterpret_cast<const uint32_t *>((reinterpret_cast<uintptr_t>(p) & ~uintptr_t(3)) +
                                                                i * RATE) + h;
 #pragma unroll
-        for (int k = 0; k < kWords; ++k) w[k] = active ? __ldg(q + 2 * k) : 0u;
-        w[kWords] = active && sh && h == 0 ? __ldg(q + 2 * kWords) : 0u;
+        for (int k = 0; k < kWords; ++k) w[k] = active ? q[2 * k] : 0u;
+        w[kWords] = active && sh && h == 0 ? q[2 * kWords] : 0u;
     };
     const bool unaligned = __any_sync(0xffffffffu, sh != 0);
     if (nfull) fetch(0);

@@ -127,8 +127,8 @@ __device__ __forceinline__ bool taken_over(const uint32_t *flag) {
 
 template <bool BY_VARIANT>
 __global__ void __launch_bounds__(kScanThreads)
-    k_prep(const uint64_t *__restrict__ lens, const uint8_t *__restrict__ variants,
-           const uint32_t *__restrict__ out_lens, uint64_t n, uint64_t *__restrict__ tile_sums, Control *ctl) {
+    k_prep(const uint64_t *lens, const uint8_t *variants,
+           const uint32_t *out_lens, uint64_t n, uint64_t *tile_sums, Control *ctl) {
     __shared__ uint32_t hist[kBuckets];
     launch_next();
     for (int b = threadIdx.x; b < kBuckets; b += blockDim.x) hist[b] = 0;
@@ -291,9 +291,9 @@ static __global__ void __launch_bounds__(kScanThreads) k_plan_tiles(uint64_t *ti
 // launch of one block for that in between took 9 to 11 us.
 template <bool BY_VARIANT>
 __global__ void __launch_bounds__(kScanThreads)
-    k_scatter(const uint64_t *__restrict__ lens, const uint8_t *__restrict__ variants,
-              const uint32_t *__restrict__ out_lens, uint64_t n, const uint64_t *__restrict__ tile_sums,
-              uint64_t ntiles, uint64_t *__restrict__ out_off, uint32_t *__restrict__ order, Control *ctl,
+    k_scatter(const uint64_t *lens, const uint8_t *variants,
+              const uint32_t *out_lens, uint64_t n, const uint64_t *tile_sums,
+              uint64_t ntiles, uint64_t *out_off, uint32_t *order, Control *ctl,
               uint64_t split) {
     __shared__ uint32_t hist[kBuckets];
     __shared__ uint32_t start[kBuckets];

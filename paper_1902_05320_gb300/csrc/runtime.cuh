@@ -83,7 +83,8 @@ cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned bloc
 // blocks of 128 threads, call after call: 45 us each became 137).
 __device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // Returns when every earlier kernel of the stream has ended and its writes are
-// visible; at once in a plain launch.
+// visible; at once in a plain launch.  Only plain loads stay behind it: no kernel that
+// calls it has __restrict__ parameters or read-only loads.
 __device__ __forceinline__ void launch_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 #endif
 

@@ -47,10 +47,10 @@ namespace kb {
 // entries of the order or over those before the queue kernel's first, taken one at
 // a time; one warp per block, so that the warps spread over the SMs.
 __global__ void __launch_bounds__(32)
-    k_sha3_lanes(const uint8_t *__restrict__ msgs, const uint64_t *__restrict__ offsets,
-                 const uint64_t *__restrict__ lens, const uint8_t *__restrict__ variants,
-                 const uint32_t *__restrict__ out_lens, const uint64_t *__restrict__ out_off,
-                 const uint32_t *__restrict__ order, uint8_t *__restrict__ digests, uint64_t n, bool all, Control *ctl,
+    k_sha3_lanes(const uint8_t *msgs, const uint64_t *offsets,
+                 const uint64_t *lens, const uint8_t *variants,
+                 const uint32_t *out_lens, const uint64_t *out_off,
+                 const uint32_t *order, uint8_t *digests, uint64_t n, bool all, Control *ctl,
                  unsigned int *status) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     launch_wait();
@@ -85,9 +85,9 @@ __global__ void __launch_bounds__(32)
 // 200 messages of up to 600 bytes, of which the hashing's chain of nine
 // permutations is 14 on this form.
 __global__ void __launch_bounds__(32)
-    k_sha3_ragged_coop(const uint8_t *__restrict__ msgs, const uint64_t *__restrict__ offsets,
-                       const uint64_t *__restrict__ lens, const uint8_t *__restrict__ variants,
-                       const uint32_t *__restrict__ out_lens, uint8_t *__restrict__ digests, unsigned int *status) {
+    k_sha3_ragged_coop(const uint8_t *msgs, const uint64_t *offsets,
+                       const uint64_t *lens, const uint8_t *variants,
+                       const uint32_t *out_lens, uint8_t *digests, unsigned int *status) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     const uint32_t i = blockIdx.x, lane = threadIdx.x;
     const Coop c(mem);

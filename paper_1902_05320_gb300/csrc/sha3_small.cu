@@ -15,8 +15,8 @@ namespace {
 // permutation instead of 1.55: the warps of an SM share one path to its shared
 // memory.)
 __global__ void __launch_bounds__(32)
-    k_sha3_uniform_coop(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len, int variant,
-                        uint8_t *__restrict__ out, uint32_t out_len) {
+    k_sha3_uniform_coop(const uint8_t *msgs, uint64_t stride, uint64_t len, int variant,
+                        uint8_t *out, uint32_t out_len) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     const Coop c(mem);
     const uint64_t m = blockIdx.x;
@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(32)
 
 template <int V>
 __global__ void __launch_bounds__(kThreads)
-    k_sha3_uniform_pair(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len, uint8_t *__restrict__ out,
+    k_sha3_uniform_pair(const uint8_t *msgs, uint64_t stride, uint64_t len, uint8_t *out,
                         uint32_t out_len, uint64_t n) {
     const uint64_t m = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 1;
     launch_wait();
@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kThreads)
 // output's lanes of the last round.
 template <int V>
 __global__ void __launch_bounds__(kThreads)
-    k_sha3_uniform_pair_one(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len, uint8_t *__restrict__ out,
+    k_sha3_uniform_pair_one(const uint8_t *msgs, uint64_t stride, uint64_t len, uint8_t *out,
                             uint32_t out_len, uint64_t n) {
     using P = Variant<V>;
     const uint64_t m = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 1;
@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kThreads)
 // (keccak_core.cuh).
 template <int V, bool MUL>
 __global__ void __launch_bounds__(kThreads, 2)
-    k_sha3_uniform_thin(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len, uint8_t *__restrict__ out,
+    k_sha3_uniform_thin(const uint8_t *msgs, uint64_t stride, uint64_t len, uint8_t *out,
                         uint32_t out_len, uint64_t n) {
     using P = Variant<V>;
     constexpr int kWords = P::rate / 4;
@@ -73,8 +73,8 @@ __global__ void __launch_bounds__(kThreads, 2)
         const uint32_t *a = reinterpret_cast<const uint32_t *>((reinterpret_cast<uintptr_t>(p) & ~uintptr_t(3)) +
                                                                i * P::rate);
 #pragma unroll
-        for (int k = 0; k < kWords; ++k) w[k] = __ldg(a + k);
-        w[kWords] = sh ? __ldg(a + kWords) : 0u;
+        for (int k = 0; k < kWords; ++k) w[k] = a[k];
+        w[kWords] = sh ? a[kWords] : 0u;
     };
     if (nfull) fetch(0);
     for (uint64_t i = 0; i <= nfull + nsq; ++i) {

@@ -40,8 +40,8 @@ constexpr int kStagedMinBlocks = 7;
 // of 8 (16 when LEN == 64).
 template <int V, int LEN, bool A8, class Rep>
 __global__ void __launch_bounds__(kThreads, min_blocks(LEN))
-    k_sha3_uniform(const uint8_t *__restrict__ msgs, uint64_t stride, uint64_t len_rt,
-                   uint8_t *__restrict__ out, uint32_t out_len, uint64_t n) {
+    k_sha3_uniform(const uint8_t *msgs, uint64_t stride, uint64_t len_rt,
+                   uint8_t *out, uint32_t out_len, uint64_t n) {
     using P = Variant<V>;
     launch_wait();
     constexpr int kOut = P::digest ? P::digest : P::rate;
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(kThreads, min_blocks(LEN))
             const uint4 *q = reinterpret_cast<const uint4 *>(p);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const uint4 v = __ldg(q + j);
+                const uint4 v = q[j];
                 Rep::set_word(A[2 * j], B[2 * j], v.x, v.y);
                 Rep::set_word(A[2 * j + 1], B[2 * j + 1], v.z, v.w);
             }
@@ -111,7 +111,7 @@ constexpr uint64_t kWaitNs = 1000000000ull;     // 1 s
 
 template <int V, class Rep>
 __global__ void __launch_bounds__(kThreads, kStagedMinBlocks)
-    k_sha3_uniform64_tma(const uint8_t *__restrict__ msgs, uint8_t *__restrict__ out, uint32_t out_len, uint64_t n,
+    k_sha3_uniform64_tma(const uint8_t *msgs, uint8_t *out, uint32_t out_len, uint64_t n,
                          unsigned int *status) {
     using P = Variant<V>;
     static_assert(64 < P::rate, "a 64-byte message is one block for every variant");

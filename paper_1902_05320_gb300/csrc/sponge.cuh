@@ -10,7 +10,11 @@
 //
 // Memory access rule: a message is read only through naturally aligned 4- or
 // 8-byte words that contain at least one of its bytes, so no access can leave
-// the page (or allocation granule) that holds the message.
+// the page (or allocation granule) that holds the message.  The loads are plain
+// ones: most kernels are set up while the kernel before them still writes
+// (launch_overlapped), and a read-only load (__ldg, or of a const __restrict__
+// parameter) promises data that stays as it is from then on, so nothing would keep
+// it behind launch_wait().
 #pragma once
 
 #include <cstdint>
@@ -22,7 +26,7 @@ namespace kb {
 
 // Little-endian 64-bit word of 8 valid bytes at an 8-byte aligned address.
 __device__ __forceinline__ void ld_word_a8(const uint8_t *p, uint32_t &lo, uint32_t &hi) {
-    const uint2 v = __ldg(reinterpret_cast<const uint2 *>(p));
+    const uint2 v = *reinterpret_cast<const uint2 *>(p);
     lo = v.x;
     hi = v.y;
 }
@@ -36,9 +40,9 @@ __device__ __forceinline__ void ld_word_any(const uint8_t *p, uint32_t nvalid, u
     const uint32_t sh = uint32_t(start & 3) * 8;
     const uintptr_t last = start + nvalid - 1;
     const uint32_t nw = uint32_t(((last & ~uintptr_t(3)) - (start & ~uintptr_t(3))) >> 2) + 1;
-    const uint32_t w0 = __ldg(a);
-    const uint32_t w1 = nw > 1 ? __ldg(a + 1) : 0u;
-    const uint32_t w2 = nw > 2 ? __ldg(a + 2) : 0u;
+    const uint32_t w0 = *a;
+    const uint32_t w1 = nw > 1 ? a[1] : 0u;
+    const uint32_t w2 = nw > 2 ? a[2] : 0u;
     lo = __funnelshift_r(w0, w1, sh);
     hi = __funnelshift_r(w1, w2, sh);
     if (nvalid < 8) {
@@ -63,11 +67,11 @@ __device__ __forceinline__ void absorb_full(uint32_t (&A)[25], uint32_t (&B)[25]
         const uintptr_t start = reinterpret_cast<uintptr_t>(p);
         const uint32_t *a = reinterpret_cast<const uint32_t *>(start & ~uintptr_t(3));
         const uint32_t sh = uint32_t(start & 3) * 8;
-        uint32_t prev = __ldg(a);
+        uint32_t prev = *a;
 #pragma unroll
         for (int k = 0; k < RATE / 8; ++k) {
-            const uint32_t w1 = __ldg(a + 2 * k + 1);
-            const uint32_t w2 = (2 * k + 2 < RATE / 4 || sh != 0) ? __ldg(a + 2 * k + 2) : 0u;
+            const uint32_t w1 = a[2 * k + 1];
+            const uint32_t w2 = (2 * k + 2 < RATE / 4 || sh != 0) ? a[2 * k + 2] : 0u;
             const uint32_t lo = __funnelshift_r(prev, w1, sh);
             const uint32_t hi = __funnelshift_r(w1, w2, sh);
             prev = w2;
@@ -199,12 +203,12 @@ __device__ __forceinline__ void absorb_full_rt(uint32_t (&A)[25], uint32_t (&B)[
         const uintptr_t start = reinterpret_cast<uintptr_t>(p);
         const uint32_t *a = reinterpret_cast<const uint32_t *>(start & ~uintptr_t(3));
         const uint32_t sh = uint32_t(start & 3) * 8;
-        uint32_t prev = __ldg(a);
+        uint32_t prev = *a;
 #pragma unroll
         for (int k = 0; k < 21; ++k) {
             if (k < nwords) {
-                const uint32_t w1 = __ldg(a + 2 * k + 1);
-                const uint32_t w2 = (2 * k + 2 < 2 * nwords || sh != 0) ? __ldg(a + 2 * k + 2) : 0u;
+                const uint32_t w1 = a[2 * k + 1];
+                const uint32_t w2 = (2 * k + 2 < 2 * nwords || sh != 0) ? a[2 * k + 2] : 0u;
                 const uint32_t lo = __funnelshift_r(prev, w1, sh);
                 const uint32_t hi = __funnelshift_r(w1, w2, sh);
                 prev = w2;
@@ -228,12 +232,12 @@ __device__ __forceinline__ void absorb_last_rt(uint32_t (&A)[25], uint32_t (&B)[
     // Aligned words 0 .. nw-1 overlap the rem message bytes.
     const uint32_t nw = rem ? uint32_t(((start + rem - 1) >> 2) - (start >> 2)) + 1 : 0u;
     int rb = int(8 * rem);  // message bits still to come, from the current 64-bit word on
-    uint32_t prev = nw ? __ldg(a) : 0u;
+    uint32_t prev = nw ? *a : 0u;
 #pragma unroll
     for (int k = 0; k < 21; ++k) {
         if (k < nwords) {
-            const uint32_t w1 = uint32_t(2 * k + 1) < nw ? __ldg(a + 2 * k + 1) : 0u;
-            const uint32_t w2 = uint32_t(2 * k + 2) < nw ? __ldg(a + 2 * k + 2) : 0u;
+            const uint32_t w1 = uint32_t(2 * k + 1) < nw ? a[2 * k + 1] : 0u;
+            const uint32_t w2 = uint32_t(2 * k + 2) < nw ? a[2 * k + 2] : 0u;
             uint32_t lo = __funnelshift_r(prev, w1, sh);
             uint32_t hi = __funnelshift_r(w1, w2, sh);
             prev = w2;
@@ -273,8 +277,8 @@ __device__ __forceinline__ void absorb_last_same(uint32_t (&A)[25], uint32_t (&B
             if constexpr (A8) {
                 ld_word_a8(p + 8 * k, lo, hi);
             } else {
-                const uint32_t w0 = __ldg(a + 2 * k), w1 = __ldg(a + 2 * k + 1);
-                const uint32_t w2 = o ? __ldg(a + 2 * k + 2) : 0u;
+                const uint32_t w0 = a[2 * k], w1 = a[2 * k + 1];
+                const uint32_t w2 = o ? a[2 * k + 2] : 0u;
                 lo = __funnelshift_r(w0, w1, sh);
                 hi = __funnelshift_r(w1, w2, sh);
             }

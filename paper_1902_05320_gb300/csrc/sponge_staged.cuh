@@ -220,23 +220,23 @@ __device__ __forceinline__ void sponge_rt_direct(const uint8_t *p, uint64_t len,
 __device__ __forceinline__ void fetch_full_seg(uint32_t (&w)[kStageWords], const uint8_t *q, int nwords, bool un) {
     const uint32_t *a = reinterpret_cast<const uint32_t *>(reinterpret_cast<uintptr_t>(q) & ~uintptr_t(3));
 #pragma unroll
-    for (int k = 0; k < 18; ++k) w[k] = __ldg(a + k);
-    if (nwords > 9 || un) w[18] = __ldg(a + 18);
+    for (int k = 0; k < 18; ++k) w[k] = a[k];
+    if (nwords > 9 || un) w[18] = a[18];
     if (nwords > 9) {
 #pragma unroll
-        for (int k = 19; k < 26; ++k) w[k] = __ldg(a + k);
-        if (nwords > 13 || un) w[26] = __ldg(a + 26);
+        for (int k = 19; k < 26; ++k) w[k] = a[k];
+        if (nwords > 13 || un) w[26] = a[26];
         if (nwords > 13) {
 #pragma unroll
-            for (int k = 27; k < 34; ++k) w[k] = __ldg(a + k);
-            if (nwords > 17 || un) w[34] = __ldg(a + 34);
+            for (int k = 27; k < 34; ++k) w[k] = a[k];
+            if (nwords > 17 || un) w[34] = a[34];
             if (nwords > 17) {
-                w[35] = __ldg(a + 35);
-                if (nwords > 18 || un) w[36] = __ldg(a + 36);
+                w[35] = a[35];
+                if (nwords > 18 || un) w[36] = a[36];
                 if (nwords > 18) {
 #pragma unroll
-                    for (int k = 37; k < 42; ++k) w[k] = __ldg(a + k);
-                    if (un) w[42] = __ldg(a + 42);
+                    for (int k = 37; k < 42; ++k) w[k] = a[k];
+                    if (un) w[42] = a[42];
                 }
             }
         }
@@ -303,7 +303,7 @@ __device__ __forceinline__ void sponge_rt_prefetch(const uint8_t *p, uint64_t le
     auto fetch_last = [&] {
         const uint32_t *a = reinterpret_cast<const uint32_t *>(reinterpret_cast<uintptr_t>(last) & ~uintptr_t(3));
 #pragma unroll
-        for (int k = 0; k < kStageWords; ++k) w[k] = uint32_t(k) < nw_last ? __ldg(a + k) : 0u;
+        for (int k = 0; k < kStageWords; ++k) w[k] = uint32_t(k) < nw_last ? a[k] : 0u;
     };
     if (nfull) fetch_full_seg(w, p, nwords, un);
     else fetch_last();

@@ -79,7 +79,7 @@ __device__ __forceinline__ void xor_bytes_at(uint32_t (&A)[25], uint32_t (&B)[25
     const uint32_t t0 = uint32_t(((pa & ~uintptr_t(3)) - qa) >> 2);            // first word holding a piece byte
     const uint32_t t1 = uint32_t((((pa + n - 1) & ~uintptr_t(3)) - qa) >> 2);  // last one
     auto word = [&](uint32_t t) -> uint32_t {
-        return (t >= t0 && t <= t1) ? __ldg(reinterpret_cast<const uint32_t *>(qa + 4 * uintptr_t(t))) : 0u;
+        return (t >= t0 && t <= t1) ? *reinterpret_cast<const uint32_t *>(qa + 4 * uintptr_t(t)) : 0u;
     };
     const int b0 = int(8 * off), b1 = int(8 * (off + n));
     uint32_t prev = word(0);
@@ -138,10 +138,10 @@ __global__ void __launch_bounds__(kThreads) k_stream_init(uint8_t *states, const
 // into out_lens[i] bytes at digests + out_off[i], and marked finalised.
 template <bool INIT, bool FINAL>
 __global__ void __launch_bounds__(kThreads, 3)
-    k_stream_step(uint8_t *states, const uint8_t *__restrict__ init_variants, const uint8_t *__restrict__ msgs,
-                  const uint64_t *__restrict__ offsets, const uint64_t *__restrict__ lens,
-                  const uint32_t *__restrict__ out_lens, const uint64_t *__restrict__ out_off,
-                  uint8_t *__restrict__ digests, uint64_t n, unsigned int *status) {
+    k_stream_step(uint8_t *states, const uint8_t *init_variants, const uint8_t *msgs,
+                  const uint64_t *offsets, const uint64_t *lens,
+                  const uint32_t *out_lens, const uint64_t *out_off,
+                  uint8_t *digests, uint64_t n, unsigned int *status) {
     const uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     launch_wait();
     if (i >= n) return;
@@ -262,9 +262,9 @@ __global__ void __launch_bounds__(kThreads, 3)
 // null in a final step: no piece.
 template <bool INIT, bool FINAL>
 __global__ void __launch_bounds__(32)
-    k_stream_step_coop(uint8_t *states, const uint8_t *__restrict__ init_variants, const uint8_t *__restrict__ msgs,
-                       const uint64_t *__restrict__ offsets, const uint64_t *__restrict__ lens,
-                       const uint32_t *__restrict__ out_lens, uint8_t *__restrict__ digests, unsigned int *status) {
+    k_stream_step_coop(uint8_t *states, const uint8_t *init_variants, const uint8_t *msgs,
+                       const uint64_t *offsets, const uint64_t *lens,
+                       const uint32_t *out_lens, uint8_t *digests, unsigned int *status) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     const Coop c(mem);
     const uint32_t i = blockIdx.x, lane = threadIdx.x;
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(32)
                     uint32_t w[3];
 #pragma unroll
                     for (uint32_t j = 0; j < 3; ++j)  // bytes [4j, 4j + 4) from q on; the piece's are [o + from, o + to)
-                        w[j] = 4 * j < o + to && 4 * j + 4 > o + from ? __ldg(q + j) : 0u;
+                        w[j] = 4 * j < o + to && 4 * j + 4 > o + from ? q[j] : 0u;
                     lo = __funnelshift_r(w[0], w[1], sh) & low_bits(8 * int(to)) & ~low_bits(8 * int(from));
                     hi = __funnelshift_r(w[1], w[2], sh) & low_bits(8 * int(to) - 32) & ~low_bits(8 * int(from) - 32);
                 }

@@ -65,3 +65,33 @@ def test_queue_kernel_takes_the_plan_over_before_it_reads_it():
     queue_cuh = sources()["queue.cuh"]
     assert "st.release.gpu" in block(queue_cuh, queue_cuh.index("void hand_over("), "{}")[0]
     assert "ld.acquire.gpu" in block(queue_cuh, queue_cuh.index("bool taken_over("), "{}")[0]
+
+
+def test_no_read_only_loads():
+    """A read-only load (__ldg, ld.global.nc, or a plain one of a const __restrict__ parameter) is for data that does not
+    change while the kernel runs, set-up included, so a compiler may move it before griddepcontrol.wait.  The sponge's
+    loads are shared by all kernels, so there are none at all; __restrict__ is left to kernels launched plainly."""
+    for name, text in sources().items():
+        assert "__ldg" not in text and "global.nc" not in text, name
+    for name, (params, body) in kernels().items():
+        if "launch_wait()" in body:
+            assert "__restrict__" not in params, name
+
+
+def test_overlapped_kernels_wait_before_they_read():
+    found = kernels()
+    launched = set()
+    for text in sources().values():
+        for m in re.finditer(r"\b(?:launch_overlapped|launch_tiled|book)\s*\(", text):
+            launched |= set(re.findall(r"\bk_\w+", block(text, m.start(), "()")[0]))
+    assert len(launched) >= 18 and launched <= set(found)
+    keccak_p = sources()["keccak_p.cu"]
+    tile, _ = block(keccak_p, keccak_p.index("void run_tile("), "{}")
+    assert tile.index("launch_wait()") < tile.index("cp.async.ca")
+    for name in launched:
+        params, body = found[name]
+        wait = re.search(r"launch_wait\(\)|run_tile\(", body)
+        assert wait, name
+        before = body[:wait.start()]
+        for pointer in re.findall(r"\*\s*(\w+)", params):
+            assert not re.search(rf"\b{pointer}\s*(\[|->)|[^&\w]\*{pointer}\b", before), (name, pointer)
