@@ -51,7 +51,13 @@ void release_device();
 uint64_t persistent_grid(const void *fn, int threads, size_t smem, uint64_t work_items,
                          const DeviceInfo &dev);
 
-inline int cuda_status(cudaError_t e) { return e == cudaSuccess ? KB_OK : KB_ERR_CUDA; }
+// The status of a runtime call.  Its error is cleared with it: the caller hears of it
+// here, and the thread's last error would be taken for that of a later plain launch.
+inline int cuda_status(cudaError_t e) {
+    if (e == cudaSuccess) return KB_OK;
+    cudaGetLastError();
+    return KB_ERR_CUDA;
+}
 
 // A launch that may be set up while the kernel before it in the stream still runs
 // (programmatic dependent launch).  The kernel calls launch_wait() before it
@@ -71,7 +77,9 @@ cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned bloc
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // as cuda_status
+    return e;
 }
 
 #ifdef __CUDACC__
