@@ -16,10 +16,11 @@
 //   3. k_sha3_queue: a persistent grid; each warp takes a group of 32
 //      consecutive entries of the order with one atomic and hashes one
 //      message per thread.  Warps run messages of nearly equal cost.  The
-//      queue has two parts of equal work: on every SM sub-partition the warp in
-//      the lowest hardware slot starts with the costlier (the longest chains
-//      start first), the others with the cheaper; either goes on to the other's
-//      part when its own is handed out.  Both parts run longest first.
+//      queue has two parts of equal work, the costlier with a group for every SM
+//      sub-partition at least: on every sub-partition the warp in the lowest
+//      hardware slot starts with the costlier (the longest chains start first),
+//      the others with the cheaper; either goes on to the other's part when its
+//      own is handed out.  Both parts run longest first.
 //   k_sha3_lanes runs the first K entries of the order (the K costliest
 //   messages; K from the plan, or given) one warp per message, concurrently with
 //   the queue kernel, which covers the entries from K on: it is launched first and
@@ -224,8 +225,15 @@ __device__ __forceinline__ uint64_t plan_split(const uint32_t (&count)[kPer], ui
 // half of the permutations of [first, n).  Where the line lies matters little between
 // 3/8 and 5/8 (2^20 messages log-uniform to 64 KiB 11.21 ms at each, 2^19 5.63 ms); at
 // 1/4 and 3/4 2^19 messages take 5.89, at 3/4 and 7/8 2^20 take 11.47 and 11.35.
-// Called as plan_split.
-__device__ __forceinline__ uint64_t plan_mid(const uint32_t (&count)[kPer], uint64_t before, uint64_t first) {
+// But the costlier part has at least `least` entries, a group for every SM
+// sub-partition: where the batch lasts as long as its longest chains, each of them
+// has to start in a slot that issues first, and a back-slot warp given one finishes
+// last (6,000 messages of 60,000 bytes beside 44,000 of 200, all in threads: 3647 us
+// at half of the work alone, 2041 with 304 groups at least, 2039 with 608, one per
+// sub-partition; 20,000 of lengths uniform to 64 KiB 3296, 2888, 2171 and with 1216
+// 2876).  Called as plan_split.
+__device__ __forceinline__ uint64_t plan_mid(const uint32_t (&count)[kPer], uint64_t before, uint64_t first,
+                                             uint64_t n, uint64_t least) {
     __shared__ unsigned long long skipped, mid;
     if (threadIdx.x == 0) {
         skipped = 0;
@@ -265,7 +273,9 @@ __device__ __forceinline__ uint64_t plan_mid(const uint32_t (&count)[kPer], uint
         }
     }
     __syncthreads();
-    return mid;
+    const uint64_t left = n > first ? n - first : 0;
+    const uint64_t floor = first + (left < least ? left : least);
+    return mid < floor ? floor : mid;
 }
 
 // Tile sums to the messages' exclusive sums, for batches of so many tiles that each
@@ -294,7 +304,7 @@ __global__ void __launch_bounds__(kScanThreads)
     k_scatter(const uint64_t *lens, const uint8_t *variants,
               const uint32_t *out_lens, uint64_t n, const uint64_t *tile_sums,
               uint64_t ntiles, uint64_t *out_off, uint32_t *order, Control *ctl,
-              uint64_t split) {
+              uint64_t split, uint32_t sub_partitions) {
     __shared__ uint32_t hist[kBuckets];
     __shared__ uint32_t start[kBuckets];
     for (int b = threadIdx.x; b < kBuckets; b += blockDim.x) hist[b] = 0;
@@ -355,10 +365,10 @@ __global__ void __launch_bounds__(kScanThreads)
         if (base + j < n) order[start[key[j]] + rank[j]] = uint32_t(base + j);
     if (blockIdx.x == 0) {
         const uint64_t first = split == kAutoSplit ? plan_split(count, m0) : split;
-        const uint64_t mid = plan_mid(count, m0, first);
+        const uint64_t mid = plan_mid(count, m0, first, n, 32ull * sub_partitions);
         if (threadIdx.x == 0) {
             ctl->queue_start = first;
-            ctl->queue_mid = mid < first ? first : mid;
+            ctl->queue_mid = mid;
         }
     }
 }

@@ -232,7 +232,8 @@ int queue_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *le
             launch_overlapped(k_plan_tiles, 1, kScanThreads, 0, stream, bf.tile_sums, ntiles) != cudaSuccess)
             return KB_ERR_CUDA;
         return cuda_status(launch_overlapped(scatter, unsigned(ntiles), kScanThreads, 0, stream, lens, variants,
-                                             out_lens, n, bf.tile_sums, ntiles, bf.out_off, bf.order, bf.ctl, split));
+                                             out_lens, n, bf.tile_sums, ntiles, bf.out_off, bf.order, bf.ctl, split,
+                                             uint32_t(4 * (sm_count > 0 ? sm_count : 1))));
     };
     int rc = KB_OK;
     if (cfg.per_variant) {

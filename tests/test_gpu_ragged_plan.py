@@ -1,0 +1,67 @@
+"""How a ragged batch is divided, judged by time where a wrong division costs a factor: between warps and threads, and
+between the queue's two parts.  Bytes are checked against hashlib on a sample."""
+import hashlib
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture
+def restore_split(cuda_lib):
+    saved = cuda_lib.keccak_tune_get(cuda_lib.KB_TUNE_QUEUE_WARP_MESSAGES)
+    yield
+    cuda_lib.keccak_tune_set(cuda_lib.KB_TUNE_QUEUE_WARP_MESSAGES, saved)
+
+
+class Batch:
+    """SHA3-256 messages of the given lengths back to back, in the given order."""
+
+    def __init__(self, cuda_lib, lens):
+        import torch
+
+        self.lib, self.n = cuda_lib, len(lens)
+        self.lens = np.asarray(lens, dtype=np.int64)
+        self.offsets = np.cumsum(self.lens) - self.lens
+        self.msgs = torch.randint(0, 256, (int(self.lens.sum()) + 16,), dtype=torch.uint8, device="cuda")
+        dev = lambda a: torch.from_numpy(a).cuda()  # noqa: E731
+        self.out = torch.zeros(32 * self.n, dtype=torch.uint8, device="cuda")
+        self.args = (self.msgs, dev(self.offsets), dev(self.lens), dev(np.ones(self.n, np.uint8)),
+                     dev(np.full(self.n, 32, np.int32)), self.out, self.n)
+
+    def ms(self, split=-1):
+        """Median time of a call with `split` messages fixed to a warp each (-1: the plan's choice)."""
+        import torch
+
+        self.lib.keccak_tune_set(self.lib.KB_TUNE_QUEUE_WARP_MESSAGES, split)
+        self.out.zero_()
+        times = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            self.lib.keccak_batch(*self.args)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        got, host = self.out.cpu().numpy().reshape(-1, 32), self.msgs.cpu().numpy()
+        for i in {0, 1, self.n // 2, self.n - 1, int(self.lens.argmax()), int(self.lens.argmin())}:
+            o, k = int(self.offsets[i]), int(self.lens[i])
+            assert got[i].tobytes() == hashlib.sha3_256(host[o:o + k].tobytes()).digest(), i
+        return float(np.median(times[2:]))
+
+
+@pytest.mark.parametrize("many", [9, 14])  # fortieths of the sub-partitions that the long messages fill
+def test_queue_long_chains_start_in_the_slots_that_issue_first(cuda_lib, restore_split, many):
+    """Long messages that give fewer sub-partitions than there are a warp each last as long as one of them; short ones
+    beside them, of less work in all than the GPU does meanwhile, add little.  (With half of the long chains left to the
+    warps that issue second they took 1.8 times as long.)"""
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n_long = 4 * sms * 32 * many // 40
+    rng = np.random.default_rng(many)
+    both = np.concatenate([np.full(n_long, 30000), np.full(7 * n_long, 200)])
+    rng.shuffle(both)
+    alone = Batch(cuda_lib, np.full(n_long, 30000)).ms(0)
+    assert Batch(cuda_lib, both).ms(0) < 1.3 * alone
