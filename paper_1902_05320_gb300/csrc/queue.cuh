@@ -166,59 +166,99 @@ __device__ __forceinline__ uint64_t bucket_cost(int b) {
 // thread per message (the rest), in picoseconds of a GB300: a permutation takes
 // kThreadChain in a thread of the queue kernel and kWarpChain in a warp of its
 // own; with the GPU full the queue kernel needs kThreadWork for each (4.65 G/s), and
-// the kLanesPerSm warps per SM beside it kWarpWork.  kWarpWork is fitted (alone they
-// reach 670 M/s, 1500 ps): the two kernels share the issue slots.  Batches of
-// lengths log-uniform to 64 KiB, us before, at 2200 and at 3000: 2,000 messages
-// 4123, 1706, 1727; 20,000 4120, 2335, 2386; 100,000 4127, 2813, 2904; 200,000
-// 4201, 3659, 3522; 300,000 4215, 4145, 4196.  A larger kThreadChain (6000000,
-// 7500000) gains a tenth at 20,000 and loses a tenth to a quarter at 300,000.
-constexpr uint64_t kThreadChain = 4800000, kWarpChain = 1700000, kThreadWork = 215, kWarpWork = 3000;
+// the kLanesPerSm warps per SM beside it kWarpWork, alone kWarpAlone: the two kernels
+// share the issue slots.  kWarpWork is fitted on lengths log-uniform to 64 KiB, us
+// before, at 2200 and at 3000: 2,000 messages 4123, 1706, 1727; 20,000 4120, 2335,
+// 2386; 100,000 4127, 2813, 2904; 200,000 4201, 3659, 3522; 300,000 4215, 4145, 4196.
+// A larger kThreadChain (6000000, 7500000) gains a tenth at 20,000 and loses a tenth
+// to a quarter at 300,000.
+constexpr uint64_t kThreadChain = 4800000, kWarpChain = 1700000, kThreadWork = 215, kWarpWork = 3000, kWarpAlone = 1750;
 constexpr uint64_t kAutoSplit = ~uint64_t(0);
 
-// The queue kernel's first entry where the plan chooses it: the number of messages
-// that are better off with a warp each.  With W permutations in all, w(b) of them in
-// buckets above b and c(b) the cost of bucket b, the batch lasts about
-// max(c(b) kThreadChain, W kThreadWork, w(b) kWarpWork, c_max kWarpChain) when the
-// buckets above b go to warps; the first term falls with b, the third rises, so the
-// split is the first b where the first is no longer the largest.  (A batch big
-// enough to fill the GPU for its longest chain's time splits off nothing.)  Called
-// by a whole block; thread t holds the counts of buckets kBuckets-1 - (kPer t + j) and
-// `before`, the messages in buckets above them.
-constexpr int kPer = (kBuckets + kScanThreads - 1) / kScanThreads;
-__device__ __forceinline__ uint64_t plan_split(const uint32_t (&count)[kPer], uint64_t before) {
-    __shared__ unsigned long long first_cut, cost_max;
-    if (threadIdx.x == 0) {
-        first_cut = ~0ull;
-        cost_max = 0;
-    }
-    uint64_t work = 0, top = 0;
+// About how long the batch lasts when the costliest messages, `moved` of the `all`
+// permutations, go to warps, the costliest left takes `next` permutations (0: none is
+// left) and the costliest of all `top`.  The warps keep kWarpWork while the queue
+// kernel runs and kWarpAlone from then on.
+__device__ __forceinline__ uint64_t split_time(uint64_t next, uint64_t moved, uint64_t all, uint64_t top) {
+    const uint64_t chain = next * kThreadChain, work = all * kThreadWork;
+    const uint64_t queue = next == 0 ? 0 : chain > work ? chain : work;
+    const uint64_t beside = moved * kWarpWork;
+    const uint64_t after = moved * kWarpAlone + queue / kWarpWork * (kWarpWork - kWarpAlone);
+    uint64_t t = beside < after ? beside : after;
+    if (t < queue) t = queue;
+    return moved && t < top * kWarpChain ? top * kWarpChain : t;
+}
+
+// The least of a warp's values into a shared word, one atomic a warp.
+__device__ __forceinline__ void warp_min_into(unsigned long long &word, uint64_t v) {
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) {
+    for (int o = 16; o > 0; o >>= 1) {
+        const uint64_t other = __shfl_xor_sync(0xffffffffu, v, o);
+        v = other < v ? other : v;
+    }
+    if ((threadIdx.x & 31) == 0) atomicMin(&word, (unsigned long long)v);
+}
+
+// The queue kernel's first entry where the plan chooses it: the number of messages
+// that are better off with a warp each.  The candidates are the edges between the
+// buckets, from none to all; of equal ones the first.  A split has to save an eighth
+// by the model to be taken: where it promises less, the warps' share of the issue
+// slots slows the chains beside them by as much (20,000 messages of lengths uniform to
+// 64 KiB 2434 us split for a promised 4%, 2171 in threads).  (The first edge at which
+// the next chain is no longer the longest term, without a look at what the moved work
+// takes, gave whole batches of one cost to warps: 20,000 messages of 64 KiB 16353 us,
+// 3942 in threads, 10,000 of 4 KiB 594 and 175.)  Called by a whole block; thread t
+// holds the counts of buckets kBuckets-1 - (kPer t + j) and, in the buckets above
+// them, `before` messages of w permutations out of the batch's `all`.
+constexpr int kPer = (kBuckets + kScanThreads - 1) / kScanThreads;
+__device__ __forceinline__ uint64_t plan_split(const uint32_t (&count)[kPer], uint64_t before, uint64_t w,
+                                               uint64_t all, uint64_t n) {
+    __shared__ unsigned long long top_cost, unsplit, best, cut;
+    if (threadIdx.x == 0) {
+        top_cost = 0;
+        unsplit = 0;
+        best = ~0ull;
+        cut = n;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {  // the first bucket that is not empty, in descending order of cost
         const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
-        if (b >= 0 && count[j]) {
-            const uint64_t c = bucket_cost(b);
-            work += count[j] * c;
-            if (top == 0) top = c;  // buckets come in descending order of cost
+        if (b >= 0 && count[j] && before == 0) {
+            top_cost = bucket_cost(b);
+            break;
         }
     }
-    uint64_t w;
-    const uint64_t all = block_exclusive_scan(work, w);  // (its barriers cover the lines above)
-    if (top) atomicMax(&cost_max, (unsigned long long)top);
     __syncthreads();
-    uint64_t m = before;
+    uint64_t time[kPer], m = before;  // of the edge before each bucket
+    uint64_t least = threadIdx.x == 0 ? split_time(0, all, all, top_cost) : ~0ull;  // every message to a warp
 #pragma unroll
     for (int j = 0; j < kPer; ++j) {
         const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+        time[j] = ~0ull;
         if (b >= 0 && count[j]) {
-            const uint64_t c = bucket_cost(b), chain = c * kThreadChain;
-            if (chain <= all * kThreadWork || chain <= w * kWarpWork || chain <= cost_max * kWarpChain)
-                atomicMin(&first_cut, (unsigned long long)m);
+            const uint64_t c = bucket_cost(b);
+            time[j] = split_time(c, w, all, top_cost);
+            if (m == 0) unsplit = time[j];
+            else least = time[j] < least ? time[j] : least;
             m += count[j];
             w += count[j] * c;
         }
     }
+    warp_min_into(best, least);
     __syncthreads();
-    return first_cut;  // where no bucket met the condition, every message gets a warp
+    if (best >= unsplit - unsplit / 8) return 0;
+    m = before;
+    least = n;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        if (time[j] == best && m > 0 && m < least) least = m;
+        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+        if (b >= 0) m += count[j];
+    }
+    warp_min_into(cut, least);
+    __syncthreads();
+    return cut;
 }
 
 // The entry where the queue kernel's cheaper part begins: entries [first, mid) have
@@ -233,20 +273,13 @@ __device__ __forceinline__ uint64_t plan_split(const uint32_t (&count)[kPer], ui
 // sub-partition; 20,000 of lengths uniform to 64 KiB 3296, 2888, 2171 and with 1216
 // 2876).  Called as plan_split.
 __device__ __forceinline__ uint64_t plan_mid(const uint32_t (&count)[kPer], uint64_t before, uint64_t first,
-                                             uint64_t n, uint64_t least) {
+                                             uint64_t w, uint64_t all, uint64_t n, uint64_t least) {
     __shared__ unsigned long long skipped, mid;
     if (threadIdx.x == 0) {
         skipped = 0;
         mid = first;
     }
-    uint64_t work = 0;
-#pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-        const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
-        if (b >= 0) work += count[j] * bucket_cost(b);
-    }
-    uint64_t w;
-    const uint64_t all = block_exclusive_scan(work, w);
+    __syncthreads();
     uint64_t m = before, u = w;
 #pragma unroll
     for (int j = 0; j < kPer; ++j) {
@@ -364,8 +397,15 @@ __global__ void __launch_bounds__(kScanThreads)
     for (int j = 0; j < kScanItems; ++j)
         if (base + j < n) order[start[key[j]] + rank[j]] = uint32_t(base + j);
     if (blockIdx.x == 0) {
-        const uint64_t first = split == kAutoSplit ? plan_split(count, m0) : split;
-        const uint64_t mid = plan_mid(count, m0, first, n, 32ull * sub_partitions);
+        uint64_t work = 0, w;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int b = kBuckets - 1 - (int(threadIdx.x) * kPer + j);
+            if (b >= 0) work += count[j] * bucket_cost(b);
+        }
+        const uint64_t all = block_exclusive_scan(work, w);
+        const uint64_t first = split == kAutoSplit ? plan_split(count, m0, w, all, n) : split;
+        const uint64_t mid = plan_mid(count, m0, first, w, all, n, 32ull * sub_partitions);
         if (threadIdx.x == 0) {
             ctl->queue_start = first;
             ctl->queue_mid = mid;

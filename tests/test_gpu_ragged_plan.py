@@ -65,3 +65,33 @@ def test_queue_long_chains_start_in_the_slots_that_issue_first(cuda_lib, restore
     rng.shuffle(both)
     alone = Batch(cuda_lib, np.full(n_long, 30000)).ms(0)
     assert Batch(cuda_lib, both).ms(0) < 1.3 * alone
+
+
+@pytest.mark.parametrize("kind", ["equal", "below a block", "few long"])
+@pytest.mark.parametrize("per_sm", [33, 66, 131])
+def test_split_leaves_equal_costs_to_threads(cuda_lib, restore_split, per_sm, kind):
+    """Where warps would take longer for the costliest class than threads do, the plan moves none of it: the time is
+    that of a thread for every message, give or take the launch beside it (at most 0.01 ms) and a tenth."""
+    import torch
+
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(per_sm)
+    lens = {"equal": np.full(n, 4096), "below a block": rng.integers(0, 136, size=n),
+            "few long": np.where(rng.random(n) < 0.5, 30000, 100)}[kind]
+    batch = Batch(cuda_lib, lens)
+    threads = batch.ms(0)
+    assert batch.ms() < 1.1 * threads + 0.01
+
+
+@pytest.mark.parametrize("kind", ["log-uniform", "a hundred long"])
+def test_split_gives_few_long_chains_a_warp_each(cuda_lib, restore_split, kind):
+    """Where a thread's chain for the costliest messages is longer than all the rest takes, they get a warp each, which
+    is a third of that chain; half of the gain is asked for."""
+    import torch
+
+    n = 66 * torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(7)
+    lens = np.exp(rng.uniform(0, np.log(65536), size=n)).astype(np.int64) if kind == "log-uniform" else \
+        np.where(np.arange(n) % (n // 100) == 0, 65536, 500)
+    batch = Batch(cuda_lib, lens)
+    assert batch.ms() < 0.67 * batch.ms(0)
