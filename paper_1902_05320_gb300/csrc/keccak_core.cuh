@@ -307,15 +307,18 @@ __device__ __forceinline__ void plain_rounds_ct(uint32_t (&L)[25], uint32_t (&H)
 // lanes) or where nothing else competes for the instruction cache (raw states,
 // 897 -> 885 us on 2^22), and costs where blocks are absorbed in between (15
 // blocks of SHA3-512 on 2^18 messages 821 -> 827 us, a 4 GiB tree 6.62 -> 6.66 ms).
-template <bool PEEL0, int TAIL, int UNROLL = 4>
+// MUL = false: every rotation by funnel shifts, for a warp alone on its sub-partition
+// (rotl64_round); only where no round is unrolled.
+template <bool PEEL0, int TAIL, int UNROLL = 4, bool MUL = true>
 __device__ __forceinline__ void keccak_f1600_plain(uint32_t (&L)[25], uint32_t (&H)[25]) {
     constexpr int kFirst = PEEL0 ? 1 : 0;
     static_assert((TAIL - kFirst) % UNROLL == 0 && TAIL <= 24, "whole passes of the loop");
+    static_assert(MUL || (!PEEL0 && TAIL == 24), "the unrolled rounds use the multiply pipe");
     if constexpr (PEEL0) plain_round_ct<0>(L, H);
 #pragma unroll 1
     for (int r = kFirst; r < TAIL; r += UNROLL) {
 #pragma unroll
-        for (int j = 0; j < UNROLL; ++j) plain_round_rt(L, H, r + j);
+        for (int j = 0; j < UNROLL; ++j) plain_round_rt<MUL>(L, H, r + j);
     }
     plain_rounds_ct<TAIL>(L, H, std::make_integer_sequence<int, 24 - TAIL>{});
 }

@@ -90,11 +90,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         } else {
             squeeze<P::rate, PlainRep>(A, B, dst + (i - nfull - 1) * P::rate, P::rate);
         }
-#pragma unroll 1
-        for (int r = 0; r < 24; r += 4) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) plain_round_rt<MUL>(A, B, r + j);
-        }
+        keccak_f1600_plain<false, 24, 4, MUL>(A, B);
     }
     squeeze<P::rate, PlainRep>(A, B, dst + uint64_t(nsq) * P::rate, dlen - nsq * P::rate);
 }

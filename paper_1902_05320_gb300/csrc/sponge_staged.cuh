@@ -133,9 +133,9 @@ __device__ __forceinline__ void absorb_staged_last(uint32_t (&A)[25], uint32_t (
 // LOOPED: all 24 rounds in the loop of four, half the code of the form with an
 // unrolled tail, for kernels whose instruction footprint matters more than the
 // immediates.
-template <bool LOOPED>
+template <bool LOOPED, bool MUL = true>
 __device__ __forceinline__ void permute_plain(uint32_t (&A)[25], uint32_t (&B)[25]) {
-    keccak_f1600_plain<false, LOOPED ? 24 : 20>(A, B);
+    keccak_f1600_plain<false, LOOPED ? 24 : 20, 4, MUL>(A, B);
 }
 
 // One whole sponge of a message of len bytes at p with variant `variant`
