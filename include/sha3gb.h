@@ -128,7 +128,9 @@ int keccak_batch(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *l
  *   SHA3GB_TUNE  "off": keccak_batch ignores tuned configurations; "full":
  *     keccak_batch tunes a size class the first time it sees it (that call
  *     is then synchronous and allocates as keccak_batch_autotune does, and
- *     not inside stream capture); "cached" or unset: configurations found by
+ *     not inside stream capture), unless all batches of the class take the
+ *     single launch of small batches (KB_TUNE_QUEUE_WARP_MESSAGES below), which
+ *     has nothing to tune; "cached" or unset: configurations found by
  *     keccak_batch_autotune or read from the file are used.
  */
 int keccak_batch_autotune(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens,

@@ -563,11 +563,13 @@ int launch_ragged_queue(const uint8_t *msgs, const uint64_t *offsets, const uint
                         const DeviceInfo &dev) {
     int err = KB_OK;
     // SHA3GB_TUNE=full: a size class seen for the first time is tuned here
-    // (synchronously), which also leaves this batch's digests.
+    // (synchronously), which also leaves this batch's digests; not one whose largest
+    // batch takes the single launch, which has no configuration.
     cudaStreamCaptureStatus cap0 = cudaStreamCaptureStatusNone;
     if (tune_mode() == TuneMode::Full && use_tuned() && tuning_get(KB_TUNE_RAGGED_SCHEDULE) == KB_SCHEDULE_QUEUE &&
         tuning_get(KB_TUNE_QUEUE_MIN_BLOCKS) == 0 && tuning_get(KB_TUNE_QUEUE_BLOCKS_PER_SM) == 0 &&
         tuning_get(KB_TUNE_QUEUE_STAGING) == 0 && tuning_get(KB_TUNE_QUEUE_WARP_MESSAGES) < 0 &&
+        !ragged_small((uint64_t(2) << size_class(n)) - 1, dev.sm_count) &&
         cudaStreamIsCapturing(stream, &cap0) == cudaSuccess && cap0 == cudaStreamCaptureStatusNone &&
         !have_tuned(n, dev))
         return autotune_ragged_queue(msgs, offsets, lens, variants, out_lens, digests, n, stream, dev, nullptr);
