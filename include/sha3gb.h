@@ -110,20 +110,23 @@ int keccak_batch(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *l
  * keccak_batch_autotune -- the autotuner of the ragged schedule: hashes the
  * given batch (same arguments and outputs as keccak_batch) once per candidate
  * configuration of the persistent queue (register budget x blocks per SM x
- * staging of message blocks, then threads per message: one thread for every
- * message, or one warp for each of the K costliest), checks that every
- * candidate writes the same bytes as the first, and records the fastest for
- * this device and this batch size class (n rounded down to a power of two);
- * later keccak_batch calls of that class use it.  Synchronous.  The chosen
- * register budget, blocks per SM and its time in ms are written to the HOST
- * pointers when they are not NULL (keccak_batch_autotune_ex reports every
- * dimension).  Allocates a temporary device copy of the outputs.
+ * staging of message blocks, then threads per message: as many of the
+ * costliest messages a warp each as the batch's plan finds worth it, or a
+ * fixed K), checks that every candidate writes the same bytes as the first,
+ * and records the fastest for this device and this batch size class (n
+ * rounded down to a power of two); later keccak_batch calls of that class use
+ * it, but for batches that take the single launch of small batches
+ * (KB_TUNE_QUEUE_WARP_MESSAGES below).  Synchronous.  The chosen register
+ * budget, blocks per SM and its time in ms are written to the HOST pointers
+ * when they are not NULL (keccak_batch_autotune_ex reports every dimension).
+ * Allocates a temporary device copy of the outputs.
  * Environment, read by the library:
  *   SHA3GB_TUNE_CACHE  a file path: configurations the autotuner finds are
  *     written there and read back by later processes on the same kind of GPU.
  *     JSON Lines, one object per GPU name, SM count and size class
  *     floor(log2 n): {"gpu": "...", "sms": S, "size_class": C,
- *     "min_blocks": M, "blocks_per_sm": B}.  Unreadable files and lines that
+ *     "min_blocks": M, "blocks_per_sm": B, "staging": KB_QUEUE_STAGING_*,
+ *     "warp_messages": K}, K = 0 for the plan's choice.  Unreadable files and lines that
  *     do not parse are ignored.
  *   SHA3GB_TUNE  "off": keccak_batch ignores tuned configurations; "full":
  *     keccak_batch tunes a size class the first time it sees it (that call
@@ -190,8 +193,8 @@ int keccak_tuned_config(uint64_t n, int64_t *min_blocks, int64_t *blocks_per_sm)
  * host where cudaMalloc (which can synchronise the whole device) is not
  * allowed, or code that must know its footprint in advance cannot accept
  * that.  This entry point runs keccak_batch's cost-bucketed queue (the same
- * kernels, in the built-in configuration with one thread per message,
- * launched directly rather than from a cached graph) with the scratch in a
+ * kernels, in the built-in configuration, launched directly rather than from
+ * a cached graph; the single launch for small batches) with the scratch in a
  * fixed device array compiled into the library, of KB_NOALLOC_SCRATCH_BYTES
  * (about 814 KiB: a 256-byte status word, the 46,336-byte control block and
  * 12 bytes per message plus the scan's tile sums for KB_NOALLOC_MAX_MESSAGES

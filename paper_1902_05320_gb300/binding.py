@@ -170,7 +170,9 @@ def keccak_batch(msgs, offsets, lens, variants, out_lens, digests, n: int, strea
 
 
 class QueueConfig(ctypes.Structure):
-    """kb_queue_config of sha3gb.h."""
+    """kb_queue_config of sha3gb.h.  ``warp_messages`` 0 fixes no number of messages that take a warp each: the plan of
+    each batch picks it (``split``), unless the KB_TUNE_QUEUE_WARP_MESSAGES knob says none; ``threads_per_message`` is
+    what is fixed."""
     _fields_ = [("min_blocks", ctypes.c_int64), ("blocks_per_sm", ctypes.c_int64), ("staging", ctypes.c_int64),
                 ("warp_messages", ctypes.c_int64), ("ms", ctypes.c_float)]
 
@@ -179,12 +181,19 @@ class QueueConfig(ctypes.Structure):
                 "staging": QUEUE_STAGING_NAMES.get(self.staging, self.staging),
                 "threads_per_message": "1" if self.warp_messages == 0 else
                 f"32 for the {self.warp_messages} costliest, 1 for the rest",
-                "warp_messages": self.warp_messages, "ms": self.ms}
+                "warp_messages": self.warp_messages, "split": self.split(), "ms": self.ms}
+
+    def split(self) -> str:
+        """Who decides how many of a batch's costliest messages take a warp each."""
+        if self.warp_messages or keccak_tune_get(KB_TUNE_QUEUE_WARP_MESSAGES) >= 0:
+            return f"fixed: {self.warp_messages}"
+        return "the plan of each batch"
 
 
 def keccak_batch_autotune(msgs, offsets, lens, variants, out_lens, digests, n: int, stream=None) -> dict:
     """Runs the ragged-schedule autotuner on this batch (digests are written
-    as by keccak_batch); returns the chosen configuration and its time."""
+    as by keccak_batch); returns the chosen configuration, who decides how many messages
+    take a warp each under it, and its time."""
     cfg = QueueConfig()
     _check(load().keccak_batch_autotune_ex(_ptr(msgs), _ptr(offsets), _ptr(lens), _ptr(variants), _ptr(out_lens),
                                            _ptr(digests), n, _stream(stream), ctypes.addressof(cfg)),
@@ -200,6 +209,7 @@ def keccak_tuned_config(n: int) -> dict:
     _check(load().keccak_tuned_config_ex(n, ctypes.addressof(cfg)), "keccak_tuned_config_ex")
     d = cfg.as_dict()
     d.pop("ms")
+    d.pop("split")
     return d
 
 

@@ -34,9 +34,11 @@ constexpr int64_t kHybridChoices[] = {32, 608};
 constexpr uint64_t kLanesPerSm = 8;
 
 // Messages per SM up to which a ragged batch takes the single launch of one warp
-// per message, in input order.  Equal long messages bound it: 1.4 ns a permutation
-// with every SM busy, against 4.6 us for any number up to 128 per SM in threads,
-// cross at 21.
+// per message, in input order.  Long messages of one length bound it: with every SM
+// busy 1.4 to 1.6 ns a permutation, against 4.6 us in threads for any number up to 128
+// per SM, cross at 18 to 21.  3,040 messages, us alone and by the queue: of 4 KiB 170
+// and 167, of 64 KiB 2334 and 2136; of 64 bytes 10 and 34, of lengths log-uniform to
+// 600 bytes 23 and 53, to 64 KiB 1545 and 1684.
 constexpr uint64_t kRaggedCoopPerSm = 20;
 
 // Device scratch of one call for n messages: the queue's control block, the

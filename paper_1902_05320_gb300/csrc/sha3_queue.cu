@@ -361,8 +361,10 @@ int size_class(uint64_t n) { return n ? 63 - __builtin_clzll(n) : 0; }
 //    "min_blocks": register budget (blocks per SM compiled for),
 //    "blocks_per_sm": blocks per SM of the launch,
 //    "staging": KB_QUEUE_STAGING_* value, "warp_messages": K}
-// Lines without the last two fields (an older form) read as direct loads and
-// K = 0.  Entries are matched on the GPU's name and SM count; lines that do
+// K = 0 fixes no number: the plan of each batch picks it.  (Lines written while 0
+// meant a thread for every message read the same; the plan finds that form where it
+// is the quicker one.)  Lines without the last two fields (an older form) read as
+// direct loads and K = 0.  Entries are matched on the GPU's name and SM count; lines that do
 // not parse are ignored, and I/O failures leave the in-memory tuning as it is.
 
 struct CacheLine {
@@ -647,9 +649,9 @@ __global__ void k_compare(const uint8_t *__restrict__ a, const uint8_t *__restri
 }
 
 // The candidates of the autotuner: every compiled (register budget, staging)
-// pair at its largest resident block count and the two below it, with one
-// thread per message; the hybrid split is tried afterwards on the best of
-// those (tune_hybrid).
+// pair at its largest resident block count and the two below it, with the split
+// that the plan chooses for the batch; fixed splits are tried afterwards on the
+// best of those.
 std::vector<QueueConfig> base_candidates(int device) {
     std::vector<QueueConfig> out;
     for (int stage : kStageCodes) {
@@ -674,7 +676,7 @@ std::vector<QueueConfig> base_candidates(int device) {
 
 // Autotuner: times every candidate on this batch, checks that each writes
 // the same bytes as the first, and keeps the fastest for batches of the same
-// size class on this device.  Then tries the hybrid split (the K costliest
+// size class on this device.  Then tries fixed splits (the K costliest
 // messages one warp each, K in kHybridChoices) on the winner.  Synchronous;
 // allocates a reference copy of the outputs for the duration of the call.
 int autotune_ragged_queue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens, const uint8_t *variants,
