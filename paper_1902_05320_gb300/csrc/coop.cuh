@@ -38,10 +38,6 @@
 
 namespace kb {
 
-// Blocks of one such warp (four per SM) up to which the next kernel of the stream
-// is set up as soon as these have started.
-constexpr uint32_t kFewBlocks = 600;
-
 // The round constants' even and odd halves.
 struct CoopRcTable {
     uint32_t w[48];

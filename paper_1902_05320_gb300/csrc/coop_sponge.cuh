@@ -106,14 +106,14 @@ __device__ __forceinline__ void coop_squeeze(const Coop &c, const uint32_t (&a)[
 // One sponge: the message of len bytes at p (PREFIX >= 0: that byte comes before
 // it), dlen output bytes to dst.  Every thread of the warp calls it with the same
 // arguments.  ONLY: the kernel hashes nothing else and has one such warp a block;
-// the next one may then be set up at once where there are few blocks, and from the
-// last message block on where there are many: its blocks are placed while this
+// the next one may then be set up at once where there are `few` blocks (few_warps),
+// and from the last message block on where there are many: its blocks are placed while this
 // kernel's still stand and would crowd some SMs, where such warps slow one another
 // (1824 leaves of 1000 bytes a call: 63 to 96 us from run to run set up at once,
 // 57.5 late; 200 ragged messages 14.4 at once, 16.8 late).
 template <int PREFIX = -1, bool ONLY = false>
 __device__ __forceinline__ void coop_sponge(const Coop &c, const uint8_t *p, uint64_t len, int variant, uint8_t *dst,
-                                            uint32_t dlen) {
+                                            uint32_t dlen, bool few = false) {
     constexpr int kShift = PREFIX >= 0 ? 1 : 0;  // bytes before the message
     const uint32_t rate = uint32_t(variant_rate(variant));
     const int nwords = int(rate / 8);
@@ -123,7 +123,7 @@ __device__ __forceinline__ void coop_sponge(const Coop &c, const uint8_t *p, uin
     const uint32_t nsq = dlen > rate ? (dlen - 1) / rate : 0;
     const uint64_t total = nfull + 1 + nsq;  // permutations
     const uint32_t o = uint32_t((reinterpret_cast<uintptr_t>(p) - kShift) & 3);  // the same for every lane word
-    if (ONLY && gridDim.x <= kFewBlocks) launch_next();
+    if (ONLY && few) launch_next();
     uint32_t a[2] = {0, 0}, e[2] = {0, 0};
     RawWord raw[2] = {};
     int64_t left[2] = {-1, -1};

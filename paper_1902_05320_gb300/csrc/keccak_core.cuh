@@ -189,7 +189,7 @@ __device__ __forceinline__ uint32_t shl_pair_mul(uint32_t lo, uint32_t hi) {
 
 // The rounds' 64-bit rotation: by multiplies for offsets of 1..11 modulo 32
 // (theta's 1 and rho's 1, 2, 3, 6, 8, 10, 36, 39, 41 and 43), by funnel shifts
-// otherwise.  A round then has 149 ALU instructions and 96 multiplies instead
+// otherwise.  A round then has 149 ALU instructions and 94 multiplies instead
 // of 180 and none: 361 -> 328 cycles a warp and sub-partition in the looped
 // permutation (333 and 324 on a later build, with equal shares a warp and with work
 // handed out in small units).  It does not reach the ALU's 298: a multiply with two

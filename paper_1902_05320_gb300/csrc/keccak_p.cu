@@ -223,10 +223,10 @@ __global__ void __launch_bounds__(kThreads) k_keccak_p_1600(uint64_t *states, in
 
 // Few states of width 64 and rounds within Keccak-f[1600]'s 24: a warp each
 // (coop.cuh), a third of the time of one thread's chain of rounds.
-__global__ void __launch_bounds__(32) k_keccak_p_1600_coop(uint64_t *states, int first_ir, int nr) {
+__global__ void __launch_bounds__(32) k_keccak_p_1600_coop(uint64_t *states, int first_ir, int nr, bool few) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     const Coop c(mem);
-    if (gridDim.x <= kFewBlocks) launch_next();
+    if (few) launch_next();
     launch_wait();
     uint2 *st = reinterpret_cast<uint2 *>(states + 25 * uint64_t(blockIdx.x));
     uint32_t a[2] = {0, 0};
@@ -258,7 +258,7 @@ int launch_tiled(K kernel, uint64_t *states, int first_ir, int nr, uint64_t n, c
 }
 
 template <int W>
-int launch_small(uint64_t *states, int first_ir, int nr, uint64_t n, cudaStream_t stream, const DeviceInfo &dev) {
+int launch_small(uint64_t *states, int first_ir, int nr, uint64_t n, cudaStream_t stream) {
     return launch_tiled(k_keccak_p_small<W>, states, first_ir, nr, n, stream);
 }
 
@@ -271,16 +271,17 @@ int launch_keccak_p(uint64_t *states, int b, int nr, uint64_t n, cudaStream_t st
     if (l < 0) return KB_ERR_INVALID;
     const int first_ir = 12 + 2 * l - nr;
     switch (l) {
-        case 0: return launch_small<1>(states, first_ir, nr, n, stream, dev);
-        case 1: return launch_small<2>(states, first_ir, nr, n, stream, dev);
-        case 2: return launch_small<4>(states, first_ir, nr, n, stream, dev);
-        case 3: return launch_small<8>(states, first_ir, nr, n, stream, dev);
-        case 4: return launch_small<16>(states, first_ir, nr, n, stream, dev);
-        case 5: return launch_small<32>(states, first_ir, nr, n, stream, dev);
+        case 0: return launch_small<1>(states, first_ir, nr, n, stream);
+        case 1: return launch_small<2>(states, first_ir, nr, n, stream);
+        case 2: return launch_small<4>(states, first_ir, nr, n, stream);
+        case 3: return launch_small<8>(states, first_ir, nr, n, stream);
+        case 4: return launch_small<16>(states, first_ir, nr, n, stream);
+        case 5: return launch_small<32>(states, first_ir, nr, n, stream);
         default: {
             if (first_ir >= 0 && n <= kCoopPerSm * uint64_t(dev.sm_count > 0 ? dev.sm_count : 1))
                 return cuda_status(
-                    launch_overlapped(k_keccak_p_1600_coop, unsigned(n), 32, 0, stream, states, first_ir, nr));
+                    launch_overlapped(k_keccak_p_1600_coop, unsigned(n), 32, 0, stream, states, first_ir, nr,
+                                      few_warps(n, dev.sm_count)));
             // Staged through shared memory below 16 rounds (2^22 states: 12 rounds
             // 574 us read directly, 463 staged; 14 rounds 560 and 532; 18 rounds
             // 647 and 669; 24 rounds 839 and 875).

@@ -253,12 +253,12 @@ __device__ __forceinline__ void load_node_block(uint32_t (&A)[25], uint32_t (&B)
 // Few leaves: one warp each (coop_sponge.cuh), which takes a third of the time of a
 // thread for a leaf's chain of permutations.
 __global__ void __launch_bounds__(32)
-    k_merkle_leaves_coop(const uint8_t *buf, uint64_t leaf_bytes, uint8_t *out) {
+    k_merkle_leaves_coop(const uint8_t *buf, uint64_t leaf_bytes, uint8_t *out, bool few) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     const Coop c(mem);
     const uint64_t i = blockIdx.x;
     launch_wait();
-    coop_sponge<0, true>(c, buf + i * leaf_bytes, leaf_bytes, 1, out + 32 * i, 32);
+    coop_sponge<0, true>(c, buf + i * leaf_bytes, leaf_bytes, 1, out + 32 * i, 32, few);
 }
 
 // Levels where a permutation's latency, not the ALU pipe's throughput, sets the
@@ -451,7 +451,8 @@ int launch_leaves(const uint8_t *buf, uint64_t n_leaves, uint64_t leaf_bytes, ui
     const uint64_t few = leaf_bytes + 1 < uint64_t(kRate) ? kCoopOnePerSm : kCoopPerSm;
     if (n_leaves <= few * sms)
         return cuda_status(
-            launch_overlapped(k_merkle_leaves_coop, unsigned(n_leaves), 32, 0, stream, buf, leaf_bytes, out));
+            launch_overlapped(k_merkle_leaves_coop, unsigned(n_leaves), 32, 0, stream, buf, leaf_bytes, out,
+                              few_warps(n_leaves, dev.sm_count)));
     const bool a8 = ((reinterpret_cast<uintptr_t>(buf) | leaf_bytes) & 7) == 0 && leaf_bytes > 0;
     // One thread per leaf and as many blocks as that takes: a leaf is a long
     // chain of permutations, and the block scheduler's dynamic placement

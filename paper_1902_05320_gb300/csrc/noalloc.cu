@@ -133,7 +133,7 @@ extern "C" int keccak_batch_noalloc(const uint8_t *msgs, const uint64_t *offsets
     // queue_issue itself.
     if (cudaMemsetAsync(status, 0, sizeof(unsigned int), st) != cudaSuccess) return KB_ERR_CUDA;
     if (ragged_small(n, s.sms))
-        return ragged_small_issue(msgs, offsets, lens, variant, out_lens, digests, n, status, st);
+        return ragged_small_issue(msgs, offsets, lens, variant, out_lens, digests, n, status, s.sms, st);
     const uint64_t grid = queue_grid_for(cfg, n, s.device, s.sms);
     return queue_issue(msgs, offsets, lens, variant, out_lens, digests, n, queue_scratch, cfg, grid, s.sms, status,
                        st);

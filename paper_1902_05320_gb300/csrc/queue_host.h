@@ -68,7 +68,7 @@ bool ragged_small(uint64_t n, int sm_count);
 // Enqueues that launch: no scratch, no allocation, no synchronisation.
 int ragged_small_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens, const uint8_t *variants,
                        const uint32_t *out_lens, uint8_t *digests, uint64_t n, unsigned int *status,
-                       cudaStream_t stream);
+                       int sm_count, cudaStream_t stream);
 
 // keccak_batch's queue path: configuration from knobs, tuned entries and the
 // cache file; graph capture and replay.

@@ -100,6 +100,10 @@ __device__ __forceinline__ void launch_wait() { asm volatile("griddepcontrol.wai
 int64_t tuning_get(int key);
 int tuning_set(int key, int64_t value);
 
+// Whether a launch of `blocks` one-warp blocks is small enough (four to an SM) for the
+// next kernel of the stream to be set up as soon as these have started (coop_sponge).
+inline bool few_warps(uint64_t blocks, int sm_count) { return blocks <= 4 * uint64_t(sm_count > 0 ? sm_count : 1); }
+
 // Launchers (one per translation unit of kernels).
 int launch_uniform(const uint8_t *msgs, uint64_t stride, uint64_t len, int variant, uint32_t out_len,
                    uint8_t *digests, uint64_t n, cudaStream_t stream, const DeviceInfo &dev);

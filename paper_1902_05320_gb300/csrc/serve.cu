@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
 // long request's latency is its chain of permutations: 1.55 us each here, 2.36
 // with a lane of the state per thread, the form before.  The launch asks for
 // kLongSmem bytes of shared memory that it does not use, so that an SM holds at
-// most nine of these warps: batches start while others' blocks occupy most SMs,
+// most eight of these warps (25.5 KiB each with the system's share, of 228): batches start while others' blocks occupy most SMs,
 // and without a limit the scheduler put up to 32 long chains on the few SMs with
 // room, where they share the path to shared memory (2000 requests of up to 1 MiB
 // at once: 26 to 51 ms from run to run without the limit, 25 to 27 with it, 40 to

@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(32)
 __global__ void __launch_bounds__(32)
     k_sha3_ragged_coop(const uint8_t *msgs, const uint64_t *offsets,
                        const uint64_t *lens, const uint8_t *variants,
-                       const uint32_t *out_lens, uint8_t *digests, unsigned int *status) {
+                       const uint32_t *out_lens, uint8_t *digests, unsigned int *status, bool few) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     const uint32_t i = blockIdx.x, lane = threadIdx.x;
     const Coop c(mem);
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(32)
         if (lane == 0) atomicOr(status, v > 5 ? KB_DEV_BAD_VARIANT : KB_DEV_BAD_OUTLEN);
         return;
     }
-    coop_sponge<-1, true>(c, p, len, v, digests + before, dlen);
+    coop_sponge<-1, true>(c, p, len, v, digests + before, dlen, few);
 }
 
 namespace {
@@ -294,9 +294,9 @@ bool ragged_small(uint64_t n, int sm_count) {
 
 int ragged_small_issue(const uint8_t *msgs, const uint64_t *offsets, const uint64_t *lens, const uint8_t *variants,
                        const uint32_t *out_lens, uint8_t *digests, uint64_t n, unsigned int *status,
-                       cudaStream_t stream) {
+                       int sm_count, cudaStream_t stream) {
     return cuda_status(launch_overlapped(k_sha3_ragged_coop, unsigned(n), 32, 0, stream, msgs, offsets, lens, variants,
-                                         out_lens, digests, status));
+                                         out_lens, digests, status, few_warps(n, sm_count)));
 }
 
 uint64_t queue_grid_for(const QueueConfig &cfg, uint64_t n, int device, int sm_count) {
@@ -576,7 +576,8 @@ int launch_ragged_queue(const uint8_t *msgs, const uint64_t *offsets, const uint
         !have_tuned(n, dev))
         return autotune_ragged_queue(msgs, offsets, lens, variants, out_lens, digests, n, stream, dev, nullptr);
     if (ragged_small(n, dev.sm_count))
-        return ragged_small_issue(msgs, offsets, lens, variants, out_lens, digests, n, dev.d_status, stream);
+        return ragged_small_issue(msgs, offsets, lens, variants, out_lens, digests, n, dev.d_status, dev.sm_count,
+                                  stream);
     const size_t bytes = queue_scratch_bytes(n);
     uint8_t *scratch = static_cast<uint8_t *>(stream_scratch(stream, bytes, &err));
     if (!scratch) return err;

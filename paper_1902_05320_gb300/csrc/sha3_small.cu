@@ -16,12 +16,12 @@ namespace {
 // memory.)
 __global__ void __launch_bounds__(32)
     k_sha3_uniform_coop(const uint8_t *msgs, uint64_t stride, uint64_t len, int variant,
-                        uint8_t *out, uint32_t out_len) {
+                        uint8_t *out, uint32_t out_len, bool few) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     const Coop c(mem);
     const uint64_t m = blockIdx.x;
     launch_wait();
-    coop_sponge<-1, true>(c, msgs + m * stride, len, variant, out + m * out_len, out_len);
+    coop_sponge<-1, true>(c, msgs + m * stride, len, variant, out + m * out_len, out_len, few);
 }
 
 template <int V>
@@ -120,7 +120,7 @@ bool launch_uniform_small(const uint8_t *msgs, uint64_t stride, uint64_t len, in
     const bool one = len < rate && out_len <= rate;
     if (n <= (one ? kCoopOnePerSm : kCoopPerSm) * sms) {
         *rc = cuda_status(launch_overlapped(k_sha3_uniform_coop, unsigned(n), 32, 0, stream, msgs, stride, len, variant,
-                                            digests, out_len));
+                                            digests, out_len, few_warps(n, dev.sm_count)));
         return true;
     }
     // One-block messages: a thread each folds round 0 and most of the last, so two

@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kThreads, kStagedMinBlocks)
 
 template <int V, int LEN, bool A8, class Rep>
 int launch_one(const uint8_t *msgs, uint64_t stride, uint64_t len, uint32_t out_len, uint8_t *digests,
-               uint64_t n, cudaStream_t stream, const DeviceInfo &dev) {
+               uint64_t n, cudaStream_t stream) {
     // A message per thread and as many blocks as that takes, so that the block
     // scheduler balances the sub-partitions' shares (k_sha3_uniform64_tma).  One-block
     // messages with (occupancy x SMs) blocks striding over them, against this: 2^22 of
@@ -201,21 +201,21 @@ int launch_variant(const uint8_t *msgs, uint64_t stride, uint64_t len, uint32_t 
         // The bit-interleaved control, selected through the tuning interface.
         if (tuning_get(KB_TUNE_REPRESENTATION) == KB_REP_INTERLEAVED) {
             if (len == 64 && a16)
-                return launch_one<V, 64, true, InterleavedRep>(msgs, stride, len, out_len, digests, n, stream, dev);
-            if (a8) return launch_one<V, -1, true, InterleavedRep>(msgs, stride, len, out_len, digests, n, stream, dev);
+                return launch_one<V, 64, true, InterleavedRep>(msgs, stride, len, out_len, digests, n, stream);
+            if (a8) return launch_one<V, -1, true, InterleavedRep>(msgs, stride, len, out_len, digests, n, stream);
         }
     }
     if (len == 64 && stride == 64 && a16 && tuning_get(KB_TUNE_STAGING) == KB_STAGING_TMA &&
         device_resident(msgs, dev.device))
         return launch_tma<V>(msgs, out_len, digests, n, stream, dev);
-    if (len == 64 && a16) return launch_one<V, 64, true, PlainRep>(msgs, stride, len, out_len, digests, n, stream, dev);
+    if (len == 64 && a16) return launch_one<V, 64, true, PlainRep>(msgs, stride, len, out_len, digests, n, stream);
     constexpr int rate = Variant<V>::rate;
     if (len < uint64_t(rate) && (Variant<V>::digest || out_len <= uint32_t(rate))) {
-        if (a8) return launch_one<V, -2, true, PlainRep>(msgs, stride, len, out_len, digests, n, stream, dev);
-        return launch_one<V, -2, false, PlainRep>(msgs, stride, len, out_len, digests, n, stream, dev);
+        if (a8) return launch_one<V, -2, true, PlainRep>(msgs, stride, len, out_len, digests, n, stream);
+        return launch_one<V, -2, false, PlainRep>(msgs, stride, len, out_len, digests, n, stream);
     }
-    if (a8) return launch_one<V, -1, true, PlainRep>(msgs, stride, len, out_len, digests, n, stream, dev);
-    return launch_one<V, -1, false, PlainRep>(msgs, stride, len, out_len, digests, n, stream, dev);
+    if (a8) return launch_one<V, -1, true, PlainRep>(msgs, stride, len, out_len, digests, n, stream);
+    return launch_one<V, -1, false, PlainRep>(msgs, stride, len, out_len, digests, n, stream);
 }
 
 }  // namespace

@@ -267,11 +267,11 @@ template <bool INIT, bool FINAL>
 __global__ void __launch_bounds__(32)
     k_stream_step_coop(uint8_t *states, const uint8_t *init_variants, const uint8_t *msgs,
                        const uint64_t *offsets, const uint64_t *lens,
-                       const uint32_t *out_lens, uint8_t *digests, unsigned int *status) {
+                       const uint32_t *out_lens, uint8_t *digests, unsigned int *status, bool few) {
     __shared__ __align__(16) uint32_t mem[Coop::kWarpWords];
     const Coop c(mem);
     const uint32_t i = blockIdx.x, lane = threadIdx.x;
-    if (gridDim.x <= kFewBlocks) launch_next();
+    if (few) launch_next();
     launch_wait();
     uint8_t *st = states + uint64_t(i) * kStateBytes;
     uint32_t *pending_field = reinterpret_cast<uint32_t *>(st + kNbufOff);
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(32)
     }
     a[0] ^= e[0];  // the open block: the tail, and the padding of a final step
     a[1] ^= e[1];
-    if (gridDim.x > kFewBlocks) launch_next();
+    if (!few) launch_next();
     if constexpr (FINAL) {
         uint8_t *dst = digests + before;
         const uint32_t nsq = dlen > rate ? (dlen - 1) / rate : 0;
@@ -424,7 +424,7 @@ int launch_stream_step(bool init, bool final_, uint8_t *states, const uint8_t *v
                                              : final_ ? k_stream_step_coop<false, true>
                                                       : k_stream_step_coop<false, false>,
                                              unsigned(n), 32, 0, stream, states, variants, msgs, offsets, lens,
-                                             out_lens, digests, dev.d_status));
+                                             out_lens, digests, dev.d_status, few_warps(n, dev.sm_count)));
     uint64_t *out_off = nullptr;
     uint64_t *zeros = nullptr;
     if (final_) {
