@@ -56,12 +56,14 @@ __device__ __forceinline__ void ld_word_any(const uint8_t *p, uint32_t nvalid, u
 template <int RATE, bool A8, class Rep>
 __device__ __forceinline__ void absorb_full(uint32_t (&A)[25], uint32_t (&B)[25], const uint8_t *p) {
     if constexpr (A8) {
+        // All words before the first XOR: with plain loads the compiler keeps to the
+        // source's order (2^22 messages of 1 KiB 6666 us, 6702 word by word; 60,000
+        // 133.4 and 138.0).
+        uint2 w[RATE / 8];
 #pragma unroll
-        for (int k = 0; k < RATE / 8; ++k) {
-            uint32_t lo, hi;
-            ld_word_a8(p + 8 * k, lo, hi);
-            Rep::xor_word(A[k], B[k], lo, hi);
-        }
+        for (int k = 0; k < RATE / 8; ++k) w[k] = reinterpret_cast<const uint2 *>(p)[k];
+#pragma unroll
+        for (int k = 0; k < RATE / 8; ++k) Rep::xor_word(A[k], B[k], w[k].x, w[k].y);
     } else {
         // RATE/4 aligned words cover the block; one more when p is unaligned.
         const uintptr_t start = reinterpret_cast<uintptr_t>(p);
