@@ -111,8 +111,8 @@ struct Control {
 // The hand-off from k_scatter to a k_sha3_queue that starts beside k_sha3_lanes.
 // griddepcontrol.wait covers the kernel before (k_sha3_lanes), whose end the queue
 // kernel must not wait for; that kernel's own wait makes k_scatter's writes visible
-// to itself alone.  So a thread of k_sha3_lanes that has waited releases a flag and
-// every thread of the queue kernel acquires it.
+// to itself alone.  So a thread of k_sha3_lanes that has waited releases a flag, and
+// a warp of every block of the queue kernel acquires it for the block.
 __device__ __forceinline__ void hand_over(uint32_t *flag) {
     asm volatile("st.release.gpu.b32 [%0], %1;" ::"l"(flag), "r"(1u) : "memory");
 }
@@ -429,7 +429,14 @@ __global__ void __launch_bounds__(kThreads, MINB)
     constexpr bool kLoop = (STAGE & kLooped) != 0;
     __shared__ uint32_t stage_mem[kRead == kStageAsync ? 2 * kStageWords * kThreads : 1];
     const int lane = threadIdx.x & 31;
-    if (beside && !taken_over(&ctl->ready)) launch_wait();
+    // One warp a block asks, so that the block's warps go on together: with each for
+    // itself some were late for the look at the slots below and took the longest
+    // chains into slots that issue second (2^20 messages at 3 blocks per SM 11.1 to
+    // 14.0 ms from call to call, now 11.1).
+    if (beside) {
+        if (threadIdx.x < 32 && !taken_over(&ctl->ready)) launch_wait();
+        __syncthreads();
+    }
     const uint64_t start = ctl->queue_start;
     const unsigned long long ngroups = n > start ? (n - start + 31) / 32 : 0;
     const unsigned long long nfront = min((unsigned long long)(ctl->queue_mid - start) / 32, ngroups);

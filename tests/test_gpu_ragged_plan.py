@@ -95,3 +95,24 @@ def test_split_gives_few_long_chains_a_warp_each(cuda_lib, restore_split, kind):
         np.where(np.arange(n) % (n // 100) == 0, 65536, 500)
     batch = Batch(cuda_lib, lens)
     assert batch.ms() < 0.67 * batch.ms(0)
+
+
+@pytest.mark.parametrize("blocks", [2, 3])
+def test_queue_beside_an_idle_warp_kernel_keeps_its_time(cuda_lib, restore_split, blocks):
+    """Where the plan moves nothing, the queue takes what it takes alone, call after call: its warps are sorted into
+    those that issue first and the others however the launch before them ends."""
+    import torch
+
+    rng = np.random.default_rng(3)
+    n = 2000 * torch.cuda.get_device_properties(0).multi_processor_count
+    batch = Batch(cuda_lib, np.exp(rng.uniform(0, np.log(16384), size=n)).astype(np.int64))
+    keys = (cuda_lib.KB_TUNE_QUEUE_MIN_BLOCKS, cuda_lib.KB_TUNE_QUEUE_BLOCKS_PER_SM, cuda_lib.KB_TUNE_QUEUE_STAGING)
+    saved = [cuda_lib.keccak_tune_get(k) for k in keys]
+    for k, v in zip(keys, (blocks, blocks, 1)):
+        cuda_lib.keccak_tune_set(k, v)
+    try:
+        alone = batch.ms(0)
+        assert max(batch.ms() for _ in range(5)) < 1.06 * alone
+    finally:
+        for k, v in zip(keys, saved):
+            cuda_lib.keccak_tune_set(k, v)

@@ -58,7 +58,9 @@ def test_queue_kernel_takes_the_plan_over_before_it_reads_it():
     assert lanes.index("launch_wait()") < lanes.index("hand_over(&ctl->ready)") < lanes.index("launch_next()")
     assert lanes.index("hand_over(&ctl->ready)") < lanes.index("return")  # on the early exit as well
     take = queue.index("taken_over(&ctl->ready)")
-    assert "if (beside && !taken_over(&ctl->ready)) launch_wait();" in queue, "no wait without the flag"
+    handed = queue[queue.index("if (beside)"):queue.index("__syncthreads();") + 16]
+    assert "if (threadIdx.x < 32 && !taken_over(&ctl->ready)) launch_wait();" in handed, "no wait without the flag"
+    take = queue.index("__syncthreads();")  # the other warps of the block go on behind it
     for read in ("ctl->queue_start", "ctl->queue_mid", "ctl->slots", "ctl->ends", "order[", "out_off"):
         assert take < queue.index(read), read
     assert "__restrict__" not in found["k_sha3_queue"][0], "read-only loads may be moved before the acquire"
